@@ -93,7 +93,9 @@ def _model_specs(case, seed):
     model = case["model"]
     kw = {k: case[k] for k in ("n_grid", "width", "n_species") if k in case}
     if model == "toys":
-        return I.toy_batch(case["toys"], n_grid=case.get("n_grid", 2000), seed=seed)
+        grid = case.get("n_grid", 2000)   # the last toy has all 15 species: theta is 22 wide
+        return (I.toy_batch(case["toys"] - 1, n_grid=grid, seed=seed)
+                + I.toy_batch(1, n_grid=grid, species=(15, 15), seed=seed + 1))
     lo = 150.0 if model == "plain" else 100.0
     if "bins" in case:
         kw["lo_npe"] = math.floor(lo / kw["width"]) * kw["width"]
