@@ -1347,36 +1347,34 @@ __global__ void __launch_bounds__(T2 + 32, 1) k_bwd2d(Work w) {
 
 // ------------------------------------------------------------------ gather
 
-__global__ void k_gather2d(Work w, int n, double* nll_out, double* grad_out, int want_grad) {
-    const int item = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp per item, lane j = parameter j (as k_gather; the window tiles' sums of -lnL and of the
+// eps gradient keep their order).
+__global__ void __launch_bounds__(128) k_gather2d(Work w, int n, double* nll_out, double* grad_out, int want_grad) {
+    const int item = blockIdx.x * 4 + (threadIdx.x >> 5), j = threadIdx.x & 31;
     if (item >= n) return;
     const Toy& T = w.toys[w.toy_of[item]];
     const int st = w.status[item];
     const int nt = (T.nw + TM - 1) / TM;
-    double s = 0.0, c = 0.0, ge = 0.0;
-    for (int t = 0; t < nt; ++t) {
-        s += w.nll2d[((size_t)item * MAX_TILES + t) * 2];
-        c += w.nll2d[((size_t)item * MAX_TILES + t) * 2 + 1];
-        ge += w.geps2d[(size_t)item * MAX_TILES + t];
-    }
-    nll_out[item] = st ? INFINITY : s + c;
-    if (!want_grad) return;
-    double* go = grad_out + (size_t)item * w.pstride;
-    const double* gp = w.gpart2d + (size_t)item * MAX_CB * (GPN + 1);
-    for (int j = 0; j < w.pstride; ++j) {
-        double g = 0.0;
-        if (!st && j < T.P) {
-            int slot = -1;
-            if (j < T.K) slot = 5 + j;
-            else if (j < T.K + 5) slot = j - T.K;
-            else if (j == T.K + 6) slot = GPN;
-            if (slot >= 0)
-                for (int q = 0; q < T.n_cb; ++q) g += gp[q * (GPN + 1) + slot];
-            else
-                g = ge;   // eps
+    if (j == 0) {
+        double s = 0.0, c = 0.0;
+#pragma unroll 4
+        for (int t = 0; t < nt; ++t) {
+            s += w.nll2d[((size_t)item * MAX_TILES + t) * 2];
+            c += w.nll2d[((size_t)item * MAX_TILES + t) * 2 + 1];
         }
-        go[j] = g;
+        nll_out[item] = st ? INFINITY : s + c;
     }
+    if (!want_grad || j >= w.pstride) return;
+    double g = 0.0;
+    if (!st && j < T.P) {
+        const int slot = j < T.K ? 5 + j : j < T.K + 5 ? j - T.K : j == T.K + 6 ? GPN : -1;
+        // the column blocks' partials, or (eps) the window tiles'
+        const double* gp = slot >= 0 ? w.gpart2d + (size_t)item * MAX_CB * (GPN + 1) + slot : w.geps2d + (size_t)item * MAX_TILES;
+        const int np = slot >= 0 ? T.n_cb : nt, step = slot >= 0 ? GPN + 1 : 1;
+#pragma unroll 8
+        for (int q = 0; q < np; ++q) g += gp[(size_t)q * step];
+    }
+    grad_out[(size_t)item * w.pstride + j] = g;
 }
 
 // ------------------------------------------------------------------ launchers
@@ -1423,7 +1421,7 @@ cudaError_t launch_eval2d(const Work& w, int n, int want_grad, int want_mu, int 
 }
 
 cudaError_t launch_gather2d(const Work& w, int n, double* nll_out, double* grad_out, int want_grad, cudaStream_t s) {
-    k_gather2d<<<(n + 127) / 128, 128, 0, s>>>(w, n, nll_out, grad_out, want_grad);
+    k_gather2d<<<(n + 3) / 4, 128, 0, s>>>(w, n, nll_out, grad_out, want_grad);
     return cudaGetLastError();
 }
 

@@ -456,33 +456,35 @@ cudaError_t launch_bwd(const Work& w, int n, int max_cb, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Final -lnL and gradient of each item (rows of stride pstride; unused slots zeroed).
-__global__ void k_gather(Work w, int n, double* nll_out, double* grad_out, int want_grad) {
-    const int item = blockIdx.x * blockDim.x + threadIdx.x;
+// Final -lnL and gradient of each item (rows of stride pstride; unused slots zeroed).  A warp
+// per item, lane j = parameter j: the partials of one column block are one contiguous row, and a
+// lane's loads do not depend on each other, so the kernel costs about one memory latency (a
+// thread per item walked its P x n_cb partials alone: 29 us for one 22-parameter evaluation,
+// 35 us for 52).  The sum over column blocks keeps its order.
+static_assert(PMAX <= 32, "one lane per parameter");
+__global__ void __launch_bounds__(128) k_gather(Work w, int n, double* nll_out, double* grad_out, int want_grad) {
+    const int item = blockIdx.x * 4 + (threadIdx.x >> 5), j = threadIdx.x & 31;
     if (item >= n) return;
     const Toy& T = w.toys[w.toy_of[item]];
     const int st = w.status[item];
-    nll_out[item] = st ? INFINITY : w.nll[item];
-    if (!want_grad) return;
-    const double* gm = w.gmid + (size_t)item * PMAX;
-    const double* gp = w.gpart + (size_t)item * MAX_CB * GPN;
-    double* go = grad_out + (size_t)item * w.pstride;
-    for (int j = 0; j < w.pstride; ++j) {
-        double g = 0.0;
-        if (!st && j < T.P) {
-            g = gm[j];
-            int slot = -1;
-            if (j < T.K) slot = 5 + j;
-            else if (j < T.K + 5) slot = j - T.K;
-            if (slot >= 0)
-                for (int cb = 0; cb < T.n_cb; ++cb) g += gp[cb * GPN + slot];
+    if (j == 0) nll_out[item] = st ? INFINITY : w.nll[item];
+    if (!want_grad || j >= w.pstride) return;
+    double g = 0.0;
+    if (!st && j < T.P) {
+        g = w.gmid[(size_t)item * PMAX + j];
+        const int slot = j < T.K ? 5 + j : j < T.K + 5 ? j - T.K : -1;
+        if (slot >= 0) {
+            const double* gp = w.gpart + (size_t)item * MAX_CB * GPN + slot;
+            const int ncb = T.n_cb;
+#pragma unroll 8
+            for (int cb = 0; cb < ncb; ++cb) g += gp[cb * GPN];
         }
-        go[j] = g;
     }
+    grad_out[(size_t)item * w.pstride + j] = g;
 }
 
 cudaError_t launch_gather(const Work& w, int n, double* nll_out, double* grad_out, int want_grad, cudaStream_t s) {
-    k_gather<<<(n + 127) / 128, 128, 0, s>>>(w, n, nll_out, grad_out, want_grad);
+    k_gather<<<(n + 3) / 4, 128, 0, s>>>(w, n, nll_out, grad_out, want_grad);
     return cudaGetLastError();
 }
 

@@ -38,24 +38,32 @@ __global__ void k_est_split(const double* theta, int tstride, int n, int E, cons
     if (skip_int) skip_int[j] = skip ? skip[pub] : 0;
 }
 
-// Joint -lnL (the sum over the estimators) and gradient of every public item.
-__global__ void k_est_join(const double* nll_int, const double* grad_int, int Pi, int n, int E, const Toy* toys,
-                           const int* toy_of, double* nll, double* grad, int P, int want_grad) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;   // public item
+// Joint -lnL (the sum over the estimators) and gradient of every public item: a warp per item, its
+// lanes the joint parameters (a thread per item walked its P x E values alone).
+__global__ void __launch_bounds__(128) k_est_join(const double* nll_int, const double* grad_int, int Pi, int n, int E,
+                                                  const Toy* toys, const int* toy_of, double* nll, double* grad, int P,
+                                                  int want_grad) {
+    const int j = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;   // public item
     if (j >= n) return;
     const int K = toys[toy_of[(size_t)j * E]].K;
-    double f = 0.0;
-    for (int e = 0; e < E; ++e) f += nll_int[(size_t)j * E + e];
-    nll[j] = f;
+    if (lane == 0) {
+        double f = 0.0;
+        for (int e = 0; e < E; ++e) f += nll_int[(size_t)j * E + e];
+        nll[j] = f;
+    }
     if (!want_grad) return;
-    double* g = grad + (size_t)j * P;
-    for (int q = 0; q < P; ++q) g[q] = 0.0;
-    for (int e = 0; e < E; ++e) {
-        const double* ge = grad_int + ((size_t)j * E + e) * Pi;
-        const int so = e == 0 ? K : K + 7 + 4 * (e - 1);
-        for (int k = 0; k < K; ++k) g[k] += ge[k];
-        for (int q = 0; q < 4; ++q) g[so + q] += ge[K + q];
-        for (int q = 4; q < 7; ++q) g[K + q] += ge[K + q];
+    const double* ge = grad_int + (size_t)j * E * Pi;
+    for (int q = lane; q < P; q += 32) {
+        double g = 0.0;
+        if (q < K || (q >= K + 4 && q < K + 7)) {          // rates, kB, eps, s_r: shared
+            for (int e = 0; e < E; ++e) g += ge[(size_t)e * Pi + q];
+        } else if (q < K + 4) {                            // LY, a, b, c of estimator 0
+            g += ge[q];
+        } else if (q < K + 7 + 4 * (E - 1)) {              // and of a further one
+            const int e = (q - K - 7) / 4 + 1;
+            g += ge[(size_t)e * Pi + K + (q - K - 7) % 4];
+        }
+        grad[(size_t)j * P + q] = g;
     }
 }
 
@@ -68,7 +76,7 @@ cudaError_t launch_est_split(const double* theta, int tstride, int n, int E, con
 
 cudaError_t launch_est_join(const double* nll_int, const double* grad_int, int Pi, int n, int E, const Toy* toys,
                             const int* toy_of, double* nll, double* grad, int P, int want_grad, cudaStream_t s) {
-    k_est_join<<<(n + 127) / 128, 128, 0, s>>>(nll_int, grad_int, Pi, n, E, toys, toy_of, nll, grad, P, want_grad);
+    k_est_join<<<(n + 3) / 4, 128, 0, s>>>(nll_int, grad_int, Pi, n, E, toys, toy_of, nll, grad, P, want_grad);
     return cudaGetLastError();
 }
 
