@@ -3,7 +3,7 @@
 //
 // Every fit owns a block of S = NLS + 2P evaluation slots in the batch and a state on the
 // device.  One iteration = one batched -lnL + gradient evaluation of every slot in use
-// (the regular evaluation kernels; unused slots are skipped) followed by k_fit, one thread
+// (the regular evaluation kernels; unused slots are skipped) followed by k_fit, one warp
 // per fit, which advances a damped Newton state machine:
 //   START  slot 0 holds the starting point: accept it, go to HESS;
 //   HESS   slots NLS + 2a, NLS + 2a + 1 hold theta +- h e_j for the a-th free parameter j:
@@ -116,7 +116,7 @@ struct FitDev {
     int* Pf;                // per fit: parameters of its dataset's row (K_t + 7 + 4 (E - 1))
     int* Kf;                // per fit: rates (K_t), the parameters before the trust-region ones
     double *theta, *g, *f;  // accepted state per fit
-    double *H, *V, *d;      // per fit
+    double *H, *V;          // per fit
     double *lo, *hi;        // per fit
     unsigned char* fr;      // per fit
     double *tt, *ft, *gt;   // per slot: evaluation input and outputs
@@ -152,108 +152,174 @@ struct FitRun {
 
 #define IDX(i, j) ((i) * P + (j))
 
-// V <- (H + damping)^-1 on the active set of the first n parameters (row stride P):
-// Cholesky of C = D H D + mu I (D = |diag H|^-1/2) for the smallest mu in
-// {mu_min, 10 mu_min, ...} (mu_min = 0 tries the undamped matrix first, then 1e-6).
-// Returns the mu used, or -1 when even mu = 1e8 fails.
-__device__ double damped_inverse(const double* H, const unsigned char* act, int n, int P, double mu_min, double* V,
-                                 double* L) {
-    int idx[PFMAX], nf = 0;
-    double D[PFMAX];
-    for (int i = 0; i < n; ++i)
-        if (act[i]) {
-            const double h = fabs(H[IDX(i, i)]);
-            D[nf] = (h > 0.0 && isfinite(h)) ? 1.0 / sqrt(h) : 1.0;
-            idx[nf++] = i;
-        }
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) V[IDX(i, j)] = 0.0;
+// The warp's working set of one fit in shared memory (k_fit: a warp per fit).  Rows are LSF
+// doubles apart: odd, so that lanes reading one column of a matrix hit different banks.
+constexpr int LSF = PFMAX | 1;
+static_assert(PFMAX % 2 == 1 && PFMAX <= 64, "odd row stride; two lanes' worth of parameters at most");
+struct FitShared {
+    double H[PFMAX * LSF], V[PFMAX * LSF], L[PFMAX * LSF], col[PFMAX * LSF];
+    double D[PFMAX], th[PFMAX], g[PFMAX], d[PFMAX], lim[PFMAX], res[PFMAX];
+    int idx[PFMAX], fidx[PFMAX];
+    unsigned char act[PFMAX], fr[PFMAX];
+};
+#define SIDX(i, j) ((i) * LSF + (j))
+
+// Indices i < n with flag[i] set, in order, into idx; returns their number (every lane).
+__device__ int warp_compact(const unsigned char* flag, int n, int* idx) {
+    const int lane = threadIdx.x & 31;
+    int nf = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const bool on = i0 + lane < n && flag[i0 + lane];
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (on) idx[nf + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
+        nf += __popc(m);
+    }
+    __syncwarp();
+    return nf;
+}
+
+// S.V <- (H + damping)^-1 on the active set of the first n parameters: Cholesky of
+// C = D H D + mu I (D = |diag H|^-1/2) for the smallest mu in {mu_min, 10 mu_min, ...}
+// (mu_min = 0 tries the undamped matrix first, then 1e-6).  Returns the mu used, or -1 when even
+// mu = 1e8 fails.  By the whole warp: a lane per row of the factor's current column, then a lane
+// per column of the inverse.  Every entry keeps the operation order of the plain serial loops, so
+// a fit's path does not depend on the number of lanes.  One thread took ~0.7 ms here for 22 free
+// parameters (its matrices in local memory, every operation waiting for the last one).
+__device__ double damped_inverse(FitShared& S, int n, double mu_min) {
+    const int lane = threadIdx.x & 31;
+    const int nf = warp_compact(S.act, n, S.idx);
+    for (int a = lane; a < nf; a += 32) {
+        const double h = fabs(S.H[SIDX(S.idx[a], S.idx[a])]);
+        S.D[a] = (h > 0.0 && isfinite(h)) ? 1.0 / sqrt(h) : 1.0;
+    }
+    for (int j = lane; j < n * n; j += 32) S.V[SIDX(j / n, j % n)] = 0.0;
+    __syncwarp();
     double mu = mu_min;
     for (int attempt = 0; attempt < 40; ++attempt, mu = (mu == 0.0 ? 1e-6 : mu * 10.0)) {
         if (mu > 1e8) return -1.0;
         bool ok = true;
-        for (int a = 0; a < nf && ok; ++a)
-            for (int b = 0; b <= a; ++b) {
-                const int ia = idx[a], ib = idx[b];
-                double c = 0.5 * (H[IDX(ia, ib)] + H[IDX(ib, ia)]) * D[a] * D[b] + (a == b ? mu : 0.0);
-                for (int k = 0; k < b; ++k) c -= L[a * nf + k] * L[b * nf + k];
-                if (a == b) {
-                    if (!(c > 0.0) || !isfinite(c)) { ok = false; break; }
-                    L[a * nf + a] = sqrt(c);
-                } else {
-                    L[a * nf + b] = c / L[b * nf + b];
-                }
+        for (int b = 0; b < nf && ok; ++b) {   // column b of L: rows a >= b
+            const int ib = S.idx[b];
+            double ca[2], dg = 0.0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int a = b + lane + 32 * q;
+                ca[q] = 0.0;
+                if (a >= nf) continue;
+                const int ia = S.idx[a];
+                double c = 0.5 * (S.H[SIDX(ia, ib)] + S.H[SIDX(ib, ia)]) * S.D[a] * S.D[b] + (a == b ? mu : 0.0);
+                for (int k = 0; k < b; ++k) c -= S.L[SIDX(a, k)] * S.L[SIDX(b, k)];
+                ca[q] = c;
             }
-        if (!ok) continue;
-        double col[PFMAX];
-        for (int c = 0; c < nf; ++c) {
+            dg = __shfl_sync(0xffffffffu, ca[0], 0);   // the diagonal entry: lane 0
+            if (!(dg > 0.0) || !isfinite(dg)) {
+                ok = false;
+                break;
+            }
+            const double r = sqrt(dg);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int a = b + lane + 32 * q;
+                if (a < nf) S.L[SIDX(a, b)] = a == b ? r : ca[q] / r;
+            }
+            __syncwarp();
+        }
+        if (!ok) {
+            __syncwarp();
+            continue;
+        }
+        for (int c = lane; c < nf; c += 32) {   // column c of the inverse
+            double* col = S.col + c;            // stride LSF
             for (int i = 0; i < nf; ++i) {
                 double t = (i == c) ? 1.0 : 0.0;
-                for (int k = 0; k < i; ++k) t -= L[i * nf + k] * col[k];
-                col[i] = t / L[i * nf + i];
+                for (int k = 0; k < i; ++k) t -= S.L[SIDX(i, k)] * col[k * LSF];
+                col[i * LSF] = t / S.L[SIDX(i, i)];
             }
             for (int i = nf - 1; i >= 0; --i) {
-                double t = col[i];
-                for (int k = i + 1; k < nf; ++k) t -= L[k * nf + i] * col[k];
-                col[i] = t / L[i * nf + i];
+                double t = col[i * LSF];
+                for (int k = i + 1; k < nf; ++k) t -= S.L[SIDX(k, i)] * col[k * LSF];
+                col[i * LSF] = t / S.L[SIDX(i, i)];
             }
-            for (int i = 0; i < nf; ++i) V[IDX(idx[i], idx[c])] = D[i] * col[i] * D[c];
+            for (int i = 0; i < nf; ++i) S.V[SIDX(S.idx[i], S.idx[c])] = S.D[i] * col[i * LSF] * S.D[c];
         }
+        __syncwarp();
         return mu;
     }
     return -1.0;
 }
 
 // Put queued fit qf into slot block jf: its start in slot 0 (to be evaluated next round), its
-// bounds, free flags and state, its dataset on the slot's evaluation items.
+// bounds, free flags and state, its dataset on the slot's evaluation items.  By a whole warp.
 __device__ void slot_load(const FitDev& F, int jf, int qf) {
-    const int P = F.P, S = F.S;
+    const int P = F.P, S = F.S, lane = threadIdx.x & 31;
     const size_t s0 = (size_t)jf * S;
-    F.slot_fit[jf] = qf;
-    for (int i = 0; i < P; ++i) {
+    for (int i = lane; i < P; i += 32) {
         F.tt[s0 * P + i] = F.q_theta0[(size_t)qf * P + i];
         F.lo[(size_t)jf * P + i] = F.q_lo[(size_t)qf * P + i];
         F.hi[(size_t)jf * P + i] = F.q_hi[(size_t)qf * P + i];
         F.fr[(size_t)jf * P + i] = F.q_fr[(size_t)qf * P + i];
     }
-    for (int i = 0; i < P * P; ++i) F.H[(size_t)jf * P * P + i] = 0.0;
-    F.Pf[jf] = F.q_Pf[qf];
-    F.Kf[jf] = F.q_Kf[qf];
-    F.ctl[jf] = F.q_ctl0[qf];
+    for (int i = lane; i < P * P; i += 32) F.H[(size_t)jf * P * P + i] = 0.0;
     const int toy = F.q_toy[qf];
-    for (int k = 0; k < S; ++k) {
+    if (lane == 0) {
+        F.slot_fit[jf] = qf;
+        F.Pf[jf] = F.q_Pf[qf];
+        F.Kf[jf] = F.q_Kf[qf];
+        F.ctl[jf] = F.q_ctl0[qf];
+    }
+    for (int k = lane; k < S; k += 32) {
         F.skip[s0 + k] = k == 0 ? 0 : 1;
         for (int e = 0; e < F.E; ++e) F.toy_of[(s0 + k) * F.E + e] = toy * F.E + e;
     }
 }
 
+// The next queued fit (or none) into slot block jf; whether there was one.  By a whole warp.
+__device__ bool slot_refill(const FitDev& F, int jf) {
+    const int lane = threadIdx.x & 31;
+    int qf = 0;
+    if (lane == 0) qf = atomicAdd(F.next_fit, 1);
+    qf = __shfl_sync(0xffffffffu, qf, 0);
+    if (qf < F.run->n_fits) {
+        slot_load(F, jf, qf);
+        return true;
+    }
+    if (lane == 0) F.slot_fit[jf] = -1;
+    for (int k = lane; k < F.S; k += 32) F.skip[(size_t)jf * F.S + k] = 1;
+    return false;
+}
+
 // A finished fit's result leaves its slot block: theta (its start beyond the fit's own P, where
-// the slot may hold a longer fit's values) and, when asked for, the covariance.
+// the slot may hold a longer fit's values) and, when asked for, the covariance.  By a whole warp;
+// V is the slot block's matrix in global memory (a fit may end without a new direction).
 __device__ void slot_store(const FitDev& F, int jf, const FitCtl& c) {
-    const int P = F.P, qf = F.slot_fit[jf], Pt = F.Pf[jf];
-    for (int i = 0; i < P; ++i)
+    const int P = F.P, qf = F.slot_fit[jf], Pt = F.Pf[jf], lane = threadIdx.x & 31;
+    for (int i = lane; i < P; i += 32)
         F.o_theta[(size_t)qf * P + i] = i < Pt ? F.theta[(size_t)jf * P + i] : F.q_theta0[(size_t)qf * P + i];
-    F.o_f[qf] = F.f[jf];
-    F.o_ctl[qf] = c;
+    if (lane == 0) {
+        F.o_f[qf] = F.f[jf];
+        F.o_ctl[qf] = c;
+    }
     double* oV = F.run->o_V;
     if (oV) {
         const double* V = F.V + (size_t)jf * P * P;
-        for (int i = 0; i < P; ++i)
-            for (int j = 0; j < P; ++j) oV[(size_t)qf * P * P + IDX(i, j)] = (i < Pt && j < Pt) ? V[IDX(i, j)] : 0.0;
+        for (int j = lane; j < P * P; j += 32) {
+            const int i = j / P, k = j - i * P;
+            oV[(size_t)qf * P * P + j] = (i < Pt && k < Pt) ? V[j] : 0.0;
+        }
     }
 }
 
-// Fill every slot block from the queue (before the first round).
-__global__ void k_fit_init(FitDev F) {
-    const int jf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (jf >= F.n) return;
-    const int qf = atomicAdd(F.next_fit, 1);
-    if (qf < F.run->n_fits) {
-        slot_load(F, jf, qf);
+// Fill every slot block from the queue (before the first round): a warp per slot block, in order
+// of the blocks (the queue head is taken by block index, not by arrival).
+__global__ void __launch_bounds__(32) k_fit_init(FitDev F) {
+    const int jf = blockIdx.x;
+    if (jf < F.run->n_fits) {
+        slot_load(F, jf, jf);
     } else {
-        F.slot_fit[jf] = -1;
-        for (int k = 0; k < F.S; ++k) F.skip[(size_t)jf * F.S + k] = 1;
+        if (threadIdx.x == 0) F.slot_fit[jf] = -1;
+        for (int k = threadIdx.x; k < F.S; k += 32) F.skip[(size_t)jf * F.S + k] = 1;
     }
+    if (jf == 0 && threadIdx.x == 0) *F.next_fit = F.n;
 }
 
 // For the autotuner: every slot of a block evaluates the block's start point (a full round).
@@ -279,68 +345,144 @@ __global__ void k_fit_ctl(FitDev F) {
     cudaGraphSetConditional(F.handle, more && !late ? 1u : 0u);
 }
 
-__global__ void k_fit(FitDev F) {
-    const int jf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (jf >= F.n || F.slot_fit[jf] < 0) return;
+// One round of every fit in flight: a warp per fit, the parameters over its lanes, the matrices in
+// shared memory.  FP64 and latency bound: a handful of warps, each a chain of dependent FP64
+// operations; every value keeps the operation order of the serial loops.  The state (c) is uniform
+// over the warp.  One thread per fit took about 1 ms a round of a 22-parameter fit, more than the
+// evaluation of its 52 slots.
+__global__ void __launch_bounds__(32) k_fit(FitDev F) {
+    const int jf = blockIdx.x, lane = threadIdx.x;
+    if (F.slot_fit[jf] < 0) return;
     const int P = F.P, S = F.S;
     FitCtl c = F.ctl[jf];
     if (c.phase == PH_DONE) return;
+    __shared__ FitShared sh;
     const size_t s0 = (size_t)jf * S;   // first slot of this fit
     const int Pt = F.Pf[jf], Kt = F.Kf[jf];
-    double* th = F.theta + (size_t)jf * P;
-    double* g = F.g + (size_t)jf * P;
-    double* V = F.V + (size_t)jf * P * P;
-    double* H = F.H + (size_t)jf * P * P;
-    double* d = F.d + (size_t)jf * P;
+    double* gth = F.theta + (size_t)jf * P;
+    double* gg = F.g + (size_t)jf * P;
+    double* gV = F.V + (size_t)jf * P * P;
+    double* gH = F.H + (size_t)jf * P * P;
     const double* lo = F.lo + (size_t)jf * P;
     const double* hi = F.hi + (size_t)jf * P;
-    const unsigned char* fr = F.fr + (size_t)jf * P;
+    double* th = sh.th;
+    double* g = sh.g;
+    double fcur = F.f[jf];
     auto slot_t = [&](int k) { return F.tt + (s0 + k) * P; };
     auto slot_g = [&](int k) { return F.gt + (s0 + k) * P; };
+    for (int i = lane; i < Pt; i += 32) {
+        th[i] = gth[i];
+        g[i] = gg[i];
+        sh.fr[i] = F.fr[(size_t)jf * P + i];
+    }
+    if (c.phase != PH_START)
+        for (int j = lane; j < Pt * Pt; j += 32) sh.H[SIDX(j / Pt, j % Pt)] = gH[IDX(j / Pt, j % Pt)];
+    else
+        for (int j = lane; j < Pt * Pt; j += 32) sh.H[SIDX(j / Pt, j % Pt)] = 0.0;
+    __syncwarp();
+    const int nfree = warp_compact(sh.fr, Pt, sh.fidx);
+    // the accepted state from slot k
+    auto accept = [&](int k) {
+        const double* tk = slot_t(k);
+        const double* gk = slot_g(k);
+        __syncwarp();
+        for (int i = lane; i < Pt; i += 32) {
+            th[i] = gth[i] = tk[i];
+            g[i] = gg[i] = gk[i];
+        }
+        fcur = F.ft[s0 + k];
+        if (lane == 0) F.f[jf] = fcur;
+        __syncwarp();
+    };
     bool to_hess = false, newdir = false, fresh = false;
 
     if (c.phase == PH_START) {
-        const double f0 = F.ft[s0];
-        for (int i = 0; i < Pt; ++i) { th[i] = slot_t(0)[i]; g[i] = slot_g(0)[i]; }
-        F.f[jf] = f0;
-        if (!isfinite(f0)) { c.phase = PH_DONE; c.status = BX_EDOMAIN; }
+        accept(0);
+        if (!isfinite(fcur)) { c.phase = PH_DONE; c.status = BX_EDOMAIN; }
         else to_hess = true;
     } else if (c.phase == PH_HESS) {
         // column j: the central difference of the gradients at theta +- h e_j; where one side was
         // not evaluable (outside the model's domain, or h below the resolution of theta_j) the
         // one-sided difference with the accepted point; with neither, no curvature (damping
-        // then carries that direction)
-        auto finite_at = [&](int k) {
-            if (!isfinite(F.ft[s0 + k])) return false;
-            const double* gk = slot_g(k);
-            for (int i = 0; i < Pt; ++i)
-                if (!isfinite(gk[i])) return false;
-            return true;
-        };
-        int a = 0, ne = 0;
-        double res[PFMAX];
-        for (int j = 0; j < Pt; ++j) {
-            if (!fr[j]) continue;
-            const int kp = NLS + 2 * a, km = kp + 1;
-            const double up = slot_t(kp)[j], dn = slot_t(km)[j];
-            const bool okp = finite_at(kp) && up > th[j], okm = finite_at(km) && dn < th[j];
-            const double* ga = okp ? slot_g(kp) : g;
-            const double* gb = okm ? slot_g(km) : g;
-            const double du = (okp ? up : th[j]) - (okm ? dn : th[j]);
-            for (int i = 0; i < Pt; ++i) H[IDX(i, j)] = (fr[i] && du > 0.0) ? (ga[i] - gb[i]) / du : 0.0;
-            if (c.hsig > 0.0 && okp && okm && up - th[j] == th[j] - dn) {   // symmetric: f's noise
-                const double h = up - th[j];
-                res[ne++] = 0.5 * fabs(F.ft[s0 + kp] + F.ft[s0 + km] - 2.0 * F.f[jf] - H[IDX(j, j)] * h * h);
-            }
-            ++a;
-        }
-        if (ne > 0) {   // median (insertion sort of at most PFMAX values)
-            for (int i = 1; i < ne; ++i)
-                for (int k = i; k > 0 && res[k - 1] > res[k]; --k) {
-                    const double t = res[k];
-                    res[k] = res[k - 1];
-                    res[k - 1] = t;
+        // then carries that direction).  The columns' flags first (a lane per column), then the
+        // columns, a lane per row.
+        int ne = 0;
+        for (int a0 = 0; a0 < nfree; a0 += 32) {
+            const int na = min(32, nfree - a0);
+            bool okp = false, okm = false, noise = false;
+            double up = 0.0, dn = 0.0, ep = 0.0, em = 0.0;
+            int jl = 0;
+            if (lane < na) {
+                jl = sh.fidx[a0 + lane];
+                const int kp = NLS + 2 * (a0 + lane), km = kp + 1;
+                up = slot_t(kp)[jl];
+                dn = slot_t(km)[jl];
+                ep = F.ft[s0 + kp];
+                em = F.ft[s0 + km];
+                bool fp = isfinite(ep), fm = isfinite(em);
+                const double* gp = slot_g(kp);
+                const double* gm = slot_g(km);
+#pragma unroll 4
+                for (int i = 0; i < Pt; ++i) {   // no short circuit: the loads do not wait for each other
+                    fp = fp & (isfinite(__ldg(gp + i)) != 0);
+                    fm = fm & (isfinite(__ldg(gm + i)) != 0);
                 }
+                okp = fp && up > th[jl];
+                okm = fm && dn < th[jl];
+                noise = c.hsig > 0.0 && okp && okm && up - th[jl] == th[jl] - dn;   // symmetric: f's noise
+            }
+            const unsigned mp = __ballot_sync(0xffffffffu, okp), mm = __ballot_sync(0xffffffffu, okm);
+            for (int a = 0; a < na; ++a) {
+                const int j = sh.fidx[a0 + a], kp = NLS + 2 * (a0 + a), km = kp + 1;
+                const bool bp = (mp >> a) & 1u, bm = (mm >> a) & 1u;
+                const double u = __shfl_sync(0xffffffffu, up, a), v = __shfl_sync(0xffffffffu, dn, a);
+                const double du = (bp ? u : th[j]) - (bm ? v : th[j]);
+                for (int i = lane; i < Pt; i += 32) {
+                    const double ga = bp ? __ldg(slot_g(kp) + i) : g[i], gb = bm ? __ldg(slot_g(km) + i) : g[i];
+                    sh.H[SIDX(i, j)] = (sh.fr[i] && du > 0.0) ? (ga - gb) / du : 0.0;
+                }
+            }
+            __syncwarp();
+            const unsigned mn = __ballot_sync(0xffffffffu, noise);
+            if (noise) {
+                const double h = up - th[jl];
+                sh.res[ne + __popc(mn & ((1u << lane) - 1u))] = 0.5 * fabs(ep + em - 2.0 * fcur - sh.H[SIDX(jl, jl)] * h * h);
+            }
+            ne += __popc(mn);
+        }
+        __syncwarp();
+        for (int j = lane; j < Pt * Pt; j += 32) gH[IDX(j / Pt, j % Pt)] = sh.H[SIDX(j / Pt, j % Pt)];
+        if (ne > 0) {   // median of the noise estimates: each value's rank among the others
+            double* res = sh.res;
+            bool nan = false;
+            for (int q = lane; q < ne; q += 32) nan = nan || isnan(res[q]);
+            if (__any_sync(0xffffffffu, nan)) {   // no total order: insertion sort by one lane
+                if (lane == 0)
+                    for (int i = 1; i < ne; ++i)
+                        for (int k = i; k > 0 && res[k - 1] > res[k]; --k) {
+                            const double t = res[k];
+                            res[k] = res[k - 1];
+                            res[k - 1] = t;
+                        }
+            } else {
+                double x[2];
+                int rk[2];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int i = lane + 32 * q;
+                    rk[q] = -1;
+                    if (i >= ne) continue;
+                    x[q] = res[i];
+                    int r = 0;
+                    for (int k = 0; k < ne; ++k) r += (res[k] < x[q] || (res[k] == x[q] && k < i)) ? 1 : 0;
+                    rk[q] = r;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    if (rk[q] >= 0) res[rk[q]] = x[q];
+            }
+            __syncwarp();
             c.fnoise = ne & 1 ? res[ne / 2] : 0.5 * (res[ne / 2 - 1] + res[ne / 2]);
         }
         newdir = fresh = true;
@@ -350,24 +492,33 @@ __global__ void k_fit(FitDev F) {
         // (the correlated resolution terms) can land far out on a descent that a shorter step
         // beats.  At the noise floor of the FP32 -lnL (an undamped step predicting less than
         // EDM_NOISE) the full step counts as a decrease while it stays within the noise.
+        // A lane per step length.
+        double fk = INFINITY;
+        bool dec = false;
+        if (lane < NLS) {
+            fk = F.ft[s0 + lane];
+            if (isfinite(fk)) {
+                double gs = 0.0;
+                const double* tk = slot_t(lane);
+#pragma unroll 4
+                for (int i = 0; i < Pt; ++i) gs += g[i] * (tk[i] - th[i]);
+                const double nz = fmax(EDM_NOISE, c.fnoise);
+                const bool noise_floor = lane == 0 && c.mu_used <= c.mu_conv && c.edm0 < nz && fk <= fcur + 2.0 * nz;
+                dec = fk <= fcur + 1e-4 * gs || noise_floor;
+            }
+        }
+        const unsigned md = __ballot_sync(0xffffffffu, dec);
         int acc = -1;
         double fbest = 0.0;
         for (int k = 0; k < NLS; ++k) {
-            const double fk = F.ft[s0 + k];
-            if (!isfinite(fk)) continue;
-            double gs = 0.0;
-            const double* tk = slot_t(k);
-            for (int i = 0; i < Pt; ++i) gs += g[i] * (tk[i] - th[i]);
-            const double nz = fmax(EDM_NOISE, c.fnoise);
-            const bool noise_floor = k == 0 && c.mu_used <= c.mu_conv && c.edm0 < nz && fk <= F.f[jf] + 2.0 * nz;
-            if ((fk <= F.f[jf] + 1e-4 * gs || noise_floor) && (acc < 0 || fk < fbest)) {
+            const double f = __shfl_sync(0xffffffffu, fk, k);
+            if (((md >> k) & 1u) && (acc < 0 || f < fbest)) {
                 acc = k;
-                fbest = fk;
+                fbest = f;
             }
         }
         if (acc >= 0) {
-            for (int i = 0; i < Pt; ++i) { th[i] = slot_t(acc)[i]; g[i] = slot_g(acc)[i]; }
-            F.f[jf] = F.ft[s0 + acc];
+            accept(acc);
             c.iters++;
             c.mu_min = 0.0;
             to_hess = true;
@@ -396,20 +547,22 @@ __global__ void k_fit(FitDev F) {
         }
     }
     if (newdir) {
-        unsigned char act[PFMAX];
-        for (int i = 0; i < Pt; ++i)
-            act[i] = fr[i] && !((th[i] <= lo[i] && g[i] > 0.0) || (th[i] >= hi[i] && g[i] < 0.0));
-        double L[PFMAX * PFMAX];
-        const double mu = damped_inverse(H, act, Pt, P, fresh ? 0.0 : c.mu_min, V, L);
+        for (int i = lane; i < Pt; i += 32)
+            sh.act[i] = sh.fr[i] && !((th[i] <= lo[i] && g[i] > 0.0) || (th[i] >= hi[i] && g[i] < 0.0));
+        __syncwarp();
+        const double mu = damped_inverse(sh, Pt, fresh ? 0.0 : c.mu_min);
+        // (a runaway leaves V zeroed)
+        for (int j = lane; j < Pt * Pt; j += 32) gV[IDX(j / Pt, j % Pt)] = sh.V[SIDX(j / Pt, j % Pt)];
         double gd = 0.0;
         if (mu >= 0.0) {
-            for (int i = 0; i < Pt; ++i) {
+            for (int i = lane; i < Pt; i += 32) {
                 double t = 0.0;
-                if (act[i])
-                    for (int k = 0; k < Pt; ++k) t -= V[IDX(i, k)] * g[k];
-                d[i] = t;
-                gd += g[i] * t;
+                if (sh.act[i])
+                    for (int k = 0; k < Pt; ++k) t -= sh.V[SIDX(i, k)] * g[k];
+                sh.d[i] = t;
             }
+            __syncwarp();
+            for (int i = 0; i < Pt; ++i) gd += g[i] * sh.d[i];
         }
         if (mu < 0.0 && c.restarts < MAX_RESTARTS) {
             // damping runaway (no damping up to 1e8 gave a positive definite matrix, or line
@@ -430,7 +583,7 @@ __global__ void k_fit(FitDev F) {
                 c.edm0 = c.edm;
                 c.mu_fresh = mu;
                 int nb = 0;
-                for (int i = 0; i < Pt; ++i) nb += (fr[i] && !act[i]) ? 1 : 0;
+                for (int i = 0; i < Pt; ++i) nb += (sh.fr[i] && !sh.act[i]) ? 1 : 0;
                 c.n_bound = nb;
             }
             if (fresh && c.edm < fmax(c.tol, FNOISE_K * c.fnoise) && mu <= c.mu_conv) {
@@ -445,65 +598,57 @@ __global__ void k_fit(FitDev F) {
                 // length (scaling the whole step instead let one tightly limited parameter stall
                 // every other one, and a first step from 10% out had sent the constant noise term c
                 // to hundreds of times its optimum).
-                double lim[PFMAX];
-                for (int i = 0; i < Pt; ++i) {
-                    lim[i] = INFINITY;
-                    if (i >= Kt && act[i]) {
-                        const double v = V[IDX(i, i)];
+                for (int i = lane; i < Pt; i += 32) {
+                    double lim = INFINITY;
+                    if (i >= Kt && sh.act[i]) {
+                        const double v = sh.V[SIDX(i, i)];
                         const double l = fmax(TR_REL * fabs(th[i]), v > 0.0 && isfinite(v) ? TR_SIG * sqrt(v) : 0.0);
-                        if (l > 0.0) lim[i] = l;
+                        if (l > 0.0) lim = l;
+                    }
+                    for (int k = 0; k < NLS; ++k) {
+                        const double a = ldexp(1.0, -k);
+                        slot_t(k)[i] = sh.fr[i] ? fmin(fmax(th[i] + fmin(fmax(a * sh.d[i], -lim), lim), lo[i]), hi[i]) : th[i];
                     }
                 }
-                for (int k = 0; k < NLS; ++k) {
-                    const double a = ldexp(1.0, -k);
-                    double* tk = slot_t(k);
-                    for (int i = 0; i < Pt; ++i)
-                        tk[i] = fr[i] ? fmin(fmax(th[i] + fmin(fmax(a * d[i], -lim[i]), lim[i]), lo[i]), hi[i]) : th[i];
-                    F.skip[s0 + k] = 0;
-                }
-                for (int k = NLS; k < S; ++k) F.skip[s0 + k] = 1;
+                for (int k = lane; k < S; k += 32) F.skip[s0 + k] = k < NLS ? 0 : 1;
                 c.evals += NLS;
             }
         }
     }
     if (to_hess) {
-        int a = 0;
-        for (int j = 0; j < Pt; ++j) {
-            if (!fr[j]) continue;
+        for (int a = lane; a < nfree; a += 32) {   // the steps (kept in lim)
+            const int j = sh.fidx[a];
             double h = c.hrel * fmax(fabs(th[j]), 1e-3);
-            const double hjj = H[IDX(j, j)];
+            const double hjj = sh.H[SIDX(j, j)];
             if (c.hsig > 0.0 && isfinite(c.edm0) && hjj > 0.0 && isfinite(hjj))
                 h = fmin(c.hsig / sqrt(hjj), 0.5 * fmax(fabs(th[j]), 1e-3));
-            double* tp = slot_t(NLS + 2 * a);
-            double* tm = slot_t(NLS + 2 * a + 1);
-            for (int i = 0; i < Pt; ++i) { tp[i] = th[i]; tm[i] = th[i]; }
-            tp[j] = fmin(th[j] + h, hi[j]);
-            tm[j] = fmax(th[j] - h, lo[j]);
-            F.skip[s0 + NLS + 2 * a] = 0;
-            F.skip[s0 + NLS + 2 * a + 1] = 0;
-            ++a;
+            sh.lim[a] = h;
         }
-        for (int k = 0; k < NLS; ++k) F.skip[s0 + k] = 1;
-        for (int k = NLS + 2 * a; k < S; ++k) F.skip[s0 + k] = 1;
-        c.evals += 2 * a;
-        c.phase = a > 0 ? PH_HESS : PH_DONE;
-        if (a == 0) { c.status = BX_OK; c.edm = 0.0; }
+        __syncwarp();
+        for (int q = lane; q < nfree * Pt; q += 32) {
+            const int a = q / Pt, i = q - a * Pt;
+            const double h = sh.lim[a], t = th[i];
+            const bool step = i == sh.fidx[a];
+            slot_t(NLS + 2 * a)[i] = step ? fmin(t + h, hi[i]) : t;
+            slot_t(NLS + 2 * a + 1)[i] = step ? fmax(t - h, lo[i]) : t;
+        }
+        for (int k = lane; k < S; k += 32) F.skip[s0 + k] = k >= NLS && k < NLS + 2 * nfree ? 0 : 1;
+        c.evals += 2 * nfree;
+        c.phase = nfree > 0 ? PH_HESS : PH_DONE;
+        if (nfree == 0) { c.status = BX_OK; c.edm = 0.0; }
     }
     if (c.phase != PH_DONE && c.evals >= c.max_evals) { c.phase = PH_DONE; c.status = BX_ENOTCONV; }
+    __syncwarp();
     if (c.phase == PH_DONE) {   // result out, the next queued fit in
         slot_store(F, jf, c);
-        const int qf = atomicAdd(F.next_fit, 1);
-        if (qf < F.run->n_fits) {
-            slot_load(F, jf, qf);
-            atomicAdd(F.active, 1);
-        } else {
-            F.slot_fit[jf] = -1;
-            for (int k = 0; k < S; ++k) F.skip[s0 + k] = 1;
-        }
+        __syncwarp();
+        if (slot_refill(F, jf) && lane == 0) atomicAdd(F.active, 1);
         return;
     }
-    atomicAdd(F.active, 1);
-    F.ctl[jf] = c;
+    if (lane == 0) {
+        atomicAdd(F.active, 1);
+        F.ctl[jf] = c;
+    }
 }
 
 }  // namespace
@@ -551,7 +696,7 @@ static int fit_alloc(bx_model* m) {
     FitDev& D = s->dev;
     struct A { void** p; size_t bytes; } plan[] = {
         {(void**)&D.theta, n * P * 8}, {(void**)&D.g, n * P * 8},      {(void**)&D.f, n * 8},
-        {(void**)&D.H, n * P * P * 8}, {(void**)&D.V, n * P * P * 8},  {(void**)&D.d, n * P * 8},
+        {(void**)&D.H, n * P * P * 8}, {(void**)&D.V, n * P * P * 8},
         {(void**)&D.lo, n * P * 8},    {(void**)&D.hi, n * P * 8},     {(void**)&D.fr, n * P},
         {(void**)&D.tt, ns * P * 8},   {(void**)&D.ft, ns * 8},        {(void**)&D.gt, ns * P * 8},
         {(void**)&D.skip, ns},         {(void**)&D.ctl, n * sizeof(FitCtl)}, {(void**)&D.active, 16},
@@ -649,7 +794,7 @@ static int fit_capture(bx_model* m, int F, int ipl) {
         if (e != cudaSuccess) break;
         st = bx_enqueue_eval(m, F * s->S, D.tt, s->P, 1, 0, D.ft, D.gt);
         if (st) break;
-        k_fit<<<(F + 63) / 64, 64, 0, s->fs>>>(D);
+        k_fit<<<F, 32, 0, s->fs>>>(D);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && st == BX_OK) {
@@ -822,7 +967,7 @@ extern "C" int bx_fit(bx_model* m, int n, const int* toy_idx, const double* thet
     auto load = [&](int nslots) -> int {
         D.n = nslots;
         CUF(cudaMemsetAsync(D.next_fit, 0, sizeof(int), s->fs));
-        k_fit_init<<<(nslots + 63) / 64, 64, 0, s->fs>>>(D);
+        k_fit_init<<<nslots, 32, 0, s->fs>>>(D);
         CUF(cudaGetLastError());
         return BX_OK;
     };
