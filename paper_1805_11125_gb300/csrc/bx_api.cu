@@ -1,6 +1,6 @@
 // bx_api.cu -- host side of the C ABI (include/bx.h): argument validation, model
 // creation (device copies of every toy, set-up kernel), workspace, and the evaluation
-// driver that enqueues k_prep -> k_fwd_* -> k_mid -> [k_bwd_*] -> k_gather on the
+// driver that enqueues the column stage -> forward -> assembly -> [k_bwd_*] -> k_gather on the
 // model's stream.
 #include <cuda_runtime.h>
 
@@ -441,6 +441,17 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
                                          static_cast<float*>(stiles),
                                          static_cast<float*>(g32), static_cast<double*>(gg), m->stream);
         if (e != cudaSuccess) st = bx_set_error(BX_ECUDA, "set-up kernel: %s", cudaGetErrorString(e));
+        if (m->precision == BX_FP64 && e == cudaSuccess && !st) {   // Gg on the sample grids
+            if (!m->w.tab64) {
+                const std::vector<double>& tab = g64_tables();
+                if ((st = upload(m, tab.data(), tab.size(), &m->w.tab64))) break;
+            }
+            void* gt;
+            if ((st = alloc_dev(m, &gt, sizeof(double) * T.n_es * g64_total(T.M)))) break;
+            T.Gt64 = static_cast<double*>(gt);
+            e = launch_setup_gt64(T, m->w.tab64, static_cast<double*>(gt), m->stream);
+            if (e != cudaSuccess) st = bx_set_error(BX_ECUDA, "set-up kernel: %s", cudaGetErrorString(e));
+        }
         m->Kmax = std::max(m->Kmax, T.K);
         m->Nmax = std::max(m->Nmax, T.Next);
         m->Mmax = std::max(m->Mmax, T.M);
@@ -463,7 +474,11 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
     m->P = m->Pi + 4 * (m->n_est - 1);
     const int cap = m->cap * m->n_est;   // internal items
     Work& w = m->w;
-    w = Work{};
+    {
+        const double* tab64 = w.tab64;
+        w = Work{};
+        w.tab64 = tab64;
+    }
     w.cap = cap;
     w.Npad = ((m->Nmax + 127) / 128) * 128;
     w.Mpad = ((m->Mmax + 127) / 128) * 128;
@@ -493,7 +508,8 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
     w.ncs2d = m->ncs2d;
     if (!m->is2d) {   // the assembly stage holds one item's spectra and columns in shared memory
         size_t need = 0, avail = 0;
-        const cudaError_t e = mid_smem_budget(w, m->Mmax, m->nwmax, m->Lmax, &need, &avail);
+        const cudaError_t e = m->precision == BX_FP64 ? mid64_smem_budget(w, m->Mmax, m->nwmax, m->Lmax, &need, &avail)
+                                                      : mid_smem_budget(w, m->Mmax, m->nwmax, m->Lmax, &need, &avail);
         const int bad = e != cudaSuccess ? 1 : need > avail ? 2 : 0;
         if (bad) {
             cudaStreamSynchronize(m->stream);
@@ -507,7 +523,15 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
                                 need, nwm, Mm, Lm, np, avail);
         }
     }
-    const size_t tv = m->precision == BX_FP64 ? sizeof(double) : sizeof(float);
+    const bool f64 = m->precision == BX_FP64;
+    const size_t tv = f64 ? sizeof(double) : sizeof(float);
+    w.gp_rows = f64 ? w.Npad / 32 : MAX_CB;
+    w.gl64 = f64 ? g64_total(m->Mmax) : 0;
+    w.wt_threads64 = f64 ? g64_wt_threads(m->Mmax) : 0;
+    // 32-sample tiles a column's samples can touch: 18 sigma at 0.1 sigma a sample and one more each
+    // side (under 186 samples); a band wider than 8 sigma puts the columns on the bins
+    w.nslot64 = m->band <= 8.0 ? 7 : (m->Mmax + 31) / 32 + 1;
+    const size_t c64 = f64 ? cap : 0;
     const bool species = m->precision == BX_TF32X3;
     struct A {
         void** p;
@@ -517,22 +541,33 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.toy_of, sizeof(int) * cap},
         {(void**)&w.col64, sizeof(Col64) * cap * w.Npad},
         {(void**)&w.colq, sizeof(double2) * cap * w.Npad},
-        {(void**)&w.colf, sizeof(float4) * cap * w.Npad},
-        {(void**)&w.colg, sizeof(ColG) * cap * w.Npad},
-        {(void**)&w.colS, sizeof(double2) * cap * w.Npad},
-        {(void**)&w.colS32, sizeof(float4) * cap * w.Npad},
-        {(void**)&w.colAl, sizeof(float) * cap * w.Npad},
+        {(void**)&w.colf, f64 ? 16 : sizeof(float4) * cap * w.Npad},
+        {(void**)&w.colg, f64 ? 16 : sizeof(ColG) * cap * w.Npad},
+        {(void**)&w.colS, f64 ? sizeof(double2) * cap * w.Npad : 16},
+        {(void**)&w.colS32, f64 ? 16 : sizeof(float4) * cap * w.Npad},
+        {(void**)&w.colAl, f64 ? 16 : sizeof(float) * cap * w.Npad},
         {(void**)&w.aW, sizeof(double) * cap * w.nes * w.Npad},
-        {(void**)&w.colr, sizeof(int2) * cap * w.Npad},
+        {(void**)&w.colr, f64 ? 16 : sizeof(int2) * cap * w.Npad},
         {(void**)&w.lam, sizeof(double) * cap * 2 * w.Mpad},
-        {(void**)&w.apart, m->any_cols && !species ? 2 * sizeof(float) * cap * m->max_tiles * w.nes * w.Npad : 16},
-        {(void**)&w.tile_cols, sizeof(int2) * cap * MAX_SETS * MAX_TILES},
-        {(void**)&w.cb_rows, sizeof(int2) * cap * MAX_CB},
+        {(void**)&w.apart, m->any_cols && !species && !f64 ? 2 * sizeof(float) * cap * m->max_tiles * w.nes * w.Npad : 16},
+        {(void**)&w.tile_cols, f64 ? 16 : sizeof(int2) * cap * MAX_SETS * MAX_TILES},
+        {(void**)&w.cb_rows, f64 ? 16 : sizeof(int2) * cap * MAX_CB},
+        {(void**)&w.qtot64, sizeof(double2) * c64 * (w.Npad / 128)},
+        {(void**)&w.gen64, sizeof(Gen64) * c64 * w.Npad},
+        {(void**)&w.colc64, sizeof(int4) * c64 * w.Npad},
+        {(void**)&w.chk64, sizeof(int2) * c64 * (w.Npad / 32) * (G64_NC + 1)},
+        {(void**)&w.cmask64, sizeof(int) * c64},
+        {(void**)&w.ap64, m->any_cols ? sizeof(double) * c64 * w.nslot64 * w.nes * w.Npad : 16},
+        {(void**)&w.F64, sizeof(double) * (f64 ? std::max((size_t)cap, (size_t)4 * std::min(cap, G64_SPLIT)) : 0) * 2 * w.gl64},
+        {(void**)&w.mc64, m->any_cols ? sizeof(double) * c64 * (w.Npad / 32) * w.nes * 32 : 16},
+        {(void**)&w.wt64, sizeof(double) * c64 * (2 + w.nes) * w.gl64},
+        {(void**)&w.wv64, sizeof(double) * c64 * 2 * w.Mpad},
+        {(void**)&w.part64, sizeof(double) * c64 * 2 * ((m->nwmax + 31) / 32) * 4},
         {(void**)&w.v, species ? 2 * tv * cap * w.Mpad * US : 16},   // hi, lo planes
         {(void**)&w.rowW, tv * cap * (2 + w.nes) * w.Mpad},
         {(void**)&w.coef, sizeof(double) * cap * (2 + w.nes) * KMAX},
         {(void**)&w.gmid, sizeof(double) * cap * PMAX},
-        {(void**)&w.gpart, sizeof(double) * cap * MAX_CB * GPN},
+        {(void**)&w.gpart, sizeof(double) * cap * w.gp_rows * GPN},
         {(void**)&w.nll, sizeof(double) * cap},
         {(void**)&w.mu, sizeof(double) * cap * m->nbmax},
         {(void**)&w.status, sizeof(int) * cap},
@@ -720,7 +755,12 @@ static int enqueue_items(bx_model* m, int n, const double* theta_dev, int tstrid
     int st;
     BxRange eval_range("bx_eval");
     if ((st = prof_mark(m, 0))) return st;
-    { BxRange r("bx_prep"); CU(launch_prep(w, n, s)); }
+    const bool f64 = m->precision == BX_FP64;
+    {
+        BxRange r("bx_prep");
+        if (f64) CU(launch_prep64(w, n, s));
+        else CU(launch_prep(w, n, s));
+    }
     if ((st = prof_mark(m, 1))) return st;
     if (m->is2d) {
         { BxRange r("bx_forward_2d"); CU(launch_eval2d(w, n, want_grad, want_mu, 1, s)); }
@@ -734,14 +774,22 @@ static int enqueue_items(bx_model* m, int n, const double* theta_dev, int tstrid
     }
     {
         BxRange r("bx_forward");
-        if (m->precision == BX_FP64) CU(launch_fwd_f64(w, n, m->max_tiles, m->any_tag, m->any_cols, s));
+        if (f64) CU(launch_fwd64(w, n, m->any_tag, m->any_cols, s));
         else if (m->precision == BX_FP32) CU(launch_fwd_f32(w, n, m->max_tiles, m->any_tag, m->any_cols, s));
         else CU(launch_fwd_tc(w, n, m->max_tiles, s));
     }
     if ((st = prof_mark(m, 2))) return st;
-    { BxRange r("bx_assembly"); CU(launch_mid(w, n, m->Mmax, m->nwmax, m->Lmax, want_grad, want_mu, s)); }
+    {
+        BxRange r("bx_assembly");
+        if (f64) CU(launch_mid64(w, n, m->Mmax, m->nwmax, m->Lmax, 1 + m->any_tag, want_grad, want_mu, s));
+        else CU(launch_mid(w, n, m->Mmax, m->nwmax, m->Lmax, want_grad, want_mu, s));
+    }
     if ((st = prof_mark(m, 3))) return st;
-    if (want_grad) { BxRange r("bx_adjoint"); CU(launch_bwd(w, n, m->max_cb, s)); }
+    if (want_grad) {
+        BxRange r("bx_adjoint");
+        if (f64) CU(launch_bwd64(w, n, s));
+        else CU(launch_bwd(w, n, m->max_cb, s));
+    }
     if ((st = prof_mark(m, 4))) return st;
     { BxRange r("bx_gather"); CU(launch_gather(w, n, nll_dev, grad_dev, want_grad, s)); }
     if ((st = prof_mark(m, 5))) return st;

@@ -13,10 +13,8 @@
 // the chain rule through mu_i = LY Q_i(kB), sigma_i^2 = a mu_i + b mu_i^2 + c gives the
 // partial gradient of (LY, a, b, c, kB), and dNLL/dr_k gets
 // sum_i s_k[i] (c_{vetoed,k} rho_vetoed[i] + c_{tagged,k} rho_tagged[i]).
-//   k_bwd_f64: exact bin mass from erfc tails and exact derivatives -(phi(z_b) - phi(z_a))/sigma,
-//              -(z_b phi(z_b) - z_a phi(z_a))/sigma, FP64 throughout (with a Gram-Charlier
-//              response its CDF and density in place of Phi and phi).
-//   k_bwd_f32: the same integrals by the forward pass's 3-point Gauss-Legendre rule
+//   (the FP64 model's adjoint is in bx_f64.cu)
+//   k_bwd_f32: the integrals by the forward pass's 3-point Gauss-Legendre rule
 //              (integrands phi, t phi, (t^2 - 1) phi) in round-to-nearest FP32, down each
 //              column by the row recurrence of bx_resp.cuh (adj_run), column sums
 //              in FP32 per chunk of rows and FP64 across chunks, the chain rule in FP64; the
@@ -32,38 +30,8 @@ namespace bx {
 
 constexpr int RCH = 256;   // rows per staged chunk
 
-__device__ __forceinline__ void chain_rule(const Col64& cc, const double2& q, const double* th, int K, double S0,
-                                           double S1, double S2, double (&g)[GPN]) {
-    const double LY = th[K], a = th[K + 1], b = th[K + 2];
-    const double mu = cc.mu, sig = cc.sig;
-    const double dmu = S1 - cc.mills / sig * S0;
-    const double dsig = S2 + cc.mills * mu / (sig * sig) * S0;
-    const double Gmu = dmu + dsig * (a + 2.0 * b * mu) / (2.0 * sig);
-    g[0] = Gmu * q.x;                       // LY
-    g[1] = dsig * mu / (2.0 * sig);         // a
-    g[2] = dsig * mu * mu / (2.0 * sig);    // b
-    g[3] = dsig / (2.0 * sig);              // c
-    g[4] = Gmu * LY * q.y;                  // kB
-}
-
 // A column's place among the sets: column ie is grid point ig of set grp (a quenching group or a
 // radial shell); species k contributes to it with the weight set_weight(T, k, grp).
-
-// rate part: g[5 + k] = w_k s_k[i] (c_vetoed,k rho_vetoed + c_tagged,k rho_tagged) for the species
-// of the column's set (grid point i, set grp, weight w_k)
-template <bool MULTI>
-__device__ __forceinline__ void rate_part(const Toy& T, int i, int grp, double rs, double rt, double (&g)[GPN]) {
-#pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        const double wk = k < T.K ? set_weight<MULTI>(T, k, grp) : 0.0;
-        if (wk != 0.0) {
-            const double t = T.tag ? T.tag[k] : 0.0;
-            g[5 + k] = wk * T.shapes[(size_t)k * T.N + i] * ((T.tag ? 1.0 - t : 1.0) * rs + t * rt);
-        } else {
-            g[5 + k] = 0.0;
-        }
-    }
-}
 
 // FP32 shape of species k at grid point ig times its weight wk in the column's set (0 outside
 // its quenching group: no load)
@@ -71,119 +39,6 @@ template <bool MULTI>
 __device__ __forceinline__ float shape_w(const Toy& T, int k, int ig, float wk) {
     if (!MULTI) return T.shapes32[(size_t)k * T.N + ig];
     return wk != 0.f ? wk * T.shapes32[(size_t)k * T.N + ig] : 0.f;
-}
-
-__device__ __forceinline__ void block_sum_gp(double (&g)[GPN], double* red, double* out) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int j = 0; j < GPN; ++j) {
-        const double s = warp_sum(g[j]);
-        if (lane == 0) red[wid * GPN + j] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < GPN) {
-        double s = 0.0;
-        for (int q = 0; q < nw; ++q) s += red[q * GPN + threadIdx.x];
-        out[threadIdx.x] = s;
-    }
-}
-
-// Species sums of the column's adjoint weights: vetoed, tagged, and one per energy slice q
-// of the Eq. 4 terms (SA[q], 0 beyond the toy's slices).
-template <bool MULTI>
-__device__ __forceinline__ void column_weights(const Work& w, const Toy& T, int item, int i, int grp, bool ok,
-                                               double& Ssub, double& Stag, double (&SA)[MAX_ES]) {
-    const double* coef = w.coef + (size_t)item * (2 + w.nes) * KMAX;
-    Ssub = Stag = 0.0;
-    for (int q = 0; q < MAX_ES; ++q) SA[q] = 0.0;
-    if (!ok) return;
-    for (int k = 0; k < T.K; ++k) {
-        const double wk = set_weight<MULTI>(T, k, grp);
-        if (wk == 0.0) continue;
-        const double s = wk * T.shapes[(size_t)k * T.N + i];
-        Ssub += coef[k] * s;
-        Stag += coef[KMAX + k] * s;
-        for (int q = 0; q < T.n_es; ++q) SA[q] += coef[(2 + q) * KMAX + k] * s;
-    }
-}
-
-template <bool MULTI>
-__global__ void __launch_bounds__(BCOLS) k_bwd_f64(Work w) {
-    // 1D item-major grid (a y dimension would cap the batch at 65535 items)
-    const int cb = blockIdx.x % w.max_cb, item = blockIdx.x / w.max_cb, tid = threadIdx.x;
-    const Toy& T = w.toys[w.toy_of[item]];
-    if (cb >= T.n_cb) return;
-    double* gp = w.gpart + ((size_t)item * MAX_CB + cb) * GPN;
-    if (w.status[item]) {
-        if (tid < GPN) gp[tid] = 0.0;
-        return;
-    }
-    const int i = cb * BCOLS + tid;   // column (of quenching group grp, grid point ig)
-    const int grp = MULTI ? i / T.Ncs : 0, ig = MULTI ? i - grp * T.Ncs : i;
-    const bool ok = MULTI ? (i < T.Next && ig < T.N) : i < T.N;
-    const int2 rr = w.cb_rows[(size_t)item * MAX_CB + cb];
-    if (MULTI && rr.x >= rr.y) {   // no column of this block has support in its quenching group
-        if (tid < GPN) gp[tid] = 0.0;
-        return;
-    }
-    const int r0 = max(rr.x, max(0, T.m_lo - T.L + 1)), r1 = min(rr.y, T.M);
-    double Ssub, Stag, SA[MAX_ES];
-    column_weights<MULTI>(w, T, item, ig, grp, ok, Ssub, Stag, SA);
-    const Col64 cc = ok ? w.col64[(size_t)item * w.Npad + i] : Col64{0.0, 1.0, 0.0, 0.0};
-    const double* rw = static_cast<const double*>(w.rowW) + (size_t)item * (2 + w.nes) * w.Mpad;
-    const int NES = T.n_es;
-    __shared__ double sW[2 + MAX_ES][RCH];   // wt_sub, wt_tag, G_W of each energy slice
-    __shared__ double red[GPN * (BCOLS / 32)];
-    double S0 = 0.0, S1 = 0.0, S2 = 0.0, Rs = 0.0, Rt = 0.0;
-    double ta = 0.0, pa = 0.0, zpa = 0.0;
-    bool fa = false;
-    const double inv_sig = 1.0 / cc.sig;
-    const bool gc = T.gc1 != 0.0 || T.gc2 != 0.0;
-    auto edge = [&](int e, double& t, double& p, double& zp, bool& f) {
-        const double z = ((double)e * T.w - cc.mu) * inv_sig;
-        f = z >= 0.0;
-        t = f ? -0.5 * erfc(z * 0.70710678118654752440) : 0.5 * erfc(-z * 0.70710678118654752440);
-        p = INV_SQRT_2PI * exp(-0.5 * z * z);
-        if (gc) {   // Gram-Charlier: CDF Phi - phi C, density phi (1 + gc1 He3 + gc2 He4)
-            t -= gc_cdf_term(T, z);
-            p *= gc_density_factor(T, z);
-        }
-        zp = z * p;
-    };
-    if (ok && r0 < r1) edge(r0, ta, pa, zpa, fa);
-    for (int c0 = r0; c0 < r1; c0 += RCH) {
-        const int nr = min(RCH, r1 - c0);
-        for (int j = tid; j < nr; j += BCOLS)
-            for (int r = 0; r < 2 + NES; ++r) sW[r][j] = rw[(size_t)r * w.Mpad + c0 + j];
-        __syncthreads();
-        if (ok) {
-            for (int j = 0; j < nr; ++j) {
-                double tb, pb, zpb;
-                bool fb;
-                edge(c0 + j + 1, tb, pb, zpb, fb);
-                double W = sW[0][j] * Ssub + sW[1][j] * Stag;
-                for (int q = 0; q < NES; ++q) W += sW[2 + q][j] * SA[q];
-                const double D = tb - ta + ((!fa && fb) ? 1.0 : 0.0);
-                S0 += W * D;
-                S1 -= W * (pb - pa);
-                S2 -= W * (zpb - zpa);
-                Rs += D * sW[0][j];
-                Rt += D * sW[1][j];
-                ta = tb; pa = pb; zpa = zpb; fa = fb;
-            }
-        }
-        __syncthreads();
-    }
-    double g[GPN];
-#pragma unroll
-    for (int j = 0; j < GPN; ++j) g[j] = 0.0;
-    if (ok) {
-        const double* th = w.theta + (size_t)item * w.tstride;
-        chain_rule(cc, w.colq[(size_t)item * w.Npad + i], th, T.K, cc.norm * S0, cc.norm * S1 * inv_sig,
-                   cc.norm * S2 * inv_sig, g);
-        rate_part<MULTI>(T, ig, grp, cc.norm * Rs, cc.norm * Rt, g);
-    }
-    block_sum_gp(g, red, gp);
 }
 
 // GC: the Gram-Charlier response, whose node sums are taken row by row (resp_adjoint32_gc): the
@@ -194,7 +49,7 @@ __global__ void __launch_bounds__(BCOLS, 7) k_bwd_f32(Work w) {
     const int cb = blockIdx.x % w.max_cb, item = blockIdx.x / w.max_cb, tid = threadIdx.x;
     const Toy& T = w.toys[w.toy_of[item]];
     if (cb >= T.n_cb) return;
-    double* gp = w.gpart + ((size_t)item * MAX_CB + cb) * GPN;
+    double* gp = w.gpart + ((size_t)item * w.gp_rows + cb) * GPN;
     if (w.status[item]) {
         if (tid < GPN) gp[tid] = 0.0;
         return;
@@ -438,21 +293,16 @@ __global__ void __launch_bounds__(BCOLS, 7) k_bwd_f32(Work w) {
 
 cudaError_t launch_bwd(const Work& w, int n, int max_cb, cudaStream_t s) {
     const unsigned grid = (unsigned)n * (unsigned)w.max_cb;   // decoded with w.max_cb
-    if (w.precision == BX_FP64) {
-        if (w.multi_set) k_bwd_f64<true><<<grid, BCOLS, 0, s>>>(w);
-        else k_bwd_f64<false><<<grid, BCOLS, 0, s>>>(w);
-    } else {
-        const bool mes = w.nes > 1;   // several energy slices of the Eq. 4 terms
-        if (w.gc) {   // the Gram-Charlier response (one quenching group)
-            if (w.multi_set && mes) k_bwd_f32<true, true, true><<<grid, BCOLS, 0, s>>>(w);
-            else if (w.multi_set) k_bwd_f32<true, false, true><<<grid, BCOLS, 0, s>>>(w);
-            else if (mes) k_bwd_f32<false, true, true><<<grid, BCOLS, 0, s>>>(w);
-            else k_bwd_f32<false, false, true><<<grid, BCOLS, 0, s>>>(w);
-        } else if (w.multi_set && mes) k_bwd_f32<true, true><<<grid, BCOLS, 0, s>>>(w);
-        else if (w.multi_set) k_bwd_f32<true, false><<<grid, BCOLS, 0, s>>>(w);
-        else if (mes) k_bwd_f32<false, true><<<grid, BCOLS, 0, s>>>(w);
-        else k_bwd_f32<false, false><<<grid, BCOLS, 0, s>>>(w);
-    }
+    const bool mes = w.nes > 1;   // several energy slices of the Eq. 4 terms
+    if (w.gc) {   // the Gram-Charlier response (one quenching group)
+        if (w.multi_set && mes) k_bwd_f32<true, true, true><<<grid, BCOLS, 0, s>>>(w);
+        else if (w.multi_set) k_bwd_f32<true, false, true><<<grid, BCOLS, 0, s>>>(w);
+        else if (mes) k_bwd_f32<false, true, true><<<grid, BCOLS, 0, s>>>(w);
+        else k_bwd_f32<false, false, true><<<grid, BCOLS, 0, s>>>(w);
+    } else if (w.multi_set && mes) k_bwd_f32<true, true><<<grid, BCOLS, 0, s>>>(w);
+    else if (w.multi_set) k_bwd_f32<true, false><<<grid, BCOLS, 0, s>>>(w);
+    else if (mes) k_bwd_f32<false, true><<<grid, BCOLS, 0, s>>>(w);
+    else k_bwd_f32<false, false><<<grid, BCOLS, 0, s>>>(w);
     return cudaGetLastError();
 }
 
@@ -474,8 +324,8 @@ __global__ void __launch_bounds__(128) k_gather(Work w, int n, double* nll_out, 
         g = w.gmid[(size_t)item * PMAX + j];
         const int slot = j < T.K ? 5 + j : j < T.K + 5 ? j - T.K : -1;
         if (slot >= 0) {
-            const double* gp = w.gpart + (size_t)item * MAX_CB * GPN + slot;
-            const int ncb = T.n_cb;
+            const double* gp = w.gpart + (size_t)item * w.gp_rows * GPN + slot;
+            const int ncb = w.precision == BX_FP64 ? (T.Next + 31) / 32 : T.n_cb;
 #pragma unroll 8
             for (int cb = 0; cb < ncb; ++cb) g += gp[cb * GPN];
         }

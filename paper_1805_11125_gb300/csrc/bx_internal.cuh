@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "bx.h"
 
 namespace bx {
@@ -45,6 +47,12 @@ constexpr double GL_W_SCALE = 1.0 / 9.0;
 // sqrt(0.5 * log2(e)): exp(-z^2 / 2) = 2^(-(z * S_EX2)^2)
 constexpr double S_EX2 = 0.84932180028801904272;
 constexpr double INV_SQRT_2PI = 0.39894228040143267794;
+
+// FP64 model (bx_f64.cu): sample grids of the response density
+constexpr int G64_R = 16;       // stencil half width (samples before and after the axis)
+constexpr int G64_NC = 7;       // sampled classes, spacing 2^c bins; then the bins themselves
+constexpr int G64_CI = G64_NC;
+constexpr int G64_SPLIT = 4;    // batches up to this size split the forward's tiles over more CTAs
 
 constexpr int GPN = 5 + KMAX;   // backward partials per column block: LY, a, b, c, kB, rates
 
@@ -92,6 +100,7 @@ struct Toy {
     const float* g32;         // [L]
     const double* Gg;         // [n_es][M]: sum over the slice's window bins m' of g[m' - m] (0 <= m'-m < L)
     const float* Gg32;        // [n_es][M]: the same in FP32, stored after Gg
+    const double* Gt64;       // FP64 model: [n_es][g64_total(M)] Gg on the class grids (transposed stencils)
     const double* cnt;        // [nb] data, concatenated (vetoed, tagged, radial, PSD, 2D slices)
     const float2* cnt32;      // [nb] the same as FP32 pairs hi + lo
     const int* rad_class;     // [K]
@@ -124,6 +133,11 @@ struct Col64 {
     double mu, sig, norm, mills;   // mean, width, 1/Phi(mu/sig), phi(mu/sig)/Phi(mu/sig)
 };
 
+// Generator constants of a column of the FP64 model (bx_f64.cu).
+struct __align__(16) Gen64 {
+    double x, y, z, w;   // mu, 1/sigma, 1 - e^(-h^2), amplitude
+};
+
 // Workspace of a model: every array has `cap` item slots.
 struct Work {
     int cap, Npad, Mpad, nbmax, pstride, n_items, max_tiles, max_cb;
@@ -142,7 +156,7 @@ struct Work {
     double2* colq;            // [cap][Npad]: Q_i, dQ_i/dkB
     float4* colf;             // [cap][Npad]: (floor(mu/w), c_hi, hs_hi, hs_lo): hs = w/sig*S_EX2, c = (1/2 - frac(mu/w)) hs
     ColG* colg;               // [cap][Npad]
-    double2* colS;            // [cap][Npad]: S_vetoed[i], S_tagged[i] (FP64 model)
+    double2* colS;            // [cap][Npad]: S_vetoed[i], S_tagged[i] times the column's amplitude (FP64 model)
     float4* colS32;           // [cap][Npad]: A_i S_h[i] for the rate-first FP32 forward as double-float pairs
                               // (vetoed hi, tagged hi, vetoed lo, tagged lo)
     float* colAl;             // [cap][Npad]: A_i - colg[i].A, the low part of the column amplitude (the
@@ -153,8 +167,8 @@ struct Work {
     double* lam;              // [cap][2][Mpad]: lambda_h[m] (rate-first forward); FP32 pairs when lam_pairs
     int lam_pairs;            // rate-first mixed precision: the forward writes lam as FP32 pairs
     int multi_set;            // some toy has several quenching groups (selects the kernels that handle them)
-    void* apart;              // [cap][max_tiles][H][nes][Npad]: column sums of R Gg_s per tile, FP64 (H = 1)
-                              // or per half tile (one warp's 64 rows), FP32 (H = 2)
+    float* apart;             // [cap][max_tiles][2][nes][Npad]: column sums of R Gg_s per half tile (one warp's
+                              // 64 rows)
     int2* tile_cols;          // [cap][MAX_SETS][MAX_TILES]: column range of each forward tile, per
                               // quenching group (tile_range); only the toy's groups are written
     int2* cb_rows;            // [cap][MAX_CB]: row range of each backward column block
@@ -162,7 +176,8 @@ struct Work {
     void* rowW;               // [cap][2 + nes][Mpad] float or double: wt_sub, wt_tag, G_W of every slice
     double* coef;             // [cap][2 + nes][KMAX]: vetoed, tagged, then each slice's Eq. 4 coefficients
     double* gmid;             // [cap][PMAX]
-    double* gpart;            // [cap][MAX_CB][GPN]
+    double* gpart;            // [cap][gp_rows][GPN]: per 128 columns (FP64 model: per 32)
+    int gp_rows;
     double* nll;              // [cap]
     double* mu;               // [cap][nbmax]
     int* status;              // [cap]
@@ -170,6 +185,20 @@ struct Work {
     unsigned long long* units;   // in-band response entries evaluated (counted when count_units)
     int count_units;
     int shells;               // some toy has radial response shells (k_prep32's SHELL instantiations)
+    // FP64 model (bx_f64.cu)
+    const double* tab64;      // stencils of every class and phase, then 2^(j/64)
+    double2* qtot64;          // [cap][Npad/128]: Birks sums of each 128-column block
+    Gen64* gen64;             // [cap][Npad]: mu, 1/sigma, 1 - e^(-h^2), amplitude
+    int4* colc64;             // [cap][Npad]: class (-1: none), kind, sample range [z, w) on the class grid
+    int2* chk64;              // [cap][Npad/32][G64_NC + 1]: sample range of each class in a 32-column chunk
+    int* cmask64;             // [cap]: classes present
+    double* ap64;             // [cap][nslot64][nes][Npad]: column sums over the column's 32-sample tiles
+    double* F64;              // [cap][2][gl64]: density sums on the class grids (small batches: [n][4][2][gl64])
+    double* mc64;             // [cap][Npad/32][nes][32]: chunk sums of the Eq. 4 marginals
+    double* wt64;             // [cap][2 + nes][gl64]: row weights on the class grids
+    double* wv64;             // [cap][2][Mpad]: 1 - n/mu on the window
+    double* part64;           // [cap][2 * window tiles][4]: -lnL sum and compensation, d/deps, domain flag
+    int nslot64, gl64, wt_threads64;
     const unsigned char* skip;   // [cap] or nullptr: items flagged 1 are not evaluated (-lnL = +inf)
     // 2D model buffers (UMMA K-major tiles of TF32 hi | lo halves, NSL slices x KB)
     float* coef2d;            // [cap][4][KMAX][NSL]: r_k dT/dr_k, dT/dr_k, r_k dT/ds_r coefficients, and the
@@ -216,7 +245,17 @@ constexpr int STATUS_SKIPPED = 1;   // item status of a skipped evaluation
 cudaError_t launch_setup_toy(const Toy& t, float* shapes32, float* shapes32l, float* S_tiles, float* g32, double* Gg,
                              cudaStream_t s);
 cudaError_t launch_prep(const Work& w, int n, cudaStream_t s);
-cudaError_t launch_fwd_f64(const Work& w, int n, int max_tiles, int any_tag, int any_cols, cudaStream_t s);
+// FP64 model: nH its spectra (1 or 2)
+const std::vector<double>& g64_tables();
+int g64_total(int M);
+int g64_wt_threads(int M);
+cudaError_t launch_setup_gt64(const Toy& t, const double* tab, double* Gt, cudaStream_t s);
+cudaError_t launch_prep64(const Work& w, int n, cudaStream_t s);
+cudaError_t launch_fwd64(const Work& w, int n, int any_tag, int any_cols, cudaStream_t s);
+cudaError_t launch_mid64(const Work& w, int n, int Mmax, int nwmax, int Lmax, int nH, int want_grad, int want_mu,
+                         cudaStream_t s);
+cudaError_t launch_bwd64(const Work& w, int n, cudaStream_t s);
+cudaError_t mid64_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail);
 cudaError_t launch_fwd_tc(const Work& w, int n, int max_tiles, cudaStream_t s);
 cudaError_t launch_fwd_f32(const Work& w, int n, int max_tiles, int any_tag, int any_cols, cudaStream_t s);
 // Dynamic shared memory the assembly kernel needs per item for these sizes, and the most the

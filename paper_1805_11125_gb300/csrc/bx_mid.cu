@@ -61,14 +61,6 @@ struct Dot32 {
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
-struct Dot64 {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <typename TV> struct DotT { using type = Dot64; };
-template <> struct DotT<float> { using type = Dot32; };
-
 // bc_term_far on FP64 arguments (the TF32X3 assembly)
 __device__ __forceinline__ bool bc_term_far_d(double n, double mu, double& term, double& wb) {
     df t;
@@ -102,9 +94,10 @@ __device__ void radial_probs(const Toy& T, double s_r, double* sF, double* sdF, 
     }
 }
 
-template <typename TV, bool SPECIES>
-__global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !SPECIES) ? 2 : 1)
-    k_mid(Work w, int want_grad, int want_mu) {
+// The assembly of the species-resolved tensor-core mode (BX_TF32X3): FP32 pile-up and weights, FP64
+// spectra and terms.
+__global__ void __launch_bounds__(MID_THREADS, 1) k_mid(Work w, int want_grad, int want_mu) {
+    using TV = float;
     extern __shared__ __align__(16) double dsm[];
     const int item = blockIdx.x, tid = threadIdx.x;
     const Toy& T = w.toys[w.toy_of[item]];
@@ -149,23 +142,16 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
     __syncthreads();
 
     // Eq. 3: the energy spectra on the full axis
-    constexpr bool species = SPECIES;
-    const double* lamg = w.lam + (size_t)item * 2 * w.Mpad;
     for (int m = tid; m < M; m += MID_THREADS) {
         double ls = 0.0, lt = 0.0;
-        if (species) {
-            const TV* vr = v + (size_t)m * US;
+        const TV* vr = v + (size_t)m * US;
 #pragma unroll
-            for (int k = 0; k < KMAX; ++k)
-                if (k < K) {
-                    const double x = (double)vr[k] + (double)vr[vlo + k];
-                    ls += s_rs[k] * x;
-                    lt += s_rt[k] * x;
-                }
-        } else {
-            ls = lamg[m];
-            lt = H == 2 ? lamg[w.Mpad + m] : 0.0;
-        }
+        for (int k = 0; k < KMAX; ++k)
+            if (k < K) {
+                const double x = (double)vr[k] + (double)vr[vlo + k];
+                ls += s_rs[k] * x;
+                lt += s_rt[k] * x;
+            }
         lam[m] = ls;
         lamT[m] = (TV)ls;
         if (H == 2) {
@@ -180,7 +166,7 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
         const int h = idx / nw, j = idx % nw, m = m_lo + j;
         const TV* x = lamT + h * M;
         const int dmax = min(m, L - 1);
-        typename DotT<TV>::type conv;
+        Dot32 conv;
         for (int d = 0; d <= dmax; ++d) conv.add(gT[d], x[m - d]);
         const double cv = conv.value();
         puT[idx] = (TV)cv;
@@ -193,67 +179,20 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
         double part[2 * KMAX];
 #pragma unroll
         for (int k = 0; k < 2 * KMAX; ++k) part[k] = 0.0;
-        if (species) {
-            for (int m = tid; m < M; m += MID_THREADS) {
-                const double inW = m >= T.es_lo[qs] && m < T.es_hi[qs] ? 1.0 : 0.0, gg = T.Gg[(size_t)qs * M + m];
-                const double GW = (1.0 - eps) * inW + eps * gg, dG = gg - inW;
-                const TV* vr = v + (size_t)m * US;
+        for (int m = tid; m < M; m += MID_THREADS) {
+            const double inW = m >= T.es_lo[qs] && m < T.es_hi[qs] ? 1.0 : 0.0, gg = T.Gg[(size_t)qs * M + m];
+            const double GW = (1.0 - eps) * inW + eps * gg, dG = gg - inW;
+            const TV* vr = v + (size_t)m * US;
 #pragma unroll
-                for (int k = 0; k < KMAX; ++k)
-                    if (k < K) {
-                        const double x = (double)vr[k] + (double)vr[vlo + k];
-                        part[k] += x * GW;
-                        part[KMAX + k] += x * dG;
-                    }
-            }
-        } else {
-            // sum_m v_k[m] G_W[m] = sum_i s_k[i] ((1 - eps) aW[i] + eps a[i]), a[i] from the
-            // per-tile column sums of the forward (valid on each tile's band only)
-            constexpr int HALF = sizeof(TV) == sizeof(float) ? 2 : 1;   // slots per tile
-            const TV* ap = static_cast<const TV*>(w.apart) + (size_t)item * w.max_tiles * HALF * w.nes * w.Npad;
-            const double* aWi = w.aW + ((size_t)item * w.nes + qs) * w.Npad;
-            const int lane = tid & 31, wid = tid >> 5;
-            {   // FP64 model (the rate-first FP32 mode runs k_mid32)
-                // column ie = grp Ncs + i of quenching group grp carries the species of that group
-                // (of radial shell grp: every species, with its fraction in the shell)
-                for (int ie = tid; ie < T.Next; ie += MID_THREADS) {
-                    const int grp = ie / T.Ncs, i = ie - grp * T.Ncs;
-                    if (i >= T.N) continue;
-                    const int2* tcols = w.tile_cols + ((size_t)item * MAX_SETS + grp) * MAX_TILES;
-                    double ag = 0.0;
-                    for (int t = 0; t < T.n_tiles; ++t) {
-                        const int2 cr = tcols[t];
-                        if (ie >= cr.x && ie < cr.y)
-                            for (int h = 0; h < HALF; ++h) ag += (double)ap[(((size_t)t * HALF + h) * w.nes + qs) * w.Npad + ie];
-                    }
-                    const double aw = aWi[ie];
-                    const double GW = (1.0 - eps) * aw + eps * ag, dG = ag - aw;
-#pragma unroll
-                    for (int k = 0; k < KMAX; ++k)
-                        if (k < K) {
-                            const double wk = set_weight<true>(T, k, grp);
-                            if (wk == 0.0) continue;
-                            const double x = T.shapes[(size_t)k * T.N + i] * wk;
-                            part[k] += x * GW;
-                            part[KMAX + k] += x * dG;
-                        }
+            for (int k = 0; k < KMAX; ++k)
+                if (k < K) {
+                    const double x = (double)vr[k] + (double)vr[vlo + k];
+                    part[k] += x * GW;
+                    part[KMAX + k] += x * dG;
                 }
-#pragma unroll
-                for (int k = 0; k < 2 * KMAX; ++k) {
-                    const double r = warp_sum(part[k]);
-                    if (lane == 0) red[wid * 2 * KMAX + k] = r;
-                }
-            }
-            __syncthreads();
-            if (tid < 2 * KMAX) {
-                double v = 0.0;
-                for (int q = 0; q < MID_WARPS; ++q) v += red[q * 2 * KMAX + tid];
-                s_SA[qs][tid] = v;
-            }
-            __syncthreads();
         }
         // s_SA[q][k] = sum v G_W,q, s_SA[q][KMAX+k] = sum v dG_W,q/deps
-        if (species) block_sum<2 * KMAX>(part, red, s_SA[qs]);
+        block_sum<2 * KMAX>(part, red, s_SA[qs]);
     }
     // radial bin probabilities (internal: uniform in volume; external: exponential from r_iv)
     if (nrad > 0) radial_probs(T, s_r, s_F, s_dF, s_pint, s_pext, s_dpext);
@@ -294,7 +233,7 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
         double term, wb = 1.0;
         if (n == 0.0) term = mu;
         else if (!(mu > 0.0 && isfinite(mu))) { dom = 1; term = 0.0; }
-        else if (sizeof(TV) == sizeof(float) && bc_term_far_d(n, mu, term, wb)) {}
+        else if (bc_term_far_d(n, mu, term, wb)) {}
         else {
             term = (mu - n) + n * log1p((n - mu) / mu);
             wb = 1.0 - n / mu;
@@ -363,7 +302,7 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
         const int h = idx / M, m = idx % M;
         const TV* wh = wvT + h * nw;
         const int d0 = max(0, m_lo - m), d1 = min(L - 1, M - 1 - m);
-        typename DotT<TV>::type acc;
+        Dot32 acc;
         for (int d = d0; d <= d1; ++d) acc.add(gT[d], wh[m + d - m_lo]);
         const double direct = (m >= m_lo) ? (1.0 - eps) * (double)wh[m - m_lo] : 0.0;
         const TV val = (TV)(direct + eps * acc.value());
@@ -378,10 +317,8 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
             mv && q < NES ? (TV)((1.0 - eps) * inW + eps * T.Gg[(size_t)q * M + m]) : (TV)0;
     }
     __syncthreads();
-    // rate gradient, part through the spectra: sum_h c_{h,k} sum_m wt_h[m] v_k[m]; only the
-    // tensor-core path has v here, the rate-first path gets it from k_bwd_* as
-    // sum_h c_{h,k} sum_i s_k[i] sum_m R[m,i] wt_h[m]
-    if (species) {
+    // rate gradient, part through the spectra: sum_h c_{h,k} sum_m wt_h[m] v_k[m]
+    {
         double part[2 * KMAX];
 #pragma unroll
         for (int k = 0; k < 2 * KMAX; ++k) part[k] = 0.0;
@@ -397,8 +334,6 @@ __global__ void __launch_bounds__(MID_THREADS, (sizeof(TV) == sizeof(float) && !
                 }
         }
         block_sum<2 * KMAX>(part, red, s_gr);
-    } else if (tid < 2 * KMAX) {
-        s_gr[tid] = 0.0;
     }
     __syncthreads();
     double* coef = w.coef + (size_t)item * (2 + w.nes) * KMAX;
@@ -845,27 +780,11 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
     }
 }
 
-template <typename TV, bool SPECIES>
-static cudaError_t launch_mid_t(const Work& w, int n, size_t smem, int want_grad, int want_mu, cudaStream_t s) {
-    // the attribute is set once per size (outside any stream capture that replays it)
-    static size_t set = 0;
-    if (smem > set) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_mid<TV, SPECIES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        set = smem;
-    }
-    k_mid<TV, SPECIES><<<n, MID_THREADS, smem, s>>>(w, want_grad, want_mu);
-    return cudaGetLastError();
-}
-
 // Dynamic shared memory of the assembly kernel the workspace's precision selects, for the
 // model's largest axis (Mmax), window (nwmax) and pile-up spectrum (Lmax).
 static size_t mid_dynamic_smem(const Work& w, int Mmax, int nwmax, int Lmax) {
-    if (w.precision != BX_FP32) {   // k_mid: lambda and mu in FP64, the rest in the kernel's type
-        const size_t tv = w.precision == BX_FP64 ? sizeof(double) : sizeof(float);
-        return (size_t)(2 * Mmax + 2 * nwmax) * sizeof(double) + (size_t)(2 * Mmax + 4 * nwmax + Lmax) * tv + 64;
-    }
+    if (w.precision != BX_FP32)   // k_mid: lambda and mu in FP64, the rest in FP32
+        return (size_t)(2 * Mmax + 2 * nwmax) * sizeof(double) + (size_t)(2 * Mmax + 4 * nwmax + Lmax) * sizeof(float) + 64;
     // k_mid32: mu pairs [2][nw], g, lambda rows, pile-up part [2][nw], weight rows (zero-padded),
     // G_W and dG_W/deps per column
     return (size_t)2 * nwmax * sizeof(float2) +
@@ -877,8 +796,7 @@ cudaError_t mid_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t
     *need = mid_dynamic_smem(w, Mmax, nwmax, Lmax);
     cudaFuncAttributes fa{};
     cudaError_t e;
-    if (w.precision == BX_FP64) e = cudaFuncGetAttributes(&fa, k_mid<double, false>);
-    else if (w.precision == BX_TF32X3) e = cudaFuncGetAttributes(&fa, k_mid<float, true>);
+    if (w.precision == BX_TF32X3) e = cudaFuncGetAttributes(&fa, k_mid);
     else e = w.nes > 1 ? cudaFuncGetAttributes(&fa, k_mid32<true>) : cudaFuncGetAttributes(&fa, k_mid32<false>);
     if (e != cudaSuccess) return e;
     int dev = 0, optin = 0;
@@ -891,8 +809,17 @@ cudaError_t mid_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t
 cudaError_t launch_mid(const Work& w, int n, int Mmax, int nwmax, int Lmax, int want_grad, int want_mu,
                        cudaStream_t s) {
     const size_t smem = mid_dynamic_smem(w, Mmax, nwmax, Lmax);
-    if (w.precision == BX_FP64) return launch_mid_t<double, false>(w, n, smem, want_grad, want_mu, s);
-    if (w.precision == BX_TF32X3) return launch_mid_t<float, true>(w, n, smem, want_grad, want_mu, s);
+    // the attribute is set once per size (outside any stream capture that replays it)
+    if (w.precision == BX_TF32X3) {
+        static size_t set = 0;
+        if (smem > set) {
+            const cudaError_t e = cudaFuncSetAttribute(k_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            set = smem;
+        }
+        k_mid<<<n, MID_THREADS, smem, s>>>(w, want_grad, want_mu);
+        return cudaGetLastError();
+    }
     static size_t set32[2] = {0, 0};
     const int mes = w.nes > 1 ? 1 : 0;   // several energy slices of the Eq. 4 terms
     if (smem > set32[mes]) {

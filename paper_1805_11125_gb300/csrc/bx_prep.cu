@@ -5,10 +5,10 @@
 //   tensor-core operand layout, FP32 pile-up spectrum,
 //   and the pile-up window marginal of every energy slice W_s of the Eq. 4 terms,
 //   Gg_s[m] = sum_{m' in W_s, 0 <= m'-m < L} g[m'-m] (FP64, then an FP32 copy after them).
-// k_prep (FP64 model) and k_prep32 (mixed-precision modes), once per item: Eq. 1's Birks map
-//   and resolution on the true-energy grid (block-wide prefix sum), the column normalisation
-//   1/Phi(mu/sigma), the window masses, the rate-weighted spectra of Eq. 3 and the band limits
-//   of every tile; k_prep32 also the FP32 parameters of the generated response.
+// k_prep32 (mixed-precision modes; the FP64 model's column stage is in bx_f64.cu), once per item:
+//   Eq. 1's Birks map and resolution on the true-energy grid (block-wide prefix sum), the column
+//   normalisation 1/Phi(mu/sigma), the window masses, the rate-weighted spectra of Eq. 3, the band
+//   limits of every tile and the FP32 parameters of the generated response.
 #include <float.h>
 #include <limits.h>
 #include <math.h>
@@ -85,220 +85,6 @@ __device__ __forceinline__ double gauss_mass(double a, double b) {
     return 1.0 - upper_tail(b) - upper_tail(-a);
 }
 
-// Block-wide exclusive scan of two doubles (256 threads); ta, tb receive the block totals.
-__device__ void block_scan2(double& a, double& b, double& ta, double& tb, double* sh) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double ia = a, ib = b;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        double xa = __shfl_up_sync(0xffffffffu, ia, o), xb = __shfl_up_sync(0xffffffffu, ib, o);
-        if (lane >= o) { ia += xa; ib += xb; }
-    }
-    if (lane == 31) { sh[wid] = ia; sh[8 + wid] = ib; }
-    __syncthreads();
-    if (wid == 0) {
-        double wa = lane < 8 ? sh[lane] : 0.0, wb = lane < 8 ? sh[8 + lane] : 0.0;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-            double xa = __shfl_up_sync(0xffffffffu, wa, o), xb = __shfl_up_sync(0xffffffffu, wb, o);
-            if (lane >= o) { wa += xa; wb += xb; }
-        }
-        if (lane < 8) { sh[16 + lane] = wa - sh[lane]; sh[24 + lane] = wb - sh[8 + lane]; }
-    }
-    __syncthreads();
-    a = sh[16 + wid] + ia - a;
-    b = sh[24 + wid] + ib - b;
-    ta = sh[16 + 7] + sh[7];
-    tb = sh[24 + 7] + sh[8 + 7];
-    __syncthreads();
-}
-
-// One thread per true-energy column, the grid walked in chunks of 256 consecutive columns
-// (coalesced loads and stores; neighbouring lanes take the same branches), the Birks prefix
-// sum carried from chunk to chunk.  Tile and column-block bounds are reduced over the warp
-// (redux) before one shared atomic per warp and tile.
-// The FP64 model's column stage: every quantity in FP64 -- the Birks prefix sums, mu, sigma,
-// 1/Phi(mu/sigma) and phi/Phi (only where mu/sigma < 9: elsewhere 1 and < 1e-18), the window
-// mass (erfc only for window edges within 9 sigma), the rate-weighted spectra
-// S_h[i] = sum_k r_k c_{h,k} s_k[i]; FP32 only for the response band (a work bound, not a
-// result).  The FP64 generator works from mu and sigma.
-template <bool MULTI>
-__global__ void __launch_bounds__(256) k_prep(Work w) {
-    const int item = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
-    if (w.skip && w.skip[item]) {   // uniform for the block: no barrier is skipped unevenly
-        if (tid == 0) w.status[item] = STATUS_SKIPPED;
-        return;
-    }
-    const Toy& T = w.toys[w.toy_of[item]];
-    const int K = T.K, N = T.N, M = T.M;
-    const double* th = w.theta + (size_t)item * w.tstride;
-    __shared__ double sh[32];
-    __shared__ int s_bad;
-    __shared__ int s_tlo[MAX_SETS][MAX_TILES], s_thi[MAX_SETS][MAX_TILES], s_rlo[MAX_CB], s_rhi[MAX_CB];
-    if (tid == 0) s_bad = 0;
-    for (int j = tid; j < MAX_SETS * MAX_TILES; j += blockDim.x) {
-        s_tlo[j / MAX_TILES][j % MAX_TILES] = INT_MAX;
-        s_thi[j / MAX_TILES][j % MAX_TILES] = INT_MIN;
-    }
-    for (int j = tid; j < MAX_CB; j += blockDim.x) { s_rlo[j] = INT_MAX; s_rhi[j] = INT_MIN; }
-    __syncthreads();
-    if (tid < T.P && !isfinite(th[tid])) s_bad = 1;
-    const double LY = th[K], a = th[K + 1], b = th[K + 2], c = th[K + 3], kB = th[K + 4];
-    if (tid == 0 && (!(LY > 0.0) || ((T.n_rad > 0 || T.n_r2 > 0) && !(th[K + 6] > 0.0)))) s_bad = 1;
-
-    const double w_ = T.w;
-    const float wf = (float)w_, inv_wf = (float)(1.0 / w_), bandf = (float)w.band;
-    const float e_min = -2.0f * wf, e_max = (M + 2.0f) * wf;
-    Col64* col = w.col64 + (size_t)item * w.Npad;
-    double2* cq = w.colq + (size_t)item * w.Npad;
-    double2* cs = w.colS + (size_t)item * w.Npad;
-    double* aW = w.aW + (size_t)item * w.nes * w.Npad;   // [nes][Npad]: one mass per energy slice
-    const int NES = T.n_es;
-    int2* cr = w.colr + (size_t)item * w.Npad;
-    int bad = 0;
-    unsigned long long inband = 0;
-    // species-specific quenching: one pass per group grp of species, with Birks constant
-    // kB xi[grp], into the group's columns [grp Ncs, grp Ncs + N); a position-dependent
-    // response: one pass per radial shell, with light yield LY lyf[grp]
-    const int NS = MULTI ? T.n_set : 1;
-    for (int grp = 0; grp < NS; ++grp) {
-    const int off = grp * T.Ncs;
-    const double xi = MULTI ? T.xi[grp] : 1.0, kBc = kB * xi;
-    const double lyf = MULTI && T.n_shell ? T.lyf[grp] : 1.0;
-    double carry_x = 0.0, carry_y = 0.0;
-    for (int c0 = 0; c0 < N; c0 += 256) {
-        const int i = c0 + tid, ie = off + i;
-        const bool in = i < N;
-        // a1: Q_i = sum_{j<i} x_j + x_i / 2, x_j = dE / (1 + kB S_j); dQ_i/dkB likewise
-        double x = 0.0, y = 0.0;
-        if (in) {
-            const double S = T.stop_pow[i], q = 1.0 + kBc * S;
-            if (!(q > 0.0)) bad = 1;
-            const double rq = 1.0 / q;
-            x = T.dE * rq;
-            y = -x * S * rq * xi;   // dx / dkB
-        }
-        double ex = x, ey = y, tx, ty;
-        block_scan2(ex, ey, tx, ty, sh);
-        int r0 = 0, r1 = 0;
-        bool valid = false;
-        bool live = in;
-        if (MULTI && in) {   // a group's column without support: only the scan above is needed
-            bool nz = false;
-            for (int k = 0; k < K; ++k)
-                if (set_weight<MULTI>(T, k, grp) != 0.0) nz |= T.shapes[(size_t)k * N + i] != 0.0;
-            if (!nz) {
-                live = false;
-                col[ie] = Col64{0.0, 1.0, 0.0, 0.0};
-                cq[ie] = make_double2(0.0, 0.0);
-                cs[ie] = make_double2(0.0, 0.0);
-                for (int q = 0; q < NES; ++q) aW[(size_t)q * w.Npad + ie] = 0.0;
-                cr[ie] = make_int2(0, 0);
-            }
-        }
-        if (live) {
-            // (a radial shell's light-yield factor folded into Q: mu = LY Q, dmu/dLY = Q)
-            double Q = carry_x + ex + 0.5 * x, dQ = carry_y + ey + 0.5 * y;
-            if (MULTI) {
-                Q *= lyf;
-                dQ *= lyf;
-            }
-            cq[ie] = make_double2(Q, dQ);
-            const double mu = LY * Q;
-            const double var = fma(fma(b, mu, a), mu, c);
-            const bool ok = var > 0.0;
-            if (!ok) bad = 1;
-            const double isig = rsqrt(fmax(var, 1e-300));
-            const double sig = var * isig;
-            const double z = mu * isig;
-            double norm = 1.0, mills = 0.0;
-            const bool gc = T.gc1 != 0.0 || T.gc2 != 0.0;
-            if (z < Q_CUT) {
-                // mass above 0 npe, 1 - F(-z), and the density at -z over it (d ln N / d(mu / sigma))
-                double Phi = z > 0.0 ? 1.0 - upper_tail(z) : upper_tail(-z), dens = INV_SQRT_2PI * exp(-0.5 * z * z);
-                if (gc) {
-                    Phi += gc_cdf_term(T, -z);
-                    dens *= gc_density_factor(T, -z);
-                }
-                norm = 1.0 / Phi;
-                mills = dens * norm;
-            }
-            col[ie] = Col64{mu, sig, norm, mills};
-            // rate-weighted spectra of the vetoed (or single) and tagged events (Eq. 3)
-            double ssub = 0.0, stag = 0.0;
-            bool nz = false;   // a species of this group has support in the column
-            for (int k = 0; k < K; ++k) {
-                const double wk = set_weight<MULTI>(T, k, grp);
-                if (wk == 0.0) continue;
-                nz |= T.shapes[(size_t)k * N + i] != 0.0;
-                const double sk = T.shapes[(size_t)k * N + i] * th[k] * wk;
-                const double t = T.tag ? T.tag[k] : 0.0;
-                ssub += (T.tag ? 1.0 - t : 1.0) * sk;
-                stag += t * sk;
-            }
-            cs[ie] = make_double2(ssub, stag);
-            // mass of the column in each energy slice of the window (Eq. 4 marginals)
-            for (int q = 0; q < NES; ++q) {
-                const double za = (T.es_lo[q] * w_ - mu) * isig, zb = (T.es_hi[q] * w_ - mu) * isig;
-                double mass = gauss_mass(za, zb);
-                if (gc) mass -= gc_cdf_term(T, zb) - gc_cdf_term(T, za);
-                aW[(size_t)q * w.Npad + ie] = mass * norm;
-            }
-            // response band: rows whose bin lies within band * sigma of mu
-            const float muf = (float)mu, sigf = (float)sig;
-            const float lo_e = fminf(fmaxf(muf - bandf * sigf, e_min), e_max);
-            const float hi_e = fminf(fmaxf(muf + bandf * sigf, e_min), e_max);
-            r0 = max(0, (int)floorf(lo_e * inv_wf));
-            r1 = min(M, (int)floorf(hi_e * inv_wf) + 1);
-            valid = ok && r0 < r1 && (!MULTI || nz);   // a group's columns without support are skipped
-            if (valid) inband += (unsigned long long)(r1 - r0);
-            cr[ie] = valid ? make_int2(r0, r1) : make_int2(0, 0);
-        }
-        carry_x += tx;
-        carry_y += ty;
-        // tile column ranges and column-block row ranges, reduced over the warp first
-        const unsigned full = 0xffffffffu;
-        const int t0 = valid ? r0 / TM : INT_MAX, t1 = valid ? (r1 - 1) / TM : INT_MIN;
-        const int tmin = __reduce_min_sync(full, t0), tmax = __reduce_max_sync(full, t1);
-        for (int t = tmin; t <= tmax; ++t) {
-            const bool touch = valid && t >= t0 && t <= t1;
-            const int lo = __reduce_min_sync(full, touch ? ie : INT_MAX);
-            const int hi = __reduce_max_sync(full, touch ? ie + 1 : INT_MIN);
-            if (lane == 0 && lo != INT_MAX) {
-                atomicMin(&s_tlo[grp][t], lo);
-                atomicMax(&s_thi[grp][t], hi);
-            }
-        }
-        // a warp's 32 columns lie in one column block (BCOLS is a multiple of 32)
-        const int rlo = __reduce_min_sync(full, valid ? r0 : INT_MAX);
-        const int rhi = __reduce_max_sync(full, valid ? r1 : INT_MIN);
-        if (lane == 0 && rlo != INT_MAX) {   // off: a multiple of BCOLS
-            atomicMin(&s_rlo[ie / BCOLS], rlo);
-            atomicMax(&s_rhi[ie / BCOLS], rhi);
-        }
-    }
-    }
-    // padding: the columns between groups and after the last one
-    for (int i = tid; i < w.Npad; i += blockDim.x) {
-        const int cpad = i / T.Ncs;
-        if (cpad < NS && i - cpad * T.Ncs < N) continue;
-        col[i] = Col64{0.0, 1.0, 0.0, 0.0};
-        cq[i] = make_double2(0.0, 0.0);
-        cs[i] = make_double2(0.0, 0.0);
-        for (int q = 0; q < NES; ++q) aW[(size_t)q * w.Npad + i] = 0.0;
-        cr[i] = make_int2(0, 0);
-    }
-    if (bad) s_bad = 1;
-    if (w.count_units && inband) atomicAdd(w.units, inband);
-    __syncthreads();
-    for (int j = tid; j < NS * MAX_TILES; j += blockDim.x)
-        w.tile_cols[(size_t)item * MAX_SETS * MAX_TILES + j] = make_int2(s_tlo[j / MAX_TILES][j % MAX_TILES],
-                                                                         s_thi[j / MAX_TILES][j % MAX_TILES]);
-    for (int j = tid; j < MAX_CB; j += blockDim.x)
-        w.cb_rows[(size_t)item * MAX_CB + j] = make_int2(s_rlo[j], s_rhi[j]);
-    if (tid == 0) w.status[item] = s_bad ? (int)BX_EDOMAIN : 0;
-}
-
 // The mixed-precision column stage takes the normalisation's Gaussian tail in FP32 from Z_F32
 // standard deviations on: Q(3) = 1.3e-3, so FP32's relative error (a few 1e-7, the argument's
 // rounding included) stays below 1e-9 absolute; nearer the mean it takes the FP64 tail.
@@ -370,6 +156,10 @@ __device__ void block_scan_df(df& a, df& b, df& ta, df& tb, float* sh) {
     __syncthreads();
 }
 
+// One thread per true-energy column, the grid walked in chunks of 256 consecutive columns
+// (coalesced loads and stores; neighbouring lanes take the same branches), the Birks prefix
+// sum carried from chunk to chunk.  Tile and column-block bounds are reduced over the warp
+// (redux) before one shared atomic per warp and tile.
 // The per-column stage of the mixed-precision modes in double-float FP32 (bx_df.cuh, ~2^-44
 // relative): the Birks prefix sums, 1/(1 + kB S), mu, sigma^2, 1/sigma by one Newton step, the
 // generator's split constants.  FP64 only where a column's Gaussian reaches 0 npe within
@@ -677,19 +467,14 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
 }
 
 cudaError_t launch_prep(const Work& w, int n, cudaStream_t s) {
-    if (w.precision == BX_FP64) {
-        if (w.multi_set) k_prep<true><<<n, 256, 0, s>>>(w);
-        else k_prep<false><<<n, 256, 0, s>>>(w);
-    } else {
-        if (w.shells) {   // radial shells of the response (their own instantiations)
-            if (w.gc) k_prep32<true, true, true><<<n, 256, 0, s>>>(w);
-            else k_prep32<true, false, true><<<n, 256, 0, s>>>(w);
-        } else if (w.gc) {
-            if (w.multi_set) k_prep32<true, true><<<n, 256, 0, s>>>(w);
-            else k_prep32<false, true><<<n, 256, 0, s>>>(w);
-        } else if (w.multi_set) k_prep32<true><<<n, 256, 0, s>>>(w);
-        else k_prep32<false><<<n, 256, 0, s>>>(w);
-    }
+    if (w.shells) {   // radial shells of the response (their own instantiations)
+        if (w.gc) k_prep32<true, true, true><<<n, 256, 0, s>>>(w);
+        else k_prep32<true, false, true><<<n, 256, 0, s>>>(w);
+    } else if (w.gc) {
+        if (w.multi_set) k_prep32<true, true><<<n, 256, 0, s>>>(w);
+        else k_prep32<false, true><<<n, 256, 0, s>>>(w);
+    } else if (w.multi_set) k_prep32<true><<<n, 256, 0, s>>>(w);
+    else k_prep32<false><<<n, 256, 0, s>>>(w);
     return cudaGetLastError();
 }
 
