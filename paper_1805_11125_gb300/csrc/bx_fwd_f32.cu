@@ -32,13 +32,22 @@
 namespace bx {
 
 constexpr int FCH32 = 32;
+constexpr int SPW = 20;    // floats of a staged column pair (16-byte rows; 14 in use)
 
 // acc += a (b + bl), Kahan-compensated: bl is the low part of the column's double-float spectrum,
-// so that the one rounding per term is the product's (independent from entry to entry)
-__device__ __forceinline__ void kahan_fma(float& acc, float& cmp, float a, float b, float bl) {
-    const float y = fmaf(a, b, fmaf(a, bl, -cmp));
+// so that the one rounding per term is the product's (independent from entry to entry).  The
+// compensation is kept negated (nc = -c).
+__device__ __forceinline__ void kahan_fma(float& acc, float& nc, float a, float b, float bl) {
+    const float y = fmaf(a, b, fmaf(a, bl, nc));
     const float t = __fadd_rn(acc, y);
-    cmp = __fsub_rn(__fsub_rn(t, acc), y);
+    nc = __fsub_rn(y, __fsub_rn(t, acc));
+    acc = t;
+}
+// The same on both halves of a pair.
+__device__ __forceinline__ void kahan_fma2(f2& acc, f2& nc, f2 a, f2 b, f2 bl) {
+    const f2 y = f2_fma(a, b, f2_fma(a, bl, nc));
+    const f2 t = f2_add(acc, y);
+    nc = f2_sub(y, f2_sub(t, acc));
     acc = t;
 }
 
@@ -65,12 +74,13 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
     // warp-private staging of 32 columns at a time (no block-wide barrier)
     __shared__ float4 sC[WPC][FCH32];
     __shared__ ColG sG[WPC][FCH32];
+    __shared__ __align__(16) float sP[GC ? 1 : WPC][GC ? 1 : FCH32 / 2][SPW];   // column pairs: ColPair's fields
     __shared__ float4 sS[WPC][FCH32];
     // column sums: one slice -> R Gg of the lane's two rows added (32 values per column);
     // several slices (MES) -> R of each of the warp's 64 rows
-    constexpr int CBR = MES ? 64 : 32;
-    __shared__ float colbuf[COLS ? WPC : 1][COLS ? CBR : 1][FCH32 + 1];
-    float(*cb)[FCH32 + 1] = colbuf[COLS ? qs : 0];
+    constexpr int CBR = MES ? 64 : 32, CBW = FCH32 + 2;   // (even rows: a pair of columns is one store)
+    __shared__ __align__(8) float colbuf[COLS ? WPC : 1][COLS ? CBR : 1][CBW];
+    float(*cb)[CBW] = colbuf[COLS ? qs : 0];
 
     const int ra = g + lane, rb = ra + 32;
     const float mfa = (float)ra, mfb = (float)rb;
@@ -99,8 +109,10 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
         centre_df(mf, cf, cg.c_lo, th, tl);
         return shape_t(wide_tag, th, tl, cg);
     };
-    auto column = [&](auto wide_tag, bool inA, bool inB, const float4& cf, const ColG& cg, const float4 S,
-                      float& Ra, float& Rb) {
+    auto column = [&](auto wide_tag, bool inA, bool inB, int c, float& Ra, float& Rb) {
+        const float4 cf = sC[qs][c];
+        const ColG cg = sG[qs][c];
+        const float4 S = sS[qs][c];
         if (inA && inB) {   // row B's centre from row A's: one double-float add
             float tha, tla, thb, tlb;
             centre_df(mfa, cf, cg.c_lo, tha, tla);
@@ -123,6 +135,73 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
             if (TAG) kahan_fma(tb, ctb, Rb, S.y, S.w);
         }
     };
+    // both rows' entries of one column added: with TAG a row's two spectra share an instruction,
+    // without it the two rows
+    auto add_col = [&](const float4& S, float Ra, float Rb) {
+        if (TAG) {
+            const f2 b = f2_pack(S.x, S.y), bl = f2_pack(S.z, S.w);
+            f2 acc = f2_pack(sa, ta), nc = f2_pack(csa, cta);
+            kahan_fma2(acc, nc, f2_dup(Ra), b, bl);
+            f2_get(acc, sa, ta);
+            f2_get(nc, csa, cta);
+            acc = f2_pack(sb, tb), nc = f2_pack(csb, ctb);
+            kahan_fma2(acc, nc, f2_dup(Rb), b, bl);
+            f2_get(acc, sb, tb);
+            f2_get(nc, csb, ctb);
+        } else {
+            f2 acc = f2_pack(sa, sb), nc = f2_pack(csa, csb);
+            kahan_fma2(acc, nc, f2_pack(Ra, Rb), f2_dup(S.x), f2_dup(S.z));
+            f2_get(acc, sa, sb);
+            f2_get(nc, csa, csb);
+        }
+    };
+    const f2 mfa2 = f2_dup(mfa), gga2 = f2_dup(gga), ggb2 = f2_dup(ggb);
+    // columns 2 pr and 2 pr + 1, both rows of every lane inside both bands (most of the work): four
+    // entries a thread in packed arithmetic, added in column order
+    auto pair = [&](int pr) {
+        f2 RA, RB;
+        if constexpr (GC) {   // four scalar evaluations in flight
+            const float4 cf0 = sC[qs][2 * pr], cf1 = sC[qs][2 * pr + 1];
+            const ColG cg0 = sG[qs][2 * pr], cg1 = sG[qs][2 * pr + 1];
+            float t0, l0, t1, l1, u0, k0, u1, k1;
+            centre_df(mfa, cf0, cg0.c_lo, t0, l0);
+            centre_df(mfa, cf1, cg1.c_lo, t1, l1);
+            centre_step32(t0, l0, cf0, u0, k0);
+            centre_step32(t1, l1, cf1, u1, k1);
+            RA = f2_pack(shape_t(std::true_type{}, t0, l0, cg0), shape_t(std::true_type{}, t1, l1, cg1));
+            RB = f2_pack(shape_t(std::true_type{}, u0, k0, cg0), shape_t(std::true_type{}, u1, k1, cg1));
+        } else {
+            const float4* P = reinterpret_cast<const float4*>(sP[GC ? 0 : qs][GC ? 0 : pr]);
+            const float4 v0 = P[0], v1 = P[1], v2 = P[2], v3 = P[3];
+            ColPair k;
+            k.x = f2_pack(v0.x, v0.y);
+            k.y = f2_pack(v0.z, v0.w);
+            k.z = f2_pack(v1.x, v1.y);
+            k.w = f2_pack(v1.z, v1.w);
+            k.cl = f2_pack(v2.x, v2.y);
+            k.kap = f2_pack(v2.z, v2.w);
+            k.Ck2 = f2_pack(v3.x, v3.y);
+            f2 th, tl, uh, ul;
+            centre_df2(mfa2, k, th, tl);
+            centre_step2(th, tl, k, f2_dup(32.0f), uh, ul);
+            resp_shape32_x4(k, th, tl, uh, ul, RA, RB);
+        }
+        float a0, a1, b0, b1;
+        f2_get(RA, a0, a1);
+        f2_get(RB, b0, b1);
+        add_col(sS[qs][2 * pr], a0, b0);
+        add_col(sS[qs][2 * pr + 1], a1, b1);
+        if (COLS) {
+            if (MES) {
+                *reinterpret_cast<float2*>(&cb[lane][2 * pr]) = make_float2(a0, a1);
+                *reinterpret_cast<float2*>(&cb[lane + 32][2 * pr]) = make_float2(b0, b1);
+            } else {
+                float x, y;
+                f2_get(f2_fma(RB, ggb2, f2_mul(RA, gga2)), x, y);
+                *reinterpret_cast<float2*>(&cb[lane][2 * pr]) = make_float2(x, y);
+            }
+        }
+    };
 
     for (int grp = 0; grp < NGRP; ++grp) {
     const int2 cr = tile_range(w, item, grp, tile);
@@ -132,7 +211,8 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
         // whether the column's band touches them (mA, mB) and whether |z| <= 1 at every row
         // of the warp (mW: t = (m - floor(mu/w)) hs + c is linear in the row m, so its two
         // end rows bound it)
-        unsigned mA, mB, mW;
+        unsigned mA, mB, mW, mP;   // mP: |t| <= 11 as well (the packed generator's range)
+        float Al = 0.f;            // the lane's column amplitude
         {
             const bool in = lane < ncol;
             const int i = c0 + lane;
@@ -140,24 +220,44 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
             const ColG cgl = in ? colg[i] : ColG{0.f, 0.f, 0.f, 0.f};
             sC[qs][lane] = cfl;
             sG[qs][lane] = cgl;
+            if (!GC) {
+                float* P = sP[GC ? 0 : qs][GC ? 0 : lane >> 1] + (lane & 1);
+                P[0] = cfl.x;
+                P[2] = cfl.y;
+                P[4] = cfl.z;
+                P[6] = cfl.w;
+                P[8] = cgl.c_lo;
+                P[10] = cgl.kap;
+                P[12] = cgl.Ck2;
+            }
+            Al = cgl.A;
             sS[qs][lane] = in ? colS[i] : make_float4(0.f, 0.f, 0.f, 0.f);
             const int2 band = in ? colr[i] : make_int2(0, 0);
             const float t0 = fmaf((float)g - cfl.x, cfl.z, cfl.y), t1 = fmaf(63.0f, cfl.z, t0);
+            const float tm = fmaxf(fabsf(t0), fabsf(t1));
             mA = __ballot_sync(0xffffffffu, band.x < g + 32 && band.y > g);
             mB = __ballot_sync(0xffffffffu, band.x < g + 64 && band.y > g + 32);
-            mW = __ballot_sync(0xffffffffu, cgl.kap * fmaxf(fabsf(t0), fabsf(t1)) <= 0.99f);
+            mW = __ballot_sync(0xffffffffu, cgl.kap * tm <= 0.99f);
+            mP = GC ? 0xffffffffu : __ballot_sync(0xffffffffu, tm <= 10.9f);
         }
         __syncwarp();
-        const unsigned mAny = mA | mB;
+        const unsigned mAny = mA | mB, m1 = mA & mB & mW & mP;
+        const unsigned m2 = m1 & (m1 >> 1) & 0x55555555u;   // column pairs for the packed path
+        if (m2 == 0x55555555u) {
+#pragma unroll 2
+            for (int pr = 0; pr < FCH32 / 2; ++pr) pair(pr);
+        } else
         for (unsigned mr = mAny; mr; mr &= mr - 1u) {   // the columns whose band touches the warp
             const int c = __ffs(mr) - 1;
-            const float4 cf = sC[qs][c];
-            const ColG cg = sG[qs][c];
-            const float4 S = sS[qs][c];
+            if ((m2 >> c) & 1u) {
+                pair(c >> 1);
+                mr &= mr - 1u;
+                continue;
+            }
             const bool inA = (mA >> c) & 1u, inB = (mB >> c) & 1u;
             float Ra = 0.f, Rb = 0.f;
-            if ((mW >> c) & 1u) column(std::true_type{}, inA, inB, cf, cg, S, Ra, Rb);
-            else column(std::false_type{}, inA, inB, cf, cg, S, Ra, Rb);
+            if ((mW >> c) & 1u) column(std::true_type{}, inA, inB, c, Ra, Rb);
+            else column(std::false_type{}, inA, inB, c, Ra, Rb);
             if (COLS) {
                 if (MES) {
                     cb[lane][c] = Ra;
@@ -172,7 +272,7 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
             float s = 0.f;
             if ((mAny >> lane) & 1u)
                 for (int j = 0; j < 32; ++j) s += cb[j][lane];
-            if (lane < ncol) apart[c0 + lane] = s * sG[qs][lane].A;
+            if (lane < ncol) apart[c0 + lane] = s * Al;
             __syncwarp();
         }
         if (COLS && MES) {
@@ -189,16 +289,16 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
             if (lane < ncol)
 #pragma unroll
                 for (int e = 0; e < MAX_ES; ++e)
-                    if (e < NES) apart[(size_t)e * w.Npad + c0 + lane] = s[e] * sG[qs][lane].A;
+                    if (e < NES) apart[(size_t)e * w.Npad + c0 + lane] = s[e] * Al;
             __syncwarp();
         }
     }
     }
     double* lam = w.lam + (size_t)item * 2 * w.Mpad;
-    if (w.lam_pairs) {   // the Kahan sum s - c as a normalised FP32 pair
+    if (w.lam_pairs) {   // the Kahan sum as a normalised FP32 pair
         float2* lp = reinterpret_cast<float2*>(lam);
         const auto pair = [](float sum, float comp) {
-            const df p = df_two_sum(sum, -comp);
+            const df p = df_two_sum(sum, comp);
             return make_float2(p.h, p.l);
         };
         if (ra < M) {
@@ -212,12 +312,12 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
         return;
     }
     if (ra < M) {
-        lam[ra] = (double)sa - (double)csa;
-        if (TAG) lam[w.Mpad + ra] = (double)ta - (double)cta;
+        lam[ra] = (double)sa + (double)csa;
+        if (TAG) lam[w.Mpad + ra] = (double)ta + (double)cta;
     }
     if (rb < M) {
-        lam[rb] = (double)sb - (double)csb;
-        if (TAG) lam[w.Mpad + rb] = (double)tb - (double)ctb;
+        lam[rb] = (double)sb + (double)csb;
+        if (TAG) lam[w.Mpad + rb] = (double)tb + (double)ctb;
     }
 }
 
