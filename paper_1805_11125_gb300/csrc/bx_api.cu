@@ -492,6 +492,7 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
     w.shells = 0;
     for (const Toy& T : m->toys_h) {
         w.shells |= T.n_shell > 0 ? 1 : 0;
+        w.max_sets = std::max(w.max_sets, T.n_set);
         w.multi_set |= (T.n_set > 1 || T.n_shell > 0) ? 1 : 0;
         w.nes = std::max(w.nes, T.n_es);
         w.gc |= (T.gc1 != 0.0 || T.gc2 != 0.0) ? 1 : 0;
@@ -552,6 +553,8 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.apart, m->any_cols && !species && !f64 ? 2 * sizeof(float) * cap * m->max_tiles * w.nes * w.Npad : 16},
         {(void**)&w.tile_cols, f64 ? 16 : sizeof(int2) * cap * MAX_SETS * MAX_TILES},
         {(void**)&w.cb_rows, f64 ? 16 : sizeof(int2) * cap * MAX_CB},
+        {(void**)&w.prep_part, f64 ? 16 : sizeof(int2) * PREP_ITEMS * PREP_PARTS * (MAX_SETS * MAX_TILES + 1)},
+        {(void**)&w.prep_count, sizeof(int) * PREP_ITEMS},
         {(void**)&w.qtot64, sizeof(double2) * c64 * (w.Npad / 128)},
         {(void**)&w.gen64, sizeof(Gen64) * c64 * w.Npad},
         {(void**)&w.colc64, sizeof(int4) * c64 * w.Npad},
@@ -599,6 +602,7 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         cudaError_t e = cudaMemcpyAsync((void*)w.toys, m->toys_h.data(), sizeof(Toy) * n_toys, cudaMemcpyHostToDevice,
                                         m->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(w.err, 0, sizeof(unsigned), m->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(w.prep_count, 0, sizeof(int) * PREP_ITEMS, m->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(w.units, 0, sizeof(unsigned long long), m->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync((void*)w.toy_of, 0, sizeof(int) * cap, m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);

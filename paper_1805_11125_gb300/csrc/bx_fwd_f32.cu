@@ -321,6 +321,244 @@ __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
     }
 }
 
+// Small batches: the 16 warps of an item (two 64-row halves of 8 tiles) leave most of the GPU idle, and
+// a warp's chunks are one serial chain.  Here a CTA takes one 64-row half: SG generator warps evaluate the
+// response of SG chunks at a time into shared memory (and take the column sums), and two more warps
+// (rows A, rows B) add the chunks' entries to the row sums in column order, one round behind.  The
+// entries and the order of every sum are those of k_fwd_f32: the results are the same bits.
+constexpr int SG = 4;
+// 128-row tiles of a batch (measured, us, split against plain: multivariate 52 items = 416 tiles 101 / 120,
+// 76 items = 608 tiles 134 / 121; one item 35 / 86; plain model 104 items = 416 tiles 120 / 146,
+// 152 items = 608 tiles 164 / 148)
+constexpr unsigned SPLIT_TILES = 480;
+constexpr int SRW = 33;   // row stride of an entry buffer
+struct SplitShared {
+    float R[2][SG][64][SRW];
+    float4 S[2][SG][FCH32];
+    unsigned m[2][SG][2];             // columns whose bands touch rows A, rows B
+    float4 C[SG][FCH32];
+    ColG G[SG][FCH32];
+    float P[SG][FCH32 / 2][SPW];
+    float gg[MAX_ES][64];             // Gg_s of the rows
+};
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+template <bool TAG, bool COLS, bool MES, bool GC>
+__global__ void __launch_bounds__(32 * (SG + 2)) k_fwd_split(Work w) {
+    extern __shared__ __align__(16) unsigned char split_raw[];
+    SplitShared& sh = *reinterpret_cast<SplitShared*>(split_raw);
+    const int unit = blockIdx.x >> 1, q = blockIdx.x & 1;
+    const int tile = unit % w.max_tiles, item = unit / w.max_tiles, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const Toy& T = w.toys[w.toy_of[item]];
+    if (tile >= T.n_tiles || w.status[item]) return;
+    const int M = T.M, g0 = tile * TM + 64 * q, NGRP = T.n_set > 1 ? T.n_set : 1, NES = MES ? T.n_es : 1;
+    constexpr int NT = 32 * (SG + 2);
+    for (int j = tid; COLS && j < NES * 64; j += NT) {
+        const int e = j >> 6, r = g0 + (j & 63);
+        sh.gg[e][j & 63] = r < M ? (MES ? T.Gg32[(size_t)e * M + r] : (float)T.Gg[r]) : 0.f;
+    }
+    int total = 0;   // chunks of 32 columns, set after set
+    for (int grp = 0; grp < NGRP; ++grp) {
+        const int2 cr = tile_range(w, item, grp, tile);
+        if (cr.x < cr.y) total += (cr.y - cr.x + FCH32 - 1) / FCH32;
+    }
+    const int rounds = (total + SG - 1) / SG;
+    __syncthreads();
+    const int row = g0 + lane + (wid == SG + 1 ? 32 : 0);   // (accumulator warps)
+    if (wid >= SG) {   // row sums: warp SG rows A, warp SG + 1 rows B
+        const int half = wid - SG;
+        float s = 0.f, cs = 0.f, t = 0.f, ct = 0.f;
+        for (int r = 0; r < rounds; ++r) {
+            const int b = r & 1;
+            bar_sync(1 + b, NT);
+            for (int k = 0; k < SG && r * SG + k < total; ++k) {
+                const float* R = sh.R[b][k][lane + 32 * half];
+                const float4* S = sh.S[b][k];
+                auto add = [&](int c) {
+                    const float x = R[c];
+                    const float4 v = S[c];
+                    if (TAG) {
+                        f2 acc = f2_pack(s, t), nc = f2_pack(cs, ct);
+                        kahan_fma2(acc, nc, f2_dup(x), f2_pack(v.x, v.y), f2_pack(v.z, v.w));
+                        f2_get(acc, s, t);
+                        f2_get(nc, cs, ct);
+                    } else {
+                        kahan_fma(s, cs, x, v.x, v.z);
+                    }
+                };
+                const unsigned m = sh.m[b][k][half];
+                if (m == 0xffffffffu) {
+#pragma unroll 8
+                    for (int c = 0; c < FCH32; ++c) add(c);
+                } else {
+                    for (unsigned mr = m; mr; mr &= mr - 1u) add(__ffs(mr) - 1);
+                }
+            }
+            if (r + 2 < rounds) bar_arrive(3 + b, NT);
+        }
+        if (row < M) {
+            double* lam = w.lam + (size_t)item * 2 * w.Mpad;
+            if (w.lam_pairs) {   // the Kahan sum as a normalised FP32 pair
+                float2* lp = reinterpret_cast<float2*>(lam);
+                const df ps = df_two_sum(s, cs), pt = df_two_sum(t, ct);
+                lp[row] = make_float2(ps.h, ps.l);
+                if (TAG) lp[w.Mpad + row] = make_float2(pt.h, pt.l);
+            } else {
+                lam[row] = (double)s + (double)cs;
+                if (TAG) lam[w.Mpad + row] = (double)t + (double)ct;
+            }
+        }
+        return;
+    }
+    // generators
+    const float mfa = (float)(g0 + lane), mfb = (float)(g0 + lane + 32);
+    const float gc3 = GC ? (float)T.gc1 : 0.f, gc4 = GC ? (float)T.gc2 : 0.f;
+    auto shape = [&](bool wide, float th, float tl, const ColG& cg) {
+        if constexpr (GC) return wide ? resp_shape32_gc_t<true>(th, tl, cg, gc3, gc4) : resp_shape32_gc_t<false>(th, tl, cg, gc3, gc4);
+        else return wide ? resp_shape32_t<true>(th, tl, cg) : resp_shape32_t<false>(th, tl, cg);
+    };
+    const size_t cbase = (size_t)item * w.Npad;
+    float* apart = static_cast<float*>(w.apart) + (((size_t)item * w.max_tiles + tile) * 2 + q) * (MES ? w.nes : 1) * w.Npad;
+    for (int r = 0; r < rounds; ++r) {
+        const int b = r & 1;
+        if (r >= 2) bar_sync(3 + b, NT);
+        int k = r * SG + wid;   // the warp's chunk
+        if (k < total) {
+            int c0 = 0, c1 = 0;
+            for (int grp = 0; grp < NGRP; ++grp) {
+                const int2 cr = tile_range(w, item, grp, tile);
+                const int n = cr.x < cr.y ? (cr.y - cr.x + FCH32 - 1) / FCH32 : 0;
+                if (k < n) {
+                    c0 = cr.x + k * FCH32;
+                    c1 = cr.y;
+                    break;
+                }
+                k -= n;
+            }
+            const int i = c0 + lane;
+            const bool in = i < c1;
+            const float4 cfl = in ? w.colf[cbase + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const ColG cgl = in ? w.colg[cbase + i] : ColG{0.f, 0.f, 0.f, 0.f};
+            const int2 band = in ? w.colr[cbase + i] : make_int2(0, 0);
+            sh.S[b][wid][lane] = in ? w.colS32[cbase + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            sh.C[wid][lane] = cfl;
+            sh.G[wid][lane] = cgl;
+            float* P = sh.P[wid][lane >> 1] + (lane & 1);
+            P[0] = cfl.x;
+            P[2] = cfl.y;
+            P[4] = cfl.z;
+            P[6] = cfl.w;
+            P[8] = cgl.c_lo;
+            P[10] = cgl.kap;
+            P[12] = cgl.Ck2;
+            const float t0 = fmaf((float)g0 - cfl.x, cfl.z, cfl.y), t1 = fmaf(63.0f, cfl.z, t0);
+            const float tm = fmaxf(fabsf(t0), fabsf(t1));
+            const unsigned mA = __ballot_sync(0xffffffffu, band.x < g0 + 32 && band.y > g0);
+            const unsigned mB = __ballot_sync(0xffffffffu, band.x < g0 + 64 && band.y > g0 + 32);
+            const unsigned mW = __ballot_sync(0xffffffffu, cgl.kap * tm <= 0.99f);
+            const unsigned mP = __ballot_sync(0xffffffffu, tm <= 10.9f);
+            if (lane == 0) {
+                sh.m[b][wid][0] = mA;
+                sh.m[b][wid][1] = mB;
+            }
+            __syncwarp();
+            float(*R)[SRW] = sh.R[b][wid];
+            const unsigned mAny = mA | mB, m1 = GC ? 0u : mA & mB & mW & mP, m2 = m1 & (m1 >> 1) & 0x55555555u;
+            auto pair = [&](int pr) {
+                const float4* Pv = reinterpret_cast<const float4*>(sh.P[wid][pr]);
+                const float4 v0 = Pv[0], v1 = Pv[1], v2 = Pv[2], v3 = Pv[3];
+                ColPair kp;
+                kp.x = f2_pack(v0.x, v0.y);
+                kp.y = f2_pack(v0.z, v0.w);
+                kp.z = f2_pack(v1.x, v1.y);
+                kp.w = f2_pack(v1.z, v1.w);
+                kp.cl = f2_pack(v2.x, v2.y);
+                kp.kap = f2_pack(v2.z, v2.w);
+                kp.Ck2 = f2_pack(v3.x, v3.y);
+                f2 th, tl, uh, ul, RA, RB;
+                centre_df2(f2_dup(mfa), kp, th, tl);
+                centre_step2(th, tl, kp, f2_dup(32.0f), uh, ul);
+                resp_shape32_x4(kp, th, tl, uh, ul, RA, RB);
+                f2_get(RA, R[lane][2 * pr], R[lane][2 * pr + 1]);
+                f2_get(RB, R[lane + 32][2 * pr], R[lane + 32][2 * pr + 1]);
+            };
+            if (m2 == 0x55555555u) {
+#pragma unroll 4
+                for (int pr = 0; pr < FCH32 / 2; ++pr) pair(pr);
+            } else {
+                for (unsigned mr = mAny; mr; mr &= mr - 1u) {
+                    const int c = __ffs(mr) - 1;
+                    if ((m2 >> c) & 1u) {
+                        pair(c >> 1);
+                        mr &= mr - 1u;
+                        continue;
+                    }
+                    const bool inA = (mA >> c) & 1u, inB = (mB >> c) & 1u, wide = (mW >> c) & 1u;
+                    const float4 cf = sh.C[wid][c];
+                    const ColG cg = sh.G[wid][c];
+                    float Ra = 0.f, Rb = 0.f, th, tl;
+                    if (inA) {
+                        centre_df(mfa, cf, cg.c_lo, th, tl);
+                        float uh = 0.f, ul = 0.f;
+                        if (inB) centre_step32(th, tl, cf, uh, ul);   // row B's centre from row A's
+                        Ra = shape(wide, th, tl, cg);
+                        if (inB) Rb = shape(wide, uh, ul, cg);
+                    } else {
+                        centre_df(mfb, cf, cg.c_lo, th, tl);
+                        Rb = shape(wide, th, tl, cg);
+                    }
+                    R[lane][c] = Ra;
+                    R[lane + 32][c] = Rb;
+                }
+            }
+            if (COLS) {   // column sums: lane = column, rows in order
+                __syncwarp();
+                const bool any = (mAny >> lane) & 1u;
+                if (MES) {
+                    float sm[MAX_ES];
+#pragma unroll
+                    for (int e = 0; e < MAX_ES; ++e) sm[e] = 0.f;
+                    if (any)
+#pragma unroll 4
+                        for (int j = 0; j < 64; ++j) {
+                            const float x = R[j][lane];
+#pragma unroll
+                            for (int e = 0; e < MAX_ES; ++e)
+                                if (e < NES) sm[e] = fmaf(x, sh.gg[e][j], sm[e]);
+                        }
+                    if (in)
+#pragma unroll
+                        for (int e = 0; e < MAX_ES; ++e)
+                            if (e < NES) apart[(size_t)e * w.Npad + i] = sm[e] * cgl.A;
+                } else {
+                    float sm = 0.f;
+                    if (any)
+#pragma unroll 8
+                        for (int j = 0; j < 32; ++j)
+                            sm = __fadd_rn(sm, fmaf(R[j + 32][lane], sh.gg[0][j + 32], __fmul_rn(R[j][lane], sh.gg[0][j])));
+                    if (in) apart[i] = sm * cgl.A;
+                }
+            }
+        }
+        bar_arrive(1 + b, NT);
+    }
+}
+
+template <bool TAG, bool COLS, bool MES>
+static cudaError_t fwd_split_variant(const Work& w, unsigned grid, cudaStream_t s) {
+    static size_t set[2] = {0, 0};   // opted in once per kernel
+    const int gc = w.gc ? 1 : 0;
+    const auto k = gc ? k_fwd_split<TAG, COLS, MES, true> : k_fwd_split<TAG, COLS, MES, false>;
+    if (!set[gc]) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SplitShared));
+        if (e != cudaSuccess) return e;
+        set[gc] = sizeof(SplitShared);
+    }
+    k<<<2 * grid, 32 * (SG + 2), sizeof(SplitShared), s>>>(w);
+    return cudaGetLastError();
+}
+
 template <int WPC, bool GC = false>
 static void fwd_f32_variant(const Work& w, unsigned grid, int any_tag, int any_cols, bool mes, cudaStream_t s) {
     const unsigned g = grid * (2 / WPC);
@@ -335,6 +573,15 @@ static void fwd_f32_variant(const Work& w, unsigned grid, int any_tag, int any_c
 cudaError_t launch_fwd_f32(const Work& w, int n, int max_tiles, int any_tag, int any_cols, cudaStream_t s) {
     const unsigned grid = (unsigned)n * (unsigned)w.max_tiles;   // decoded with w.max_tiles
     const bool mes = w.nes > 1;   // several energy slices of the Eq. 4 terms
+    // up to SPLIT_TILES tiles the generators of k_fwd_split find idle SMs
+    if (grid <= SPLIT_TILES) {
+        if (any_tag && any_cols && mes) return fwd_split_variant<true, true, true>(w, grid, s);
+        if (any_cols && mes) return fwd_split_variant<false, true, true>(w, grid, s);
+        if (any_tag && any_cols) return fwd_split_variant<true, true, false>(w, grid, s);
+        if (any_tag) return fwd_split_variant<true, false, false>(w, grid, s);
+        if (any_cols) return fwd_split_variant<false, true, false>(w, grid, s);
+        return fwd_split_variant<false, false, false>(w, grid, s);
+    }
     if (w.gc) fwd_f32_variant<2, true>(w, grid, any_tag, any_cols, mes, s);   // one tile shape for GC models
     else if (w.fwd_wpc == 1) fwd_f32_variant<1>(w, grid, any_tag, any_cols, mes, s);
     else fwd_f32_variant<2>(w, grid, any_tag, any_cols, mes, s);

@@ -54,6 +54,8 @@ constexpr int G64_NC = 7;       // sampled classes, spacing 2^c bins; then the b
 constexpr int G64_CI = G64_NC;
 constexpr int G64_SPLIT = 4;    // batches up to this size split the forward's tiles over more CTAs
 
+constexpr int PREP_PARTS = 8, PREP_ITEMS = 152;   // k_prep32: parts of an item, batches that use them
+
 constexpr int GPN = 5 + KMAX;   // backward partials per column block: LY, a, b, c, kB, rates
 
 enum : unsigned { ERR_TIMEOUT = 1u, ERR_TMEM = 2u };
@@ -185,6 +187,10 @@ struct Work {
     unsigned long long* units;   // in-band response entries evaluated (counted when count_units)
     int count_units;
     int shells;               // some toy has radial response shells (k_prep32's SHELL instantiations)
+    // the mixed-precision column stage in several CTAs per item (small batches; nullptr: never)
+    int2* prep_part;          // [PREP_ITEMS][PREP_PARTS][MAX_SETS * MAX_TILES + 1]: each part's tile ranges, status
+    int max_sets;             // column sets (quenching groups, radial shells) of any toy
+    int* prep_count;          // [PREP_ITEMS]: parts done (0 between evaluations)
     // FP64 model (bx_f64.cu)
     const double* tab64;      // stencils of every class and phase, then 2^(j/64)
     double2* qtot64;          // [cap][Npad/128]: Birks sums of each 128-column block

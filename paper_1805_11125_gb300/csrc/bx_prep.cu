@@ -168,11 +168,15 @@ __device__ void block_scan_df(df& a, df& b, df& ta, df& tb, float* sh) {
 // masses come from FP32 tails and go out as FP32 pairs.
 // SHELL: the sets are the radial shells of a position-dependent response (every species in every
 // set with its fraction, a light-yield factor per set) instead of quenching groups.
-template <bool MULTI, bool GC = false, bool SHELL = false>
-__global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
-    const int item = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+// PARTS (small batches): an item's chunks of 256 columns are shared by nparts CTAs.  Each repeats
+// the Birks scans of the chunks before its own (the same operations, so the same sums), and the last CTA
+// of an item to finish merges the tiles' column ranges and the status.
+template <bool MULTI, bool GC, bool SHELL, bool PARTS>
+__global__ void __launch_bounds__(256, 3) k_prep32(Work w, int np) {
+    const int nparts = PARTS ? np : 1;
+    const int item = PARTS ? blockIdx.x / nparts : blockIdx.x, part = PARTS ? blockIdx.x % nparts : 0, tid = threadIdx.x, lane = tid & 31;
     if (w.skip && w.skip[item]) {
-        if (tid == 0) w.status[item] = STATUS_SKIPPED;
+        if (tid == 0 && part == 0) w.status[item] = STATUS_SKIPPED;
         return;
     }
     const Toy& T = w.toys[w.toy_of[item]];
@@ -241,7 +245,10 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
     // species-specific quenching: one pass per group grp of species, with Birks constant
     // kB xi[grp], into the group's columns [grp Ncs, grp Ncs + N)
     const int NS = MULTI ? T.n_set : 1;
+    const int per_set = (N + 255) / 256, nchunk = NS * per_set;   // chunks, set after set
+    const int ch0 = PARTS ? part * nchunk / nparts : 0, ch1 = PARTS ? (part + 1) * nchunk / nparts : nchunk;
     for (int grp = 0; grp < NS; ++grp) {
+    if (PARTS && (grp * per_set >= ch1 || (grp + 1) * per_set <= ch0)) continue;   // none of this part's chunks
     const int off = grp * T.Ncs;
     constexpr bool shell = MULTI && SHELL;   // a radial shell: light yield LY lyf[grp]
     const df lyf = shell ? df_from(T.lyf[grp]) : df{1.f, 0.f};
@@ -249,6 +256,8 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
     const df kBc = MULTI ? df_mul(kB, xid) : kB;
     df carry_x{0.f, 0.f}, carry_y{0.f, 0.f};
     for (int c0 = 0; c0 < N; c0 += 256) {
+        const int ch = grp * per_set + c0 / 256;
+        if (PARTS && ch >= ch1) break;
         const int i = c0 + tid, ie = off + i;
         const bool in = i < N;
         df S{0.f, 0.f}, x{0.f, 0.f}, y{0.f, 0.f};
@@ -268,6 +277,11 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
         }
         df ex = x, ey = y, tx, ty;
         block_scan_df(ex, ey, tx, ty, sh);
+        if (PARTS && ch < ch0) {   // another part's chunk: its sums only
+            carry_x = df_add(carry_x, tx);
+            carry_y = df_add(carry_y, ty);
+            continue;
+        }
         int r0 = 0, r1 = 0;
         bool valid = false;
         bool live = in;
@@ -443,7 +457,7 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
     }
     }
     // padding: the columns between groups and after the last one
-    for (int i = tid; i < w.Npad; i += blockDim.x) {
+    for (int i = tid + part * 256; i < w.Npad; i += 256 * nparts) {
         const int cpad = i / T.Ncs;
         if (cpad < NS && i - cpad * T.Ncs < N) continue;
         col[i] = Col64{0.0, 1.0, 0.0, 0.0};
@@ -458,23 +472,73 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w) {
     if (bad) s_bad = 1;
     if (w.count_units && inband) atomicAdd(w.units, inband);
     __syncthreads();
-    for (int j = tid; j < NS * MAX_TILES; j += blockDim.x)
+    const int nt = NS * MAX_TILES;
+    // row ranges of the column blocks: each lies in one chunk; part 0 clears the blocks beyond the last
+    const int nblk = ((NS - 1) * T.Ncs + N + BCOLS - 1) / BCOLS;
+    for (int j = tid; j < MAX_CB; j += blockDim.x) {
+        if (!PARTS) {
+            w.cb_rows[(size_t)item * MAX_CB + j] = make_int2(s_rlo[j], s_rhi[j]);
+            continue;
+        }
+        const int set = MULTI ? min(NS - 1, j * BCOLS / T.Ncs) : 0;
+        const int ch = set * per_set + (j * BCOLS - set * T.Ncs) / 256;
+        if (j < nblk ? (ch >= ch0 && ch < ch1) : part == 0)
+            w.cb_rows[(size_t)item * MAX_CB + j] = make_int2(s_rlo[j], s_rhi[j]);
+    }
+    if (PARTS) {   // this part's ranges out; the last part of the item merges them
+        int2* mine = w.prep_part + ((size_t)item * PREP_PARTS + part) * (MAX_SETS * MAX_TILES + 1);
+        for (int j = tid; j < nt; j += blockDim.x) mine[j] = make_int2(s_tlo[j / MAX_TILES][j % MAX_TILES], s_thi[j / MAX_TILES][j % MAX_TILES]);
+        if (tid == 0) mine[MAX_SETS * MAX_TILES] = make_int2(s_bad, 0);
+        __threadfence();
+        __syncthreads();
+        __shared__ int s_last;
+        if (tid == 0) s_last = atomicAdd(&w.prep_count[item], 1) == nparts - 1;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        const int2* all = w.prep_part + (size_t)item * PREP_PARTS * (MAX_SETS * MAX_TILES + 1);
+        for (int j = tid; j < nt; j += blockDim.x) {
+            int lo = INT_MAX, hi = INT_MIN;
+            for (int q = 0; q < nparts; ++q) {
+                const int2 r = __ldcg(&all[(size_t)q * (MAX_SETS * MAX_TILES + 1) + j]);
+                lo = min(lo, r.x);
+                hi = max(hi, r.y);
+            }
+            w.tile_cols[(size_t)item * MAX_SETS * MAX_TILES + j] = make_int2(lo, hi);
+        }
+        if (tid == 0) {
+            int any = 0;
+            for (int q = 0; q < nparts; ++q) any |= __ldcg(&all[(size_t)q * (MAX_SETS * MAX_TILES + 1) + MAX_SETS * MAX_TILES]).x;
+            w.status[item] = any ? (int)BX_EDOMAIN : 0;
+            w.prep_count[item] = 0;   // for the next evaluation
+        }
+        return;
+    }
+    for (int j = tid; j < nt; j += blockDim.x)
         w.tile_cols[(size_t)item * MAX_SETS * MAX_TILES + j] = make_int2(s_tlo[j / MAX_TILES][j % MAX_TILES],
                                                                          s_thi[j / MAX_TILES][j % MAX_TILES]);
-    for (int j = tid; j < MAX_CB; j += blockDim.x)
-        w.cb_rows[(size_t)item * MAX_CB + j] = make_int2(s_rlo[j], s_rhi[j]);
     if (tid == 0) w.status[item] = s_bad ? (int)BX_EDOMAIN : 0;
 }
 
-cudaError_t launch_prep(const Work& w, int n, cudaStream_t s) {
+template <bool PARTS>
+static void prep_variant(const Work& w, unsigned grid, int np, cudaStream_t s) {
     if (w.shells) {   // radial shells of the response (their own instantiations)
-        if (w.gc) k_prep32<true, true, true><<<n, 256, 0, s>>>(w);
-        else k_prep32<true, false, true><<<n, 256, 0, s>>>(w);
+        if (w.gc) k_prep32<true, true, true, PARTS><<<grid, 256, 0, s>>>(w, np);
+        else k_prep32<true, false, true, PARTS><<<grid, 256, 0, s>>>(w, np);
     } else if (w.gc) {
-        if (w.multi_set) k_prep32<true, true><<<n, 256, 0, s>>>(w);
-        else k_prep32<false, true><<<n, 256, 0, s>>>(w);
-    } else if (w.multi_set) k_prep32<true><<<n, 256, 0, s>>>(w);
-    else k_prep32<false><<<n, 256, 0, s>>>(w);
+        if (w.multi_set) k_prep32<true, true, false, PARTS><<<grid, 256, 0, s>>>(w, np);
+        else k_prep32<false, true, false, PARTS><<<grid, 256, 0, s>>>(w, np);
+    } else if (w.multi_set) k_prep32<true, false, false, PARTS><<<grid, 256, 0, s>>>(w, np);
+    else k_prep32<false, false, false, PARTS><<<grid, 256, 0, s>>>(w, np);
+}
+
+cudaError_t launch_prep(const Work& w, int n, cudaStream_t s) {
+    // about one CTA per SM and column set: more repeat the scans without finding idle SMs (one item of
+    // one set: 52 us in one part, 25 in eight; 38 items 54 in one, 62 in eight; four sets, 52 items: 226
+    // in one, 114 in eight)
+    const int np = w.prep_part && n <= PREP_ITEMS ? max(1, min(PREP_PARTS, 152 * w.max_sets / n)) : 1;
+    if (np > 1) prep_variant<true>(w, (unsigned)n * np, np, s);
+    else prep_variant<false>(w, n, 1, s);
     return cudaGetLastError();
 }
 
