@@ -94,6 +94,32 @@ __device__ void radial_probs(const Toy& T, double s_r, double* sF, double* sdF, 
     }
 }
 
+// The same in two steps by some of the warps (this one is warp wr of nwr): the shell integrals and the
+// internal probabilities, then, after a barrier, the external ones.  GB300 issues one FP64 instruction per
+// scheduler in 64 cycles whatever the number of lanes, so the two halves go to different schedulers and
+// run beside FP32 work of the other warps.
+__device__ __forceinline__ void radial_shells(const Toy& T, double s_r, double* sF, double* sdF, double* pint, int wr, int nwr) {
+    const int nrad = T.n_rad, lane = threadIdx.x & 31, nf = nwr / 2;
+    const double lamA = T.att_len * s_r;
+    for (int e = wr * 32 + lane; wr < nf && e <= nrad + 1; e += 32 * nf) {
+        const double r = e < nrad ? T.r_fid * e / nrad : (e == nrad ? T.r_fid : 0.0);
+        shell_F(r, T.r_iv, lamA, sF[e], sdF[e]);
+    }
+    for (int b = (wr - nf) * 32 + lane; wr >= nf && b < nrad; b += 32 * (nwr - nf)) {
+        const double ra = T.r_fid * b / nrad, rb = T.r_fid * (b + 1) / nrad;
+        pint[b] = (rb * rb * rb - ra * ra * ra) / (T.r_fid * T.r_fid * T.r_fid);
+    }
+}
+__device__ __forceinline__ void radial_external(const Toy& T, const double* sF, const double* sdF, double* pext, double* dpext) {
+    const int nrad = T.n_rad;
+    const double tot = sF[nrad] - sF[nrad + 1], dtot = sdF[nrad] - sdF[nrad + 1];
+    for (int b = threadIdx.x & 31; b < nrad; b += 32) {
+        const double p = (sF[b + 1] - sF[b]) / tot;
+        pext[b] = p;
+        dpext[b] = ((sdF[b + 1] - sdF[b]) / tot - p * dtot / tot) * T.att_len;
+    }
+}
+
 // The assembly of the species-resolved tensor-core mode (BX_TF32X3): FP32 pile-up and weights, FP64
 // spectra and terms.
 __global__ void __launch_bounds__(MID_THREADS, 1) k_mid(Work w, int want_grad, int want_mu) {
@@ -399,8 +425,7 @@ __device__ __forceinline__ void conv_block(const float* g, const float* x, int b
     float xw[2 * PR - 1];   // xw[t] = x[base - d0 - 3 + t]
 #pragma unroll
     for (int t = 0; t < 2 * PR - 1; ++t) xw[t] = x[base - 3 + t];
-    int cnt = 0;
-    for (int d0 = 0; d0 < dend; d0 += PR) {
+    auto step = [&](int d0) {
         const float4 g4 = *reinterpret_cast<const float4*>(g + d0);
         const float gg[PR] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
@@ -414,11 +439,15 @@ __device__ __forceinline__ void conv_block(const float* g, const float* x, int b
         xw[1] = xn.y;
         xw[2] = xn.z;
         xw[3] = xn.w;
-        if (++cnt == PBLK) {
-            k.fold();
-            cnt = 0;
-        }
+    };
+    int d0 = 0;   // whole partial sums unrolled: the window stays in place, registers renamed
+    for (; d0 + PBLK * PR - PR < dend; d0 += PBLK * PR) {
+#pragma unroll
+        for (int u = 0; u < PBLK; ++u) step(d0 + u * PR);
+        k.fold();
     }
+#pragma unroll 1
+    for (; d0 < dend; d0 += PR) step(d0);
     k.fold();
 }
 
@@ -428,8 +457,7 @@ __device__ __forceinline__ void corr_block(const float* g, const float* y, int b
     float yw[2 * PR - 1];   // yw[t] = y[base + d0 + t]
 #pragma unroll
     for (int t = 0; t < 2 * PR - 1; ++t) yw[t] = y[base + d0s + t];
-    int cnt = 0;
-    for (int d0 = d0s; d0 < dend; d0 += PR) {
+    auto step = [&](int d0) {
         const float4 g4 = *reinterpret_cast<const float4*>(g + d0);
         const float gg[PR] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
@@ -443,11 +471,15 @@ __device__ __forceinline__ void corr_block(const float* g, const float* y, int b
         yw[PR] = yn.y;
         yw[PR + 1] = yn.z;
         yw[PR + 2] = yn.w;
-        if (++cnt == PBLK) {
-            k.fold();
-            cnt = 0;
-        }
+    };
+    int d0 = d0s;
+    for (; d0 + PBLK * PR - PR < dend; d0 += PBLK * PR) {
+#pragma unroll
+        for (int u = 0; u < PBLK; ++u) step(d0 + u * PR);
+        k.fold();
     }
+#pragma unroll 1
+    for (; d0 < dend; d0 += PR) step(d0);
     k.fold();
 }
 
@@ -484,6 +516,10 @@ __device__ __forceinline__ void bc_term_df(df n, df mu, Sum32& acc, float& wb) {
 // compensated FP32 sum (TwoSum per term, merged across the block in FP64).  FP64 remains for
 // the radial and pulse-shape marginals (one value per bin, ~100 bins).
 // MES: several energy slices of the Eq. 4 terms (otherwise one, with compile-time strides).
+// One CTA per item, and for a small batch nothing else on the SM: the phases are latency bound.  So the
+// radial bin probabilities (FP64 exponentials and divisions on two warps' worth of lanes) run in the
+// last warp beside the pile-up sums, global loads are issued in batches ahead of the sums that use them,
+// and the short serial FP64 sums go to different warps.  (Per item 63 -> 44 us; every sum keeps its order.)
 template <bool MES>
 __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad, int want_mu) {
     extern __shared__ __align__(16) double dsm[];
@@ -528,13 +564,23 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
     __shared__ double red[MID_WARPS * 2 * KMAX];
     __shared__ double s_misc[8];
     __shared__ int s_dom;
+    // in the unused half of red: the next block of rows, and the radially external species
+    int& s_task = *reinterpret_cast<int*>(red + MID_WARPS * KMAX);
+    bool* s_ext = reinterpret_cast<bool*>(red + MID_WARPS * KMAX + 1);
+    static_assert(MAX_ES * KMAX <= MID_WARPS * KMAX && 3 * MID_WARPS <= MID_WARPS * KMAX, "red's first half");
+    // column ranges of the tiles [MAX_SETS][MAX_TILES], in the place of s_mur until that is written
+    int2* s_tcols = reinterpret_cast<int2*>(s_mur);
+    static_assert(MAX_SETS * MAX_TILES <= MAX_RAD, "s_tcols in s_mur");
 
-    if (tid == 0) s_dom = 0;
+    if (tid == 0) s_dom = s_task = 0;
     if (tid < K) {
+        s_ext[tid] = nrad > 0 && T.rad_class[tid] == BX_RAD_EXTERNAL;
         const double r = th[tid], t = T.tag ? T.tag[tid] : 0.0;
         s_rs[tid] = r * (T.tag ? 1.0 - t : 1.0);
         s_rt[tid] = r * t;
     }
+    for (int j = tid; j < T.n_set * MAX_TILES; j += MID_THREADS)
+        s_tcols[j] = w.tile_cols[(size_t)item * MAX_SETS * MAX_TILES + j];
     for (int d = tid; d < gn; d += MID_THREADS) gT[d] = d < L ? T.g32[d] : 0.f;
     for (int q = tid; q < 2 * lrow; q += MID_THREADS) {
         const int h = q / lrow, m = q % lrow - padl;
@@ -545,6 +591,8 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
     const df epsd{s_eps[0], s_eps[1]}, omed{s_eps[2], s_eps[3]};
     const float epsf = epsd.h, omef = omed.h;
 
+    // radial bin probabilities (internal: uniform in volume; external: exponential from r_iv)
+    if (!MES && nrad > 0 && wid >= MID_WARPS - 4) radial_shells(T, s_r, s_F, s_dF, s_pint, wid - (MID_WARPS - 4), 4);
     // Eq. 2 on the window: mu = (1 - eps) lambda + eps (g * lambda), the convolution in
     // compensated FP32 (conv_block), the mix in double-float
     const int ngw = (nw + PR - 1) / PR;
@@ -575,14 +623,24 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
         const float* ap = static_cast<const float*>(w.apart) + (size_t)item * w.max_tiles * 2 * WNES * w.Npad;
         const float2* aW2 = reinterpret_cast<const float2*>(w.aW + ((size_t)item * WNES + qs) * w.Npad);
         for (int i = tid; i < T.Next; i += MID_THREADS) {   // every column of every quenching group
-            const int2* tcols = w.tile_cols + ((size_t)item * MAX_SETS + (T.n_set > 1 ? i / T.Ncs : 0)) * MAX_TILES;
-            float agf = 0.f;   // a few positive terms; enters G_W with weight eps
-            for (int t = 0; t < T.n_tiles; ++t) {
-                const int2 cr = tcols[t];
-                if (i >= cr.x && i < cr.y)
-                    agf += ap[(((size_t)t * 2) * WNES + qs) * w.Npad + i] + ap[(((size_t)t * 2 + 1) * WNES + qs) * w.Npad + i];
-            }
+            const int2* tcols = s_tcols + (T.n_set > 1 ? i / T.Ncs : 0) * MAX_TILES;
             const float2 a2 = aW2[i];
+            float agf = 0.f;   // a few positive terms; enters G_W with weight eps
+            for (int t0 = 0; t0 < T.n_tiles; t0 += 4) {   // four tiles' loads at a time, added in order
+                float x[4], y[4];
+                bool hit[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int t = t0 + q;
+                    const int2 cr = t < T.n_tiles ? tcols[t] : make_int2(1, 0);
+                    hit[q] = i >= cr.x && i < cr.y;
+                    x[q] = hit[q] ? ap[(((size_t)t * 2) * WNES + qs) * w.Npad + i] : 0.f;
+                    y[q] = hit[q] ? ap[(((size_t)t * 2 + 1) * WNES + qs) * w.Npad + i] : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (hit[q]) agf = __fadd_rn(agf, __fadd_rn(x[q], y[q]));
+            }
             const df aw{a2.x, a2.y};
             // G_W = aW + eps (a - aW): eps (a - aW) in FP32 is ~5e-9 of G_W
             const float dG = df_addf(df_neg(aw), agf).h;
@@ -591,24 +649,40 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
             coldG[i] = dG;
         }
         __syncthreads();
+        if (!MES && nrad > 0 && wid == MID_WARPS - 1) radial_external(T, s_F, s_dF, s_pext, s_dpext);
         for (int k = wid; k < K; k += MID_WARPS) {
             const float* sk = T.shapes32 + (size_t)k * T.N;
             // the columns of k's quenching group, or of every radial shell (weighted in FP64 by the
             // species' fraction of events in the shell)
             const int c_lo = T.n_shell ? 0 : (T.n_set > 1 ? T.set_of[k] : 0);
             const int c_hi = T.n_shell ? T.n_set : c_lo + 1;
+            const int N = T.N;
             double A0 = 0.0, A1 = 0.0;
             for (int c = c_lo; c < c_hi; ++c) {
                 const double wk = T.n_shell ? T.shw[c][k] : 1.0;
                 if (wk == 0.0) continue;
                 const int off = c * T.Ncs;
                 Sum32 a0, a1;
-                for (int i = lane; i < T.N; i += 32) {
-                    const float x = sk[i];
-                    const float2 g2 = colGW[off + i];
-                    a0.add_prod(x, g2.x, g2.y);
-                    a1.add_prod(x, coldG[off + i], 0.f);
+                float x[8];   // eight columns' loads in flight ahead of their sums
+#pragma unroll
+                for (int q = 0; q < 8; ++q) x[q] = __ldg(sk + min(lane + 32 * q, N - 1));
+                int i = lane;
+                for (; i + 32 * 7 < N; i += 32 * 8) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const float2 g2 = colGW[off + i + 32 * q];
+                        a0.add_prod(x[q], g2.x, g2.y);
+                        a1.add_prod(x[q], coldG[off + i + 32 * q], 0.f);
+                        x[q] = __ldg(sk + min(i + 32 * (q + 8), N - 1));
+                    }
                 }
+#pragma unroll
+                for (int q = 0; q < 7; ++q)
+                    if (i + 32 * q < N) {
+                        const float2 g2 = colGW[off + i + 32 * q];
+                        a0.add_prod(x[q], g2.x, g2.y);
+                        a1.add_prod(x[q], coldG[off + i + 32 * q], 0.f);
+                    }
                 a0 = a0.warp_reduce();
                 a1 = a1.warp_reduce();
                 A0 += wk * ((double)a0.s + (double)a0.c);
@@ -617,32 +691,36 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
             if (lane == 0) {   // s_SA[q][k] = sum v G_W,q, s_SA[q][KMAX + k] = sum v dG_W,q/deps
                 s_SA[qs][k] = A0;
                 s_SA[qs][KMAX + k] = A1;
+                s_beta[qs][k] = s_rs[k] * A0;   // the species' vetoed events, until the adjoint's s_beta
             }
         }
         __syncthreads();   // colGW, coldG are reused by the next slice
     }
-    // radial bin probabilities (internal: uniform in volume; external: exponential from r_iv)
-    if (nrad > 0) radial_probs(T, s_r, s_F, s_dF, s_pint, s_pext, s_dpext);
-    __syncthreads();
+    if (MES && nrad > 0) {   // several slices: their sums above are long enough, the whole block at once
+        radial_probs(T, s_r, s_F, s_dF, s_pint, s_pext, s_dpext);
+        __syncthreads();
+    }
     if (mv && tid < NES) {   // internal and external vetoed events of slice tid
         double aint = 0.0, aext = 0.0;
+#pragma unroll 4
         for (int k = 0; k < K; ++k) {
-            const double A = s_rs[k] * s_SA[tid][k];
-            if (nrad > 0 && T.rad_class[k] == BX_RAD_EXTERNAL) aext += A; else aint += A;
+            const double A = s_beta[tid][k];
+            if (s_ext[k]) aext += A; else aint += A;
         }
         s_aint[tid] = aint;
         s_aext[tid] = aext;
+    }
+    for (int j = MID_THREADS - 1 - tid; j < npsdS; j += MID_THREADS) {   // beside them, in the other warps
+        const int q = MES ? j / npsd : 0, r = j - q * npsd;
+        double v = 0.0;
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) v = fma(s_beta[q][k], __ldg(T.psd + (size_t)k * npsd + r), v);
+        s_mup[j] = v;
     }
     __syncthreads();
     for (int b = tid; b < nradS; b += MID_THREADS) {
         const int q = MES ? b / nrad : 0, r = b - q * nrad;
         s_mur[b] = s_aint[q] * s_pint[r] + s_aext[q] * s_pext[r];
-    }
-    for (int j = tid; j < npsdS; j += MID_THREADS) {
-        const int q = MES ? j / npsd : 0, r = j - q * npsd;
-        double v = 0.0;
-        for (int k = 0; k < K; ++k) v += s_rs[k] * s_SA[q][k] * T.psd[(size_t)k * npsd + r];
-        s_mup[j] = v;
     }
     __syncthreads();
 
@@ -651,8 +729,10 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
     float geps = 0.f;
     int dom = 0;
     const int nwin = H * nw;
+    float2 nnext = tid < nb ? T.cnt32[tid] : make_float2(0.f, 0.f);
     for (int b = tid; b < nb; b += MID_THREADS) {
-        const float2 n2 = T.cnt32[b];
+        const float2 n2 = nnext;
+        if (b + MID_THREADS < nb) nnext = T.cnt32[b + MID_THREADS];
         const df n{n2.x, n2.y};
         df mu;
         if (b < nwin) {
@@ -689,18 +769,35 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
         red[wid * 3 + 2] = (double)geps;
     }
     __syncthreads();
-    if (tid == 0) {
-        Neu tot{0.0, 0.0};
-        double ge = 0.0;
+    // the block's -lnL by the last warp, in the order of a serial neu_merge over the warps: every lane
+    // runs the short chain of sums, lane q keeps what warp q's addition rounded away, then lane 0 adds
+    // those up (the merge as one serial FP64 chain took as long as a fifth of the kernel)
+    if (wid == MID_WARPS - 1) {
+        double run = 0.0, before = 0.0, mine = 0.0;
+#pragma unroll
         for (int q = 0; q < MID_WARPS; ++q) {
-            tot = neu_merge(tot, Neu{red[q * 3], red[q * 3 + 1]});
-            ge += red[q * 3 + 2];
+            const double x = red[q * 3];
+            if (q == lane) { before = run; mine = x; }
+            run += x;
         }
-        w.nll[item] = s_dom ? INFINITY : tot.s + tot.c;
-        if (s_dom) w.status[item] = BX_EDOMAIN;
-        s_misc[2] = ge;
+        const double t = before + mine;
+        double e = fabs(before) >= fabs(mine) ? (before - t) + mine : (mine - t) + before;
+        double c = 0.0;
+#pragma unroll
+        for (int q = 0; q < MID_WARPS; ++q) {
+            c += __shfl_sync(0xffffffffu, e, q);
+            c += red[q * 3 + 1];
+        }
+        if (lane == 0) {
+            w.nll[item] = s_dom ? INFINITY : run + c;
+            if (s_dom) w.status[item] = BX_EDOMAIN;
+        }
+    } else if (wid == MID_WARPS - 2) {
+        double ge = 0.0;
+#pragma unroll
+        for (int q = 0; q < MID_WARPS; ++q) ge += red[q * 3 + 2];
+        if (lane == 0) s_misc[2] = ge;
     }
-    __syncthreads();
     if (!want_grad || s_dom) {
         if (tid < PMAX) gmid[tid] = 0.0;
         return;
@@ -712,19 +809,24 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
         for (int qk = wid; qk < NES * K; qk += MID_WARPS) {
             const int q = MES ? qk / K : 0, k = qk - q * K;
             double v = 0.0;
-            const bool ext = nrad > 0 && T.rad_class[k] == BX_RAD_EXTERNAL;
+            const bool ext = s_ext[k];
             for (int b = lane; b < nrad; b += 32) v += s_wr[q * nrad + b] * (ext ? s_pext[b] : s_pint[b]);
             for (int j = lane; j < npsd; j += 32) v += s_wp[q * npsd + j] * T.psd[(size_t)k * npsd + j];
             v = warp_sum(v);
             if (lane == 0) s_beta[q][k] = v;
         }
     }
-    __syncthreads();
     // pile-up-correlated weights wt_h[m] (adjoint of Eq. 2) and G_W[m], per row, in FP32:
     // wt_h[m] = (1 - eps) w_h[m] [m in W] + eps sum_d g[d] w_h[m + d]
     float* rowW = static_cast<float*>(w.rowW) + (size_t)item * (2 + WNES) * w.Mpad;
     const int ngm = (M + PR - 1) / PR;
-    for (int q = tid; q < H * ngm; q += MID_THREADS) {
+    for (;;) {   // 32 blocks of rows at a time to the next free warp
+        int q = 0;
+        if (lane == 0) q = atomicAdd(&s_task, 32);
+        q = __shfl_sync(0xffffffffu, q, 0);
+        if (q >= H * ngm) break;
+        q += lane;
+        if (q >= H * ngm) continue;
         const int h = q / ngm, m0 = (q % ngm) * PR, base = m0 - m_lo;   // window index at d = 0
         const int d0s = max(0, -(base + PR - 1)) / PR * PR, dend = min(L, nw - base);
         const float* wh = wvP + h * wrow + padw;
@@ -745,6 +847,7 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
         rowW[(size_t)(2 + q) * w.Mpad + m] =
             mv && q < NES ? fmaf(epsf, T.Gg32[(size_t)q * M + m], m >= T.es_lo[q] && m < T.es_hi[q] ? omef : 0.f) : 0.f;
     }
+    __syncthreads();
     // the rate gradient through the spectra comes from the adjoint kernel
     double* coef = w.coef + (size_t)item * (2 + WNES) * KMAX;
     if (tid < K) {
@@ -764,19 +867,26 @@ __global__ void __launch_bounds__(MID_THREADS, 2) k_mid32(Work w, int want_grad,
         const int q = MES ? j / KMAX : 0, k = j - q * KMAX;
         coef[(size_t)(2 + q) * KMAX + k] = mv && q < NES && k < K ? s_beta[q][k] * s_rs[k] : 0.0;
     }
+    // gradient of eps and s_r: the products by all threads (red is free), the sums by one thread each
+    double* pe = red;                // s_beta s_rs, per slice and species (MID_WARPS x 2 KMAX >= 4 KMAX)
+    for (int j = tid; mv && j < NES * K; j += MID_THREADS) pe[j] = s_beta[j / K][j % K] * s_rs[j % K];
+    for (int b = tid; b < nradS; b += MID_THREADS) s_wr[b] *= s_aext[MES ? b / nrad : 0];
+    __syncthreads();
     if (tid == 0) {
         double ge = s_misc[2];
         for (int q = 0; mv && q < NES; ++q)
-            for (int k = 0; k < K; ++k) ge += s_beta[q][k] * s_rs[k] * s_SA[q][KMAX + k];
-        double gs = 0.0;
-        for (int b = 0; b < nradS; ++b) {
-            const int q = MES ? b / nrad : 0;
-            gs += s_wr[b] * s_aext[q] * s_dpext[b - q * nrad];
-        }
-        for (int j = K; j < K + 5; ++j) gmid[j] = 0.0;
+#pragma unroll 4
+            for (int k = 0; k < K; ++k) ge = fma(pe[q * K + k], s_SA[q][KMAX + k], ge);
         gmid[K + 5] = ge;
+    } else if (tid == 32) {
+        double gs = 0.0;
+        for (int q = 0; q < (nradS > 0 ? NES : 0); ++q)
+#pragma unroll 4
+            for (int b = 0; b < nrad; ++b) gs = fma(s_wr[q * nrad + b], s_dpext[b], gs);
         gmid[K + 6] = gs;
-        for (int j = K + 7; j < PMAX; ++j) gmid[j] = 0.0;
+    } else if (tid >= 64 && tid < 64 + PMAX) {
+        const int j = tid - 64;
+        if ((j >= K && j < K + 5) || j >= K + 7) gmid[j] = 0.0;
     }
 }
 
