@@ -574,7 +574,6 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.nll, sizeof(double) * cap},
         {(void**)&w.mu, sizeof(double) * cap * m->nbmax},
         {(void**)&w.status, sizeof(int) * cap},
-        {(void**)&w.err, sizeof(unsigned)},
         {(void**)&w.units, sizeof(unsigned long long)},
         {(void**)&w.coef2d, m->is2d ? sizeof(float) * cap * 4 * KMAX * NSL : 16},
         {(void**)&w.tr2d, m->is2d ? sizeof(float) * cap * (w.Npad / KB) * 3 * NSL * KB : 16},
@@ -589,8 +588,7 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.geps2d, m->is2d ? sizeof(double) * cap * MAX_TILES : 16},
         {(void**)&w.gpart2d, m->is2d ? sizeof(double) * cap * MAX_CB * (GPN + 1) : 16},
         {(void**)&m->theta_d, sizeof(double) * m->cap * m->P},
-        {(void**)&m->nll_d, sizeof(double) * m->cap},
-        {(void**)&m->grad_d, sizeof(double) * m->cap * m->P},
+        {(void**)&m->res_d, sizeof(double) * (1 + (size_t)m->cap * (1 + m->P))},   // error word, -lnL, gradients
         {(void**)&m->est_theta, m->n_est > 1 ? sizeof(double) * cap * m->Pi : 16},
         {(void**)&m->est_nll, m->n_est > 1 ? sizeof(double) * cap : 16},
         {(void**)&m->est_grad, m->n_est > 1 ? sizeof(double) * cap * m->Pi : 16},
@@ -599,6 +597,16 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
     for (auto& a : plan)
         if ((st = alloc_dev(m, a.p, a.bytes))) break;
     if (!st) {
+        w.err = reinterpret_cast<unsigned*>(m->res_d);
+        m->nll_d = m->res_d + 1;
+        m->grad_d = m->nll_d + m->cap;
+        void* pin = nullptr;   // without it every host call takes the pageable copies
+        if (cudaHostAlloc(&pin, HOST_PIN_BYTES, cudaHostAllocDefault) == cudaSuccess) {
+            m->pinned.push_back(pin);
+            m->host_pin = static_cast<double*>(pin);
+        } else {
+            cudaGetLastError();
+        }
         cudaError_t e = cudaMemcpyAsync((void*)w.toys, m->toys_h.data(), sizeof(Toy) * n_toys, cudaMemcpyHostToDevice,
                                         m->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(w.err, 0, sizeof(unsigned), m->stream);
@@ -691,16 +699,21 @@ extern "C" int bx_model_n_bins(const bx_model* m, int toy) {
     return nb;
 }
 
-// Read and clear the sticky device error word (synchronises the stream).
-int bx_take_device_error(bx_model* m) {
-    unsigned err = 0;
-    CU(cudaStreamSynchronize(m->stream));
-    CU(cudaMemcpy(&err, m->w.err, sizeof err, cudaMemcpyDeviceToHost));
+// Clear the sticky device error word and report what it held.
+static int clear_device_error(bx_model* m, unsigned err) {
     if (err) {
         CU(cudaMemset(m->w.err, 0, sizeof(unsigned)));
         return bx_set_error(BX_ETIMEOUT, "a device-side wait exceeded its time budget (error word 0x%x)", err);
     }
     return BX_OK;
+}
+
+// Read and clear the sticky device error word (synchronises the stream).
+int bx_take_device_error(bx_model* m) {
+    unsigned err = 0;
+    CU(cudaStreamSynchronize(m->stream));
+    CU(cudaMemcpy(&err, m->w.err, sizeof err, cudaMemcpyDeviceToHost));
+    return clear_device_error(m, err);
 }
 
 extern "C" int bx_model_status(bx_model* m) {
@@ -852,12 +865,31 @@ static int eval_host(bx_model* m, int n, const int* toy_idx, const double* theta
             if (!std::isfinite(theta[(size_t)j * P + q]))
                 return bx_set_error(BX_EINVAL, "theta[%d][%d] is not finite", j, q);
     }
-    CU(cudaMemcpyAsync(m->theta_d, theta, sizeof(double) * n * P, cudaMemcpyHostToDevice, m->stream));
-    if ((st = bx_enqueue_eval(m, n, m->theta_d, P, want_grad, want_mu, m->nll_d, m->grad_d))) return st;
-    if (nll) CU(cudaMemcpyAsync(nll, m->nll_d, sizeof(double) * n, cudaMemcpyDeviceToHost, m->stream));
-    if (grad && want_grad)
-        CU(cudaMemcpyAsync(grad, m->grad_d, sizeof(double) * n * P, cudaMemcpyDeviceToHost, m->stream));
-    if ((st = bx_take_device_error(m))) return st;
+    // A small call is bound by its copies and synchronisations: from a pinned buffer, and with the error
+    // word, -lnL and the gradients as one block, it makes one copy each way and waits once (pageable
+    // copies wait one by one: one multivariate FP32 call 177 -> 158 us).  Larger calls go straight from and to the caller's arrays.
+    const size_t nt = (size_t)n * P, nr = 1 + n + (grad && want_grad ? nt : 0);
+    if (m->host_pin && nll && (nt + nr) * sizeof(double) <= HOST_PIN_BYTES) {
+        double *pt = m->host_pin, *pr = pt + nt;
+        std::copy(theta, theta + nt, pt);
+        CU(cudaMemcpyAsync(m->theta_d, pt, sizeof(double) * nt, cudaMemcpyHostToDevice, m->stream));
+        if ((st = bx_enqueue_eval(m, n, m->theta_d, P, want_grad, want_mu, m->nll_d, m->nll_d + n))) return st;
+        CU(cudaMemcpyAsync(pr, m->res_d, sizeof(double) * nr, cudaMemcpyDeviceToHost, m->stream));
+        CU(cudaStreamSynchronize(m->stream));
+        std::copy(pr + 1, pr + 1 + n, nll);
+        if (grad && want_grad) std::copy(pr + 1 + n, pr + nr, grad);
+        unsigned err;
+        memcpy(&err, pr, sizeof err);
+        st = clear_device_error(m, err);
+    } else {
+        CU(cudaMemcpyAsync(m->theta_d, theta, sizeof(double) * nt, cudaMemcpyHostToDevice, m->stream));
+        if ((st = bx_enqueue_eval(m, n, m->theta_d, P, want_grad, want_mu, m->nll_d, m->grad_d))) return st;
+        if (nll) CU(cudaMemcpyAsync(nll, m->nll_d, sizeof(double) * n, cudaMemcpyDeviceToHost, m->stream));
+        if (grad && want_grad)
+            CU(cudaMemcpyAsync(grad, m->grad_d, sizeof(double) * nt, cudaMemcpyDeviceToHost, m->stream));
+        st = bx_take_device_error(m);
+    }
+    if (st) return st;
     if (nll)
         for (int j = 0; j < n; ++j)
             if (std::isinf(nll[j]))

@@ -19,7 +19,10 @@ struct BxRange {
 
 struct FitState;
 
+constexpr size_t HOST_PIN_BYTES = 64 << 10;   // a model's pinned buffer: host calls up to this size
+
 struct bx_model {
+    double* host_pin = nullptr;   // theta, then the results, of a small host call
     int n_toys = 0, precision = BX_FP32, cap = 1;
     double band = 8.0;
     unsigned long long watchdog_ns = 2000000000ull;
@@ -34,6 +37,7 @@ struct bx_model {
     int ncs2d = 0;                   // class-sum rows of the 2D templates (the most over the toys)
     std::vector<int> toy_tmp, toy_cached;
     double* theta_d = nullptr;
+    double* res_d = nullptr;   // [1 + cap (1 + P)]: error word, -lnL and gradients of a host call, in one block
     double* nll_d = nullptr;
     double* grad_d = nullptr;
     FitState* fit = nullptr;
