@@ -69,7 +69,26 @@ __device__ __forceinline__ void tile_put(float* tile, int n, int c, float x) {
     tile[NSL * KB + o] = tf32_rna(x - h);
 }
 
-// D (+)= A B^T over one k-block, split products small-first.
+// The pile-up GEMMs' A tiles are Toeplitz: with the tile's rows taken in reverse (A row l is output row
+// 127 - l), entry (l, c) of k-block it depends on l + c + 32 it alone.  So the core matrices (8 rows x 4
+// columns, 128 bytes) of every tile are a window of one table, core p = elements x + 4 p + i + k: the
+// descriptor's strides are 128 bytes along K and 256 along M, overlapping, and the next k-block starts
+// 1024 bytes on.  One table (two TF32 parts) serves TP_KB k-blocks instead of a 128 x 32 tile written,
+// split and fenced for each: the generation took 2/3 of these kernels.
+constexpr int TP_KB = 20;                              // k-blocks per table: what two CTAs per SM leave
+constexpr int TP_CORES = TP_KB * (KB / 4) + 2 * (TM / 8) - 2;
+constexpr int TP_FLOATS = TP_CORES * 32;               // one part of the table
+constexpr size_t TP_SMEM = (size_t)(2 * TP_FLOATS + 2 * TILE_FLOATS) * 4 + 128;
+
+// Table of core p, element (i, k) = g[x + sgn (4 p + i + k)] (0 outside [0, L)), by the whole block.
+__device__ __forceinline__ void toeplitz_table(float* hi, float* lo, const float* g, int L, int x, int sgn) {
+    for (int q = threadIdx.x; q < TP_FLOATS; q += blockDim.x) {
+        const int d = x + sgn * (4 * (q >> 5) + ((q >> 2) & 7) + (q & 3));
+        split_store(hi, lo, q, d >= 0 && d < L ? g[d] : 0.f);
+    }
+}
+
+// D (+)= A B^T over one k-block, split products small-first; Ahi, Alo: the k-block's first core matrix.
 __device__ __forceinline__ void mma_kblock(uint32_t d, const float* Ahi, const float* Alo, const float* B,
                                            bool accumulate) {
     constexpr uint32_t idesc = umma_idesc_tf32(TM, NSL);
@@ -77,18 +96,15 @@ __device__ __forceinline__ void mma_kblock(uint32_t d, const float* Ahi, const f
     uint32_t acc = accumulate ? 1u : 0u;
 #pragma unroll
     for (int q = 0; q < KB / 8; ++q) {
-        umma_tf32(d, umma_desc(ahi + q * 2 * (TM * 16), TM * 16, 128), umma_desc(blo + q * 2 * (NSL * 16), NSL * 16, 128),
-                  idesc, acc);
+        umma_tf32(d, umma_desc(ahi + q * 256, 128, 256), umma_desc(blo + q * 2 * (NSL * 16), NSL * 16, 128), idesc, acc);
         acc = 1u;
     }
 #pragma unroll
     for (int q = 0; q < KB / 8; ++q)
-        umma_tf32(d, umma_desc(alo + q * 2 * (TM * 16), TM * 16, 128), umma_desc(bhi + q * 2 * (NSL * 16), NSL * 16, 128),
-                  idesc, 1u);
+        umma_tf32(d, umma_desc(alo + q * 256, 128, 256), umma_desc(bhi + q * 2 * (NSL * 16), NSL * 16, 128), idesc, 1u);
 #pragma unroll
     for (int q = 0; q < KB / 8; ++q)
-        umma_tf32(d, umma_desc(ahi + q * 2 * (TM * 16), TM * 16, 128), umma_desc(bhi + q * 2 * (NSL * 16), NSL * 16, 128),
-                  idesc, 1u);
+        umma_tf32(d, umma_desc(ahi + q * 256, 128, 256), umma_desc(bhi + q * 2 * (NSL * 16), NSL * 16, 128), idesc, 1u);
 }
 
 // Half a k-block (K = 16 of B's 32 rows, half `half`): the same three products as mma_kblock on
@@ -116,7 +132,7 @@ __device__ __forceinline__ void mma_half(uint32_t d, const float* Ahi, const flo
 }
 
 struct Pipe {
-    uint64_t mma_bar;
+    uint64_t mma_bar[2];
     uint64_t b_bar[2];
     uint32_t tmem;
     int abort;
@@ -751,15 +767,14 @@ __global__ void __launch_bounds__(TF + 32, 1) k_fwd2d(Work w) {
 
 // ------------------------------------------------------------------ pile-up + -lnL
 
-// Window tile t: rows m = m_lo + 128 t + r.  A[r, c] = g[m - m'] (input row m' = 32 kb + c),
-// B = Y tiles; D = sum_d g[d] Y[m - d, b].  Epilogue: mu, the Baker-Cousins terms (cancellation-
+// Window tile t: rows m = m_lo + 128 t + 127 - l.  A[l, c] = g[m - m'] (input row m' = 32 kb + c, a
+// Toeplitz table), B = Y tiles; k-block it + 1 is multiplied into the other accumulator while it is drained; D = sum_d g[d] Y[m - d, b].  Epilogue: mu, the Baker-Cousins terms (cancellation-
 // free FP32 form where mu/2 <= n <= 2 mu, double-float otherwise; compensated sums), w = 1 - n/mu.
-__global__ void __launch_bounds__(T2) k_pile2d(Work w, int want_mu) {
+__global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
     extern __shared__ unsigned char smem_raw[];
-    float* Ahi = align128(smem_raw);
-    float* Alo = Ahi + A_FLOATS;
-    float* Bt = Alo + A_FLOATS;       // [2][TILE_FLOATS]
-    float* gs = Bt + 2 * TILE_FLOATS;  // [L]
+    float* Ahi = align128(smem_raw);   // Toeplitz table of g, TP_KB k-blocks
+    float* Alo = Ahi + TP_FLOATS;
+    float* Bt = Alo + TP_FLOATS;       // [2][TILE_FLOATS]
     __shared__ Pipe pp;
     __shared__ double red[3][T2 / 32];
     const int t = blockIdx.x % w.win_tiles, item = blockIdx.x / w.win_tiles, tid = threadIdx.x;
@@ -775,68 +790,76 @@ __global__ void __launch_bounds__(T2) k_pile2d(Work w, int want_mu) {
     }
     const double* th = w.theta + (size_t)item * w.tstride;
     const double eps = th[T.K + 5];
-    const int r = tid & (TM - 1), h = tid >> 7, warp = tid >> 5;
+    const int warp = tid >> 5;
     const int mw0 = T.m_lo + t * TM;                       // first output row
     const int in_lo = max(0, mw0 - (L - 1)), in_hi = min(M, mw0 + TM);
     const int kb0 = in_lo / KB, nblk = (in_hi + KB - 1) / KB - kb0;
-    for (int d = tid; d < L; d += blockDim.x) gs[d] = T.g32[d];
     const float* yg = w.y2d + (size_t)item * w.row_kb * YTILE_FLOATS;
     float pu[NSL / 2];
 #pragma unroll
     for (int j = 0; j < NSL / 2; ++j) pu[j] = 0.f;
     if (tid == 0) {
-        mbar_init(&pp.mma_bar, 1);
+        mbar_init(&pp.mma_bar[0], 1);
+        mbar_init(&pp.mma_bar[1], 1);
         mbar_init(&pp.b_bar[0], 1);
         mbar_init(&pp.b_bar[1], 1);
         pp.abort = 0;
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(&pp.tmem, NSL);
+        tmem_alloc(&pp.tmem, 2 * NSL);   // two accumulators
         tmem_relinquish();
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tbase = pp.tmem;
     int issued = 0, waited = 0, committed = 0;
-    if (tid == 0 && nblk > 0) {
-        mbar_arrive_expect_tx(&pp.b_bar[0], TILE_BYTES);
-        bulk_g2s(Bt, yg + (size_t)kb0 * YTILE_FLOATS, TILE_BYTES, &pp.b_bar[0]);
-        issued = 1;
-    }
-    const int m = mw0 + r;
-    for (int it = 0; it < nblk; ++it) {
-        if (it > 0 && !mbar_wait(&pp.mma_bar, (it - 1) & 1, w.watchdog_ns)) atomicOr(&pp.abort, 1);
-        tc_fence_after();
-        __syncthreads();
-        if (pp.abort) break;
-        if (it > 0) drain_add(tbase, 0, pu, true);   // k-block it - 1, summed in registers
-        if (tid == 0 && it + 1 < nblk) {
-            mbar_arrive_expect_tx(&pp.b_bar[(it + 1) & 1], TILE_BYTES);
-            bulk_g2s(Bt + ((it + 1) & 1) * TILE_FLOATS, yg + (size_t)(kb0 + it + 1) * YTILE_FLOATS, TILE_BYTES,
-                     &pp.b_bar[(it + 1) & 1]);
-            ++issued;
-        }
-        const int mp0 = (kb0 + it) * KB;
-#pragma unroll
-        for (int c = 16 * h; c < 16 * h + 16; ++c) {
-            const int d = m - (mp0 + c);
-            split_store(Ahi, Alo, a_off(r, c), (m < M && d >= 0 && d < L) ? gs[d] : 0.f);
-        }
+    auto copy_b = [&](int it) {   // thread 0: k-block it's B tile into its stage
+        mbar_arrive_expect_tx(&pp.b_bar[it & 1], TILE_BYTES);
+        bulk_g2s(Bt + (it & 1) * TILE_FLOATS, yg + (size_t)(kb0 + it) * YTILE_FLOATS, TILE_BYTES, &pp.b_bar[it & 1]);
+        ++issued;
+    };
+    if (tid == 0)
+        for (int it = 0; it < min(nblk, 2); ++it) copy_b(it);
+    // the table from k-block it on: d = m - m' = mw0 + 127 - l - 32 (kb0 + it) - c
+    auto table = [&](int it) {
+        toeplitz_table(Ahi, Alo, T.g32, L, mw0 + TM - 1 - (kb0 + it) * KB, -1);
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) {
-            tc_fence_after();
-            if (!mbar_wait(&pp.b_bar[it & 1], (it >> 1) & 1, w.watchdog_ns)) {
-                atomicOr(&pp.abort, 1);
-            } else {
-                ++waited;
-                mma_kblock(tbase, Ahi, Alo, Bt + (it & 1) * TILE_FLOATS, false);
-                umma_commit(&pp.mma_bar);
-                ++committed;
-            }
+    };
+    table(0);
+    tc_fence_after();
+    const uint32_t tbase = pp.tmem;
+    auto multiply = [&](int it) {   // thread 0; accumulator it & 1 is drained
+        tc_fence_after();
+        if (!mbar_wait(&pp.b_bar[it & 1], (it >> 1) & 1, w.watchdog_ns)) {
+            atomicOr(&pp.abort, 1);
+        } else {
+            ++waited;
+            const int o = it % TP_KB * (KB / 4) * 32;
+            mma_kblock(tbase + (uint32_t)((it & 1) * NSL), Ahi + o, Alo + o, Bt + (it & 1) * TILE_FLOATS, false);
+            umma_commit(&pp.mma_bar[it & 1]);
+            ++committed;
+        }
+    };
+    if (tid == 0 && nblk > 0) multiply(0);
+    for (int it = 0; it < nblk; ++it) {
+        const bool next = it + 1 < nblk, fresh = next && (it + 1) % TP_KB == 0;   // fresh: a new table first
+        if (tid == 0 && next && !fresh && !pp.abort) multiply(it + 1);
+        __syncwarp();
+        const bool got = __all_sync(0xffffffffu, mbar_wait(&pp.mma_bar[it & 1], (it >> 1) & 1, w.watchdog_ns));
+        tc_fence_after();
+        if (!got) {
+            atomicOr(&pp.abort, 1);
+        } else {
+            if (tid == 0 && it + 2 < nblk) copy_b(it + 2);   // the stage k-block it has left
+            __syncwarp();
+            drain_add(tbase, (it & 1) * NSL, pu, true);      // summed in registers
+        }
+        tc_fence_before();
+        __syncthreads();
+        if (pp.abort) break;
+        if (fresh) {
+            table(it + 1);
+            if (tid == 0) multiply(it + 1);
         }
     }
     if (tid == 0) {
@@ -846,22 +869,24 @@ __global__ void __launch_bounds__(T2) k_pile2d(Work w, int want_mu) {
     __syncthreads();
     const int nc = pp.committed;
     bool done = true;
-    if (nc > 0) done = mbar_wait(&pp.mma_bar, (nc - 1) & 1, w.watchdog_ns > CLEANUP_NS ? w.watchdog_ns : CLEANUP_NS);
+    if (nc > 0)
+        done = mbar_wait(&pp.mma_bar[(nc - 1) & 1], ((nc - 1) >> 1) & 1,
+                         w.watchdog_ns > CLEANUP_NS ? w.watchdog_ns : CLEANUP_NS);
     tc_fence_after();
     const bool ok = !pp.abort && done && nc == nblk;
-    if (ok && nblk > 0) drain_add(tbase, 0, pu, true);
     if (!ok && tid == 0) atomicOr(w.err, ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tbase, NSL);
+    if (warp == 0) tmem_dealloc(tbase, 2 * NSL);
 
     // epilogue: row of this thread and its 64 slices; the pile-up sums go through the idle
     // operand buffers (thread-private, every copy and MMA has completed) so that the loop
     // below may index them
     float* pus = Ahi;
+    static_assert(2 * TP_FLOATS + 2 * TILE_FLOATS >= (NSL / 2) * T2, "the pile-up sums in the operand buffers");
 #pragma unroll
     for (int q = 0; q < NSL / 2; ++q) pus[q * T2 + tid] = pu[q];
-    const int row = mw0 + (warp & 3) * 32 + (tid & 31), j = row - T.m_lo;
+    const int row = mw0 + TM - 1 - ((warp & 3) * 32 + (tid & 31)), j = row - T.m_lo;
     const int b0 = (warp >> 2) * (NSL / 2);
     // Per bin in FP32 with double-float where it matters: mu = (1 - eps) Y + eps (g * Y) and
     // n - mu carry ~2^-44 relative error, the Baker-Cousins term is formed without
@@ -941,10 +966,10 @@ __global__ void __launch_bounds__(T2) k_pile2d(Work w, int want_mu) {
         nacc = neu_merge(nacc, other);
         geps += __shfl_xor_sync(0xffffffffu, geps, o);
     }
-    if ((tid & 31) == 0) {
-        red[0][warp] = nacc.s;
-        red[1][warp] = nacc.c;
-        red[2][warp] = geps;
+    if ((tid & 31) == 31) {   // the warp's first row; the warps in the order of their rows
+        red[0][warp ^ 3] = nacc.s;
+        red[1][warp ^ 3] = nacc.c;
+        red[2][warp ^ 3] = geps;
     }
     __syncthreads();
     if (tid == 0) {
@@ -962,25 +987,23 @@ __global__ void __launch_bounds__(T2) k_pile2d(Work w, int want_mu) {
 
 // ------------------------------------------------------------------ adjoint of Eq. 2
 
-// Output rows m = 128 t + r over the whole axis; A[r, c] = g[(m_lo + j) - m] with window row
-// j = 32 kb + c, B = w tiles; Wt = (1 - eps) w + eps D, stored as the adjoint's B tiles.
-__global__ void __launch_bounds__(T2) k_corr2d(Work w) {
+// Output rows m = 128 t + 127 - l over the whole axis; A[l, c] = g[(m_lo + j) - m] with window row
+// j = 32 kb + c (a Toeplitz table; the w tiles hold zeros beyond the window), B = w tiles; Wt = (1 - eps) w + eps D, stored as the adjoint's B tiles.
+__global__ void __launch_bounds__(T2, 2) k_corr2d(Work w) {
     extern __shared__ unsigned char smem_raw[];
-    float* Ahi = align128(smem_raw);
-    float* Alo = Ahi + A_FLOATS;
-    float* Bt = Alo + A_FLOATS;
-    float* gs = Bt + 2 * TILE_FLOATS;
+    float* Ahi = align128(smem_raw);   // Toeplitz table of g, TP_KB k-blocks
+    float* Alo = Ahi + TP_FLOATS;
+    float* Bt = Alo + TP_FLOATS;       // [2][TILE_FLOATS]
     __shared__ Pipe pp;
     const int t = blockIdx.x % w.max_tiles, item = blockIdx.x / w.max_tiles, tid = threadIdx.x;
     const Toy& T = w.toys[w.toy_of[item]];
     if (t >= T.n_tiles || w.status[item]) return;
     const int nw = T.nw, M = T.M, L = T.L, m_lo = T.m_lo;
     const double eps = w.theta[(size_t)item * w.tstride + T.K + 5];
-    const int r = tid & (TM - 1), h = tid >> 7, warp = tid >> 5;
+    const int warp = tid >> 5;
     const int m0 = t * TM;
     const int j_lo = max(0, m0 - m_lo), j_hi = min(nw, m0 + TM - 1 - m_lo + L);
     const int kb0 = j_lo / KB, nblk = j_hi > j_lo ? (j_hi + KB - 1) / KB - kb0 : 0;
-    for (int d = tid; d < L; d += blockDim.x) gs[d] = T.g32[d];
     const float* wg = w.w2d + (size_t)item * w.win_kb * TILE_FLOATS;
     float acc[NSL / 2];
 #pragma unroll
@@ -988,7 +1011,8 @@ __global__ void __launch_bounds__(T2) k_corr2d(Work w) {
     bool ok = true;
     if (nblk > 0) {
         if (tid == 0) {
-            mbar_init(&pp.mma_bar, 1);
+            mbar_init(&pp.mma_bar[0], 1);
+            mbar_init(&pp.mma_bar[1], 1);
             mbar_init(&pp.b_bar[0], 1);
             mbar_init(&pp.b_bar[1], 1);
             pp.abort = 0;
@@ -998,47 +1022,49 @@ __global__ void __launch_bounds__(T2) k_corr2d(Work w) {
             tmem_alloc(&pp.tmem, NSL);
             tmem_relinquish();
         }
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        const uint32_t tbase = pp.tmem;
         int issued = 0, waited = 0, committed = 0;
-        if (tid == 0) {
-            mbar_arrive_expect_tx(&pp.b_bar[0], TILE_BYTES);
-            bulk_g2s(Bt, wg + (size_t)kb0 * TILE_FLOATS, TILE_BYTES, &pp.b_bar[0]);
-            issued = 1;
-        }
-        const int m = m0 + r;
-        for (int it = 0; it < nblk; ++it) {
-            if (it > 0 && !mbar_wait(&pp.mma_bar, (it - 1) & 1, w.watchdog_ns)) atomicOr(&pp.abort, 1);
-            __syncthreads();
-            if (pp.abort) break;
-            if (tid == 0 && it + 1 < nblk) {
-                mbar_arrive_expect_tx(&pp.b_bar[(it + 1) & 1], TILE_BYTES);
-                bulk_g2s(Bt + ((it + 1) & 1) * TILE_FLOATS, wg + (size_t)(kb0 + it + 1) * TILE_FLOATS, TILE_BYTES,
-                         &pp.b_bar[(it + 1) & 1]);
-                ++issued;
-            }
-            const int j0 = (kb0 + it) * KB;
-#pragma unroll
-            for (int c = 16 * h; c < 16 * h + 16; ++c) {
-                const int d = m_lo + j0 + c - m;
-                split_store(Ahi, Alo, a_off(r, c), (j0 + c < nw && d >= 0 && d < L) ? gs[d] : 0.f);
-            }
+        auto copy_b = [&](int it) {   // thread 0: k-block it's B tile into its stage
+            mbar_arrive_expect_tx(&pp.b_bar[it & 1], TILE_BYTES);
+            bulk_g2s(Bt + (it & 1) * TILE_FLOATS, wg + (size_t)(kb0 + it) * TILE_FLOATS, TILE_BYTES, &pp.b_bar[it & 1]);
+            ++issued;
+        };
+        if (tid == 0)
+            for (int it = 0; it < min(nblk, 2); ++it) copy_b(it);
+        uint32_t tbase = 0;
+        for (int c0 = 0; c0 < nblk; c0 += TP_KB) {
+            // every MMA on the previous table has completed before it is overwritten
+            bool got = true;
+            if (c0 > 0) got = mbar_wait(&pp.mma_bar[(c0 - 1) & 1], ((c0 - 1) >> 1) & 1, w.watchdog_ns);
+            if (!got) atomicOr(&pp.abort, 1);
+            // d = m_lo + j - m = m_lo + 32 (kb0 + it) + c - m0 - 127 + l
+            if (got) toeplitz_table(Ahi, Alo, T.g32, L, m_lo + (kb0 + c0) * KB - m0 - (TM - 1), 1);
             fence_proxy_async_smem();
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
-                tc_fence_after();
-                if (!mbar_wait(&pp.b_bar[it & 1], (it >> 1) & 1, w.watchdog_ns)) {
-                    atomicOr(&pp.abort, 1);
-                } else {
+            tc_fence_after();
+            tbase = pp.tmem;
+            if (tid == 0 && !pp.abort) {
+                for (int it = c0; it < min(nblk, c0 + TP_KB); ++it) {
+                    if (!mbar_wait(&pp.b_bar[it & 1], (it >> 1) & 1, w.watchdog_ns)) {
+                        atomicOr(&pp.abort, 1);
+                        break;
+                    }
                     ++waited;
-                    mma_kblock(tbase, Ahi, Alo, Bt + (it & 1) * TILE_FLOATS, it > 0);
-                    umma_commit(&pp.mma_bar);
+                    const int o = (it - c0) * (KB / 4) * 32;
+                    mma_kblock(tbase, Ahi + o, Alo + o, Bt + (it & 1) * TILE_FLOATS, it > 0);
+                    umma_commit(&pp.mma_bar[it & 1]);
                     ++committed;
+                    if (it > 0 && it + 1 < nblk) {   // refill the stage that k-block it - 1 leaves
+                        if (!mbar_wait(&pp.mma_bar[(it - 1) & 1], ((it - 1) >> 1) & 1, w.watchdog_ns)) {
+                            atomicOr(&pp.abort, 1);
+                            break;
+                        }
+                        copy_b(it + 1);
+                    }
                 }
             }
+            __syncthreads();
+            if (pp.abort) break;
         }
         if (tid == 0) {
             if (!drain_copies(pp, waited, issued)) atomicOr(&pp.abort, 1);
@@ -1047,16 +1073,18 @@ __global__ void __launch_bounds__(T2) k_corr2d(Work w) {
         __syncthreads();
         const int nc = pp.committed;
         bool done = true;
-        if (nc > 0) done = mbar_wait(&pp.mma_bar, (nc - 1) & 1, w.watchdog_ns > CLEANUP_NS ? w.watchdog_ns : CLEANUP_NS);
+        if (nc > 0)
+            done = mbar_wait(&pp.mma_bar[(nc - 1) & 1], ((nc - 1) >> 1) & 1,
+                             w.watchdog_ns > CLEANUP_NS ? w.watchdog_ns : CLEANUP_NS);
         tc_fence_after();
-        ok = !pp.abort && done && nc == nblk;
+        ok = __all_sync(0xffffffffu, !pp.abort && done && nc == nblk);
         if (ok) drain_add(tbase, 0, acc, false);
         else if (tid == 0) atomicOr(w.err, ERR_TIMEOUT);
         tc_fence_before();
         __syncthreads();
         if (warp == 0) tmem_dealloc(tbase, NSL);
     }
-    const int row = m0 + (warp & 3) * 32 + (tid & 31), j = row - m_lo;
+    const int row = m0 + TM - 1 - ((warp & 3) * 32 + (tid & 31)), j = row - m_lo;
     const int b0 = (warp >> 2) * (NSL / 2);
     const float* wtile = (j >= 0 && j < nw) ? wg + (size_t)(j / KB) * TILE_FLOATS : nullptr;
     float* otile = w.wt2d + ((size_t)item * w.row_kb + row / KB) * TILE_FLOATS;
@@ -1379,7 +1407,6 @@ __global__ void __launch_bounds__(128) k_gather2d(Work w, int n, double* nll_out
 
 // ------------------------------------------------------------------ launchers
 
-static size_t smem_gemm(int extra_floats) { return (size_t)(2 * A_FLOATS + 2 * TILE_FLOATS + extra_floats) * 4 + 128; }
 
 template <typename F>
 static cudaError_t set_smem(F* kern, size_t bytes, size_t& cached) {
@@ -1406,13 +1433,11 @@ cudaError_t launch_eval2d(const Work& w, int n, int want_grad, int want_mu, int 
             k_fwd2d<false><<<(unsigned)n * (unsigned)w.max_tiles, TF + 32, sm, s>>>(w);
         }
     } else if (stage == 2) {
-        const size_t sm = smem_gemm(w.Lmax);
-        if ((e = set_smem(k_pile2d, sm, c_pile)) != cudaSuccess) return e;
-        k_pile2d<<<(unsigned)n * (unsigned)w.win_tiles, T2, sm, s>>>(w, want_mu);
+        if ((e = set_smem(k_pile2d, TP_SMEM, c_pile)) != cudaSuccess) return e;
+        k_pile2d<<<(unsigned)n * (unsigned)w.win_tiles, T2, TP_SMEM, s>>>(w, want_mu);
     } else if (stage == 3 && want_grad) {
-        const size_t sm = smem_gemm(w.Lmax);
-        if ((e = set_smem(k_corr2d, sm, c_corr)) != cudaSuccess) return e;
-        k_corr2d<<<(unsigned)n * (unsigned)w.max_tiles, T2, sm, s>>>(w);
+        if ((e = set_smem(k_corr2d, TP_SMEM, c_corr)) != cudaSuccess) return e;
+        k_corr2d<<<(unsigned)n * (unsigned)w.max_tiles, T2, TP_SMEM, s>>>(w);
         const size_t sb = (size_t)(6 * A_FLOATS + 2 * TILE_FLOATS + 3 * KMAX * NSL) * 4 + 128;
         if ((e = set_smem(k_bwd2d, sb, c_bwd)) != cudaSuccess) return e;
         k_bwd2d<<<(unsigned)n * (unsigned)w.max_cb, T2 + 32, sb, s>>>(w);
