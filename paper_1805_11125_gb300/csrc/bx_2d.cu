@@ -58,9 +58,10 @@ __device__ __forceinline__ void split_store(float* hi, float* lo, int off, float
     hi[off] = h;
     lo[off] = tf32_rna(x - h);
 }
+// (read-only loads: the stores of a loop over slices do not hold back the next slices' loads)
 __device__ __forceinline__ float tile_get(const float* tile, int n, int c) {
     const int o = b_off(n, c);
-    return tile[o] + tile[NSL * KB + o];
+    return __ldg(tile + o) + __ldg(tile + NSL * KB + o);
 }
 __device__ __forceinline__ void tile_put(float* tile, int n, int c, float x) {
     const float h = tf32_rna(x);
@@ -208,28 +209,27 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
         }
     }
     __syncthreads();
-    if (tid < K) {
-        const int k = tid;
+    // the normalisations: NR, dNR and NP in three warps (three FP64 pipes), eight terms' loads in flight
+    if (tid < 96 && (tid & 31) < K) {
+        const int k = tid & 31, which = tid >> 5;
         const bool ext = nR > 0 && T.rad_class[k] == BX_RAD_EXTERNAL;
-        double NR = 0.0, dNR = 0.0, NP = 0.0;
+        const double *U = T.U2 + (size_t)k * NSL + b2, *q2 = T.psd2 + (size_t)k * nP;
+        const double* pr = which == 1 ? s_dpe : ext ? s_pe : s_pi;
+        double v = 0.0;
         if (T.joint2) {   // one set, the grid; its normalisation in NR (and d/ds_r in dNR)
-            for (int r = 0; r < nR; ++r)
-                for (int j = 0; j < nP; ++j) {
-                    const double qU = T.psd2[(size_t)k * nP + j] * T.U2[(size_t)k * NSL + b2 + r * nP + j];
-                    NR += (ext ? s_pe[r] : s_pi[r]) * qU;
-                    if (ext) dNR += s_dpe[r] * qU;
-                }
+            if (which == 0 || (which == 1 && ext))
+                for (int r = 0; r < nR; ++r)
+#pragma unroll 8
+                    for (int j = 0; j < nP; ++j) v = fma(pr[r], __ldg(q2 + j) * __ldg(U + r * nP + j), v);
+        } else if (which < 2) {
+            if (which == 0 || ext)
+#pragma unroll 8
+                for (int r = 0; r < nR; ++r) v = fma(pr[r], __ldg(U + r), v);
         } else {
-            for (int r = 0; r < nR; ++r) {
-                const double U = T.U2[(size_t)k * NSL + b2 + r];
-                NR += (ext ? s_pe[r] : s_pi[r]) * U;
-                if (ext) dNR += s_dpe[r] * U;
-            }
-            for (int j = 0; j < nP; ++j) NP += T.psd2[(size_t)k * nP + j] * T.U2[(size_t)k * NSL + b2 + nR + j];
+#pragma unroll 8
+            for (int j = 0; j < nP; ++j) v = fma(__ldg(q2 + j), __ldg(U + nR + j), v);
         }
-        s_NR[k] = NR;
-        s_dNR[k] = dNR;
-        s_NP[k] = NP;
+        (which == 0 ? s_NR : which == 1 ? s_dNR : s_NP)[k] = v;
     }
     __syncthreads();
     {   // the class form of the coefficients of T_r (k_trate): alpha[set][k], q[b][class]
@@ -282,11 +282,12 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
         __syncthreads();
         const float2* alg = w.alpha2d + (size_t)item * 4 * KMAX;
         float2* W = w.wcls2d + (size_t)item * w.ncs2d * w.Npad;
-        for (int i = tid; i < T.N; i += blockDim.x) {
+        for (int i0 = tid & ~31; i0 < T.N; i0 += blockDim.x) {
+            const int i = i0 + (tid & 31);
             df sk[KMAX];
 #pragma unroll
             for (int k = 0; k < KMAX; ++k)
-                sk[k] = k < K ? df{T.shapes32[(size_t)k * T.N + i], T.shapes32l[(size_t)k * T.N + i]} : df{0.f, 0.f};
+                sk[k] = k < K && i < T.N ? df{T.shapes32[(size_t)k * T.N + i], T.shapes32l[(size_t)k * T.N + i]} : df{0.f, 0.f};
             for (int ss = 0; ss < 4; ++ss)
                 for (int c = 0; c < T.n_cls[ss]; ++c) {
                     df acc{0.f, 0.f};
@@ -296,8 +297,10 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
                             const float2 a = alg[ss * KMAX + k];
                             acc = df_add(acc, df_mul(df{a.x, a.y}, sk[k]));
                         }
-                    W[(size_t)(s_off[ss] + c) * w.Npad + i] = make_float2(acc.h, acc.l);
-                    atomicMax(&s_wmax[s_off[ss] + c], __float_as_uint(fabsf(acc.h)));
+                    if (i < T.N) W[(size_t)(s_off[ss] + c) * w.Npad + i] = make_float2(acc.h, acc.l);
+                    // one atomic a warp: 32 to one address take turns
+                    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(acc.h)));
+                    if ((tid & 31) == 0) atomicMax(&s_wmax[s_off[ss] + c], top);
                 }
         }
         __syncthreads();
@@ -900,14 +903,16 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
     const bool live = ok && row < M;   // j < nw
     float* wtile = (j / KB < w.win_kb) ? w.w2d + ((size_t)item * w.win_kb + j / KB) * TILE_FLOATS : nullptr;
     const float* ytile = yg + (size_t)(row / KB) * YTILE_FLOATS;
+    const float2* cnt = T.cnt32;
+    const int n_sl = T.n_sl;
 #pragma unroll 4
     for (int q = 0; q < NSL / 2; ++q) {
         const int b = b0 + q;
         float wb = 0.f;
-        if (live && b < T.n_sl) {
+        if (live && b < n_sl) {
             const int o = b_off(b, row % KB);
             // Y = yh + yl (the pair the GEMM used) + the FP32 remainder, as a double-float
-            const float yh = ytile[o], yl = __fadd_rn(ytile[NSL * KB + o], ytile[2 * NSL * KB + o]);
+            const float yh = __ldg(ytile + o), yl = __fadd_rn(__ldg(ytile + NSL * KB + o), __ldg(ytile + 2 * NSL * KB + o));
             const float pq = pus[q * T2 + tid];
             // mu as a double-float
             float p1 = __fmul_rn(c1h, yh), e1 = fmaf(c1h, yh, -p1);
@@ -918,7 +923,7 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
             float sl = __fadd_rn(__fsub_rn(p1, __fsub_rn(sh, bb)), __fsub_rn(p2, bb));
             sl = __fadd_rn(sl, __fadd_rn(e1, e2));
             const float muh = __fadd_rn(sh, sl), mul = __fsub_rn(sl, __fsub_rn(muh, sh));
-            const float2 n = T.cnt32[(size_t)b * nw + j];
+            const float2 n = __ldg(cnt + (size_t)b * nw + j);
             float term, wf = 1.f;
             if (n.x == 0.f) {
                 term = muh;
