@@ -36,7 +36,9 @@
 
 namespace bx {
 
-constexpr int T2 = 256;                            // threads of the 2D GEMM kernels
+constexpr int T2 = 256;                            // threads of the adjoint GEMM that generate its operand
+constexpr int TP = 512;                            // threads of the pile-up GEMMs
+constexpr int PS = NSL * TM / TP;                  // slices of one row that a thread drains and finishes
 constexpr int TILE_FLOATS = 2 * NSL * KB;          // one B tile (hi | lo), 32 KB
 constexpr uint32_t TILE_BYTES = TILE_FLOATS * 4;
 // a Y tile: the B tile (hi | lo) of the pile-up GEMM, then the FP32 remainder y - hi - lo (exact),
@@ -163,14 +165,14 @@ __device__ __forceinline__ float trunc_comp(float d) {
     return __int_as_float(__float_as_int(d) & 0xFF800000) * (1.25f * 1.1920928955078125e-7f);
 }
 
-// Read this thread's 64 accumulator columns (warp q: TMEM lanes 32 (q % 4) + lane, columns
-// 64 (q / 4) .. + 63) and add them into acc; with `comp` each value is corrected by its
+// Read this thread's PS accumulator columns (warp q: TMEM lanes 32 (q % 4) + lane, columns
+// PS (q / 4) .. + PS - 1) and add them into acc; with `comp` each value is corrected by its
 // expected truncation (one k-block accumulated from zero).
-__device__ __forceinline__ void drain_add(uint32_t tbase, int col0, float (&acc)[NSL / 2], bool comp) {
+__device__ __forceinline__ void drain_add(uint32_t tbase, int col0, float (&acc)[PS], bool comp) {
     const int warp = threadIdx.x >> 5;
-    const uint32_t base = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(col0 + (warp >> 2) * (NSL / 2));
+    const uint32_t base = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(col0 + (warp >> 2) * PS);
 #pragma unroll
-    for (int j = 0; j < NSL / 2; j += 8) {
+    for (int j = 0; j < PS; j += 8) {
         float v[8];
         tmem_ld8(base + (uint32_t)j, v);
 #pragma unroll
@@ -184,28 +186,29 @@ __device__ __forceinline__ void drain_add(uint32_t tbase, int col0, float (&acc)
 //   b = 0 vetoed: 1 - t_k;  b = 1 tagged: t_k;  radial rho: (1 - t_k) p_k[rho](s_r) / N^R_k(s_r);
 //   pulse shape j: (1 - t_k) q_k[j] / N^P_k, with N_k = sum_{b in the set} q_k[b] U2[k][b];
 //   joint grid (rho, j): (1 - t_k) p_k[rho](s_r) q_k[j] / N_k(s_r), one set (the grid).
-__global__ void __launch_bounds__(512) k_coef2d(Work w) {
-    const int item = blockIdx.x, tid = threadIdx.x;
+// A small batch leaves most SMs idle: np CTAs share an item (launch_eval2d), each with the item's short
+// FP64 part (the same bits in all of them) and its share of the columns and of the coefficients.
+__global__ void __launch_bounds__(512) k_coef2d(Work w, int np) {
+    const int item = blockIdx.x / np, part = blockIdx.x % np, tid = threadIdx.x;
     if (w.status[item]) return;
     const Toy& T = w.toys[w.toy_of[item]];
     const int K = T.K, nR = T.n_r2, nP = T.n_p2, b2 = T.b_r2;
     const double* th = w.theta + (size_t)item * w.tstride;
     __shared__ double s_pi[NSL], s_pe[NSL], s_dpe[NSL], s_NR[KMAX], s_dNR[KMAX], s_NP[KMAX];
+    __shared__ double s_F[NSL + 2], s_dF[NSL + 2];   // n_r2 < NSL
     if (nR > 0) {
         const double lamA = T.att_len * th[K + 6];
-        double Ft, dFt, F0, dF0;
-        shell_F(T.r_fid, T.r_iv, lamA, Ft, dFt);
-        shell_F(0.0, T.r_iv, lamA, F0, dF0);
-        const double tot = Ft - F0, dtot = dFt - dF0;
+        // the shell integrals at the bin edges and at r_fid, one a thread
+        for (int e = tid; e <= nR + 1; e += blockDim.x)
+            shell_F(e <= nR ? T.r_fid * e / nR : T.r_fid, T.r_iv, lamA, s_F[e], s_dF[e]);
+        __syncthreads();
+        const double tot = s_F[nR + 1] - s_F[0], dtot = s_dF[nR + 1] - s_dF[0];
         for (int b = tid; b < nR; b += blockDim.x) {
             const double ra = T.r_fid * b / nR, rb = T.r_fid * (b + 1) / nR;
             s_pi[b] = (rb * rb * rb - ra * ra * ra) / (T.r_fid * T.r_fid * T.r_fid);
-            double Fa, dFa, Fb, dFb;
-            shell_F(ra, T.r_iv, lamA, Fa, dFa);
-            shell_F(rb, T.r_iv, lamA, Fb, dFb);
-            const double p = (Fb - Fa) / tot;
+            const double p = (s_F[b + 1] - s_F[b]) / tot;
             s_pe[b] = p;
-            s_dpe[b] = ((dFb - dFa) / tot - p * dtot / tot) * T.att_len;
+            s_dpe[b] = ((s_dF[b + 1] - s_dF[b]) / tot - p * dtot / tot) * T.att_len;
         }
     }
     __syncthreads();
@@ -269,6 +272,7 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
     {   // the class sums W[set, c][i] of every column, their largest values, and from those an upper
         // bound of each slice's T_r: utmax[b] sum_c q[b][c] max_i W[set(b), c][i]
         __shared__ unsigned s_wmax[4 * KMAX];
+        __shared__ bool s_last;
         __shared__ int s_off[5];
         if (tid == 0) {
             int o = 0;
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
         __syncthreads();
         const float2* alg = w.alpha2d + (size_t)item * 4 * KMAX;
         float2* W = w.wcls2d + (size_t)item * w.ncs2d * w.Npad;
-        for (int i0 = tid & ~31; i0 < T.N; i0 += blockDim.x) {
+        for (int i0 = (tid & ~31) + part * blockDim.x; i0 < T.N; i0 += np * blockDim.x) {
             const int i = i0 + (tid & 31);
             df sk[KMAX];
 #pragma unroll
@@ -304,8 +308,25 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
                 }
         }
         __syncthreads();
+        bool last = true;   // the CTA that finishes the item: it has every part's largest values
+        if (np > 1) {
+            int2* all = w.prep_part + (size_t)item * PREP_PARTS * (MAX_SETS * MAX_TILES + 1);
+            if (tid < 4 * KMAX) all[part * 4 * KMAX + tid].x = (int)s_wmax[tid];
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_last = atomicAdd(&w.prep_count[item], 1) == np - 1;
+            __syncthreads();
+            last = s_last;
+            if (last) {
+                __threadfence();
+                if (tid < 4 * KMAX)
+                    for (int q = 0; q < np; ++q) s_wmax[tid] = max(s_wmax[tid], (unsigned)__ldcg(&all[q * 4 * KMAX + tid]).x);
+                if (tid == 0) w.prep_count[item] = 0;
+                __syncthreads();
+            }
+        }
         const float2* qc = w.qcls2d + (size_t)item * NSL * KMAX;
-        for (int b = tid; b < NSL; b += blockDim.x) {
+        for (int b = tid; last && b < NSL; b += blockDim.x) {
             const int ss = b == 0 ? 0 : (T.has_tag && b == 1) ? 1 : (T.joint2 || b < b2 + nR) ? 2 : 3;
             double bound = 0.0;
             if (b < T.n_sl)
@@ -318,7 +339,7 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w) {
         }
     }
     float* out = w.coef2d + (size_t)item * 4 * KMAX * NSL;
-    for (int idx = tid; idx < KMAX * NSL; idx += blockDim.x) {
+    for (int idx = tid + part * blockDim.x; idx < KMAX * NSL; idx += np * blockDim.x) {
         const int k = idx / NSL, b = idx % NSL;
         double c = 0.0, dc = 0.0, r = 0.0;
         if (k < K) {
@@ -773,13 +794,13 @@ __global__ void __launch_bounds__(TF + 32, 1) k_fwd2d(Work w) {
 // Window tile t: rows m = m_lo + 128 t + 127 - l.  A[l, c] = g[m - m'] (input row m' = 32 kb + c, a
 // Toeplitz table), B = Y tiles; k-block it + 1 is multiplied into the other accumulator while it is drained; D = sum_d g[d] Y[m - d, b].  Epilogue: mu, the Baker-Cousins terms (cancellation-
 // free FP32 form where mu/2 <= n <= 2 mu, double-float otherwise; compensated sums), w = 1 - n/mu.
-__global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
+__global__ void __launch_bounds__(TP, 2) k_pile2d(Work w, int want_mu) {
     extern __shared__ unsigned char smem_raw[];
     float* Ahi = align128(smem_raw);   // Toeplitz table of g, TP_KB k-blocks
     float* Alo = Ahi + TP_FLOATS;
     float* Bt = Alo + TP_FLOATS;       // [2][TILE_FLOATS]
     __shared__ Pipe pp;
-    __shared__ double red[3][T2 / 32];
+    __shared__ double red[3][TP / 32];
     const int t = blockIdx.x % w.win_tiles, item = blockIdx.x / w.win_tiles, tid = threadIdx.x;
     const Toy& T = w.toys[w.toy_of[item]];
     const int nw = T.nw, M = T.M, L = T.L;
@@ -798,9 +819,9 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
     const int in_lo = max(0, mw0 - (L - 1)), in_hi = min(M, mw0 + TM);
     const int kb0 = in_lo / KB, nblk = (in_hi + KB - 1) / KB - kb0;
     const float* yg = w.y2d + (size_t)item * w.row_kb * YTILE_FLOATS;
-    float pu[NSL / 2];
+    float pu[PS];
 #pragma unroll
-    for (int j = 0; j < NSL / 2; ++j) pu[j] = 0.f;
+    for (int j = 0; j < PS; ++j) pu[j] = 0.f;
     if (tid == 0) {
         mbar_init(&pp.mma_bar[0], 1);
         mbar_init(&pp.mma_bar[1], 1);
@@ -886,11 +907,11 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
     // operand buffers (thread-private, every copy and MMA has completed) so that the loop
     // below may index them
     float* pus = Ahi;
-    static_assert(2 * TP_FLOATS + 2 * TILE_FLOATS >= (NSL / 2) * T2, "the pile-up sums in the operand buffers");
+    static_assert(2 * TP_FLOATS + 2 * TILE_FLOATS >= PS * TP, "the pile-up sums in the operand buffers");
 #pragma unroll
-    for (int q = 0; q < NSL / 2; ++q) pus[q * T2 + tid] = pu[q];
+    for (int q = 0; q < PS; ++q) pus[q * TP + tid] = pu[q];
     const int row = mw0 + TM - 1 - ((warp & 3) * 32 + (tid & 31)), j = row - T.m_lo;
-    const int b0 = (warp >> 2) * (NSL / 2);
+    const int b0 = (warp >> 2) * (PS);
     // Per bin in FP32 with double-float where it matters: mu = (1 - eps) Y + eps (g * Y) and
     // n - mu carry ~2^-44 relative error, the Baker-Cousins term is formed without
     // cancellation (log1p_minus_x32 where mu/2 <= n <= 2 mu, bc_term_far in double-float
@@ -906,14 +927,14 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
     const float2* cnt = T.cnt32;
     const int n_sl = T.n_sl;
 #pragma unroll 4
-    for (int q = 0; q < NSL / 2; ++q) {
+    for (int q = 0; q < PS; ++q) {
         const int b = b0 + q;
         float wb = 0.f;
         if (live && b < n_sl) {
             const int o = b_off(b, row % KB);
             // Y = yh + yl (the pair the GEMM used) + the FP32 remainder, as a double-float
             const float yh = __ldg(ytile + o), yl = __fadd_rn(__ldg(ytile + NSL * KB + o), __ldg(ytile + 2 * NSL * KB + o));
-            const float pq = pus[q * T2 + tid];
+            const float pq = pus[q * TP + tid];
             // mu as a double-float
             float p1 = __fmul_rn(c1h, yh), e1 = fmaf(c1h, yh, -p1);
             e1 = fmaf(c1h, yl, fmaf(c1l, yh, e1));
@@ -980,7 +1001,7 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
     if (tid == 0) {
         Neu tot{0.0, 0.0};
         double ge = 0.0;
-        for (int q = 0; q < T2 / 32; ++q) {
+        for (int q = 0; q < TP / 32; ++q) {
             tot = neu_merge(tot, Neu{red[0][q], red[1][q]});
             ge += red[2][q];
         }
@@ -994,7 +1015,7 @@ __global__ void __launch_bounds__(T2, 2) k_pile2d(Work w, int want_mu) {
 
 // Output rows m = 128 t + 127 - l over the whole axis; A[l, c] = g[(m_lo + j) - m] with window row
 // j = 32 kb + c (a Toeplitz table; the w tiles hold zeros beyond the window), B = w tiles; Wt = (1 - eps) w + eps D, stored as the adjoint's B tiles.
-__global__ void __launch_bounds__(T2, 2) k_corr2d(Work w) {
+__global__ void __launch_bounds__(TP, 2) k_corr2d(Work w) {
     extern __shared__ unsigned char smem_raw[];
     float* Ahi = align128(smem_raw);   // Toeplitz table of g, TP_KB k-blocks
     float* Alo = Ahi + TP_FLOATS;
@@ -1010,9 +1031,9 @@ __global__ void __launch_bounds__(T2, 2) k_corr2d(Work w) {
     const int j_lo = max(0, m0 - m_lo), j_hi = min(nw, m0 + TM - 1 - m_lo + L);
     const int kb0 = j_lo / KB, nblk = j_hi > j_lo ? (j_hi + KB - 1) / KB - kb0 : 0;
     const float* wg = w.w2d + (size_t)item * w.win_kb * TILE_FLOATS;
-    float acc[NSL / 2];
+    float acc[PS];
 #pragma unroll
-    for (int q = 0; q < NSL / 2; ++q) acc[q] = 0.f;
+    for (int q = 0; q < PS; ++q) acc[q] = 0.f;
     bool ok = true;
     if (nblk > 0) {
         if (tid == 0) {
@@ -1090,12 +1111,12 @@ __global__ void __launch_bounds__(T2, 2) k_corr2d(Work w) {
         if (warp == 0) tmem_dealloc(tbase, NSL);
     }
     const int row = m0 + TM - 1 - ((warp & 3) * 32 + (tid & 31)), j = row - m_lo;
-    const int b0 = (warp >> 2) * (NSL / 2);
+    const int b0 = (warp >> 2) * (PS);
     const float* wtile = (j >= 0 && j < nw) ? wg + (size_t)(j / KB) * TILE_FLOATS : nullptr;
     float* otile = w.wt2d + ((size_t)item * w.row_kb + row / KB) * TILE_FLOATS;
     const float e = (float)eps, ome = (float)(1.0 - eps);
 #pragma unroll
-    for (int q = 0; q < NSL / 2; ++q) {
+    for (int q = 0; q < PS; ++q) {
         const int b = b0 + q;
         float v = 0.f;
         if (ok && row < M && b < T.n_sl) {
@@ -1426,7 +1447,9 @@ cudaError_t launch_eval2d(const Work& w, int n, int want_grad, int want_mu, int 
     static size_t c_fwd = 0, c_fwd_bf = 0, c_pile = 0, c_corr = 0, c_bwd = 0;
     cudaError_t e = cudaSuccess;
     if (stage == 1) {
-        k_coef2d<<<n, 512, 0, s>>>(w);
+        // the forward stage of one item: 174 us with one CTA here, 129 with eight
+        const int np = w.prep_part && n <= PREP_ITEMS ? max(1, min(PREP_PARTS, 152 / n)) : 1;
+        k_coef2d<<<n * np, 512, 0, s>>>(w, np);
         const size_t sm = (size_t)(6 * A_FLOATS + 2 * TILE3_FLOATS) * 4 + 128;
         if (w.precision == BX_BF16X3) {
             k_trate<true><<<(unsigned)n * (unsigned)w.tr_kb, NSL * TRS<true>, 0, s>>>(w);
@@ -1439,10 +1462,10 @@ cudaError_t launch_eval2d(const Work& w, int n, int want_grad, int want_mu, int 
         }
     } else if (stage == 2) {
         if ((e = set_smem(k_pile2d, TP_SMEM, c_pile)) != cudaSuccess) return e;
-        k_pile2d<<<(unsigned)n * (unsigned)w.win_tiles, T2, TP_SMEM, s>>>(w, want_mu);
+        k_pile2d<<<(unsigned)n * (unsigned)w.win_tiles, TP, TP_SMEM, s>>>(w, want_mu);
     } else if (stage == 3 && want_grad) {
         if ((e = set_smem(k_corr2d, TP_SMEM, c_corr)) != cudaSuccess) return e;
-        k_corr2d<<<(unsigned)n * (unsigned)w.max_tiles, T2, TP_SMEM, s>>>(w);
+        k_corr2d<<<(unsigned)n * (unsigned)w.max_tiles, TP, TP_SMEM, s>>>(w);
         const size_t sb = (size_t)(6 * A_FLOATS + 2 * TILE_FLOATS + 3 * KMAX * NSL) * 4 + 128;
         if ((e = set_smem(k_bwd2d, sb, c_bwd)) != cudaSuccess) return e;
         k_bwd2d<<<(unsigned)n * (unsigned)w.max_cb, T2 + 32, sb, s>>>(w);
