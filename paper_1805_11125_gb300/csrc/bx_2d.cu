@@ -15,8 +15,8 @@
 //
 // Every GEMM is M = 128 (output rows, or true-energy columns in the adjoint) x N = NSL x
 // K = 32 per k-block.  The A tile is generated by the CUDA cores into shared memory (the
-// response by the bias-free FP32 generator of bx_resp.cuh, or the pile-up kernel g), the
-// B tile arrives by a bulk copy from a tile written by the previous stage.  The forward
+// response by the bias-free FP32 generator of bx_resp.cuh) or is a window of a table of the
+// pile-up kernel g (toeplitz_table), the B tile arrives by a bulk copy from a tile written by the previous stage.  The forward
 // splits both operands in three (split3: an 8-bit hi on a grid shared by the k-block's
 // row or slice, then TF32 mid and lo), which makes the hi*hi products exact in the FP32
 // accumulator; the other GEMMs split into TF32 hi and lo, and one thread issues hi*lo,

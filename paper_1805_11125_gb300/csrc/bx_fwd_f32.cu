@@ -7,6 +7,11 @@
 // and, for models with Eq. 4 terms, the response is also reduced over rows,
 //     a_t[i] = sum_{m in tile t} R[m,i] Gg[m],
 // from which k_mid forms every species' window marginal after pile-up.
+// Two kernels with the same sums in the same order: k_fwd_f32 for large batches (below) and k_fwd_split
+// for up to SPLIT_TILES tiles, where generator warps evaluate chunks of columns side by side for an
+// accumulator warp.  Both evaluate a pair of columns x a pair of rows a thread in packed FP32
+// arithmetic (two lane operations per issue slot: the forward was bound by issue, not by the FMA rate)
+// wherever |z| <= 1 holds for both columns, and entry by entry elsewhere.
 // Unit = (row tile of TM output bins, item); 64 threads, warp q owning the two 32-row
 // groups m0 + 64q + [0, 32) and m0 + 64q + [32, 64), one row of each per thread.  The warps
 // never wait for each other: each stages 32 columns' parameters at a time in its own shared

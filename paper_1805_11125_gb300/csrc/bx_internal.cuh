@@ -1,14 +1,15 @@
 // bx_internal.cuh -- device-side data layout and PTX helpers of the binned -lnL engine.
 //
 // One evaluation (an "item" = one toy at one parameter point) runs as
-//   k_prep   per-column FP64 quantities of Eq. 1 (Birks map, mean, width, normalisation),
+// (in FP32 modes; the FP64 model has its own kernels in bx_f64.cu)
+//   k_prep32 per-column quantities of Eq. 1 (Birks map, mean, width, normalisation),
 //            the rate-weighted shapes S_h[i] = sum_k r_k c_{h,k} s_k[i] of the Eq. 3
 //            spectra, the window mass of every column, band limits, FP32 column parameters;
 //   k_fwd_*  response generated on the fly (Eq. 1) and reduced both ways: row sums
 //            lambda_h[m] = sum_i R[m,i] S_h[i] and, for the Eq. 4 terms, column sums
 //            a[i] = sum_m R[m,i] Gg[m] (the tensor-core variant instead contracts with every
 //            species shape, v[m][k] = sum_i R[m,i] s_k[i]);
-//   k_mid    Eq. 2 pile-up, Eq. 4 marginals, -lnL (FP64, compensated), adjoint row weights;
+//   k_mid*   Eq. 2 pile-up, Eq. 4 marginals, -lnL (compensated sums), adjoint row weights;
 //   k_bwd_*  adjoint of Eq. 1 per true-energy column: response parameters through the
 //            chain rule to LY, a, b, c, kB, and the rates through sum_m R[m,i] wt_h[m];
 //   k_gather final -lnL and gradient per item.
