@@ -45,6 +45,7 @@ __device__ __forceinline__ float shape_w(const Toy& T, int k, int ig, float wk) 
 // row recurrence of the Gaussian does not carry the polynomial factor.
 template <bool MULTI, bool MES, bool GC = false>
 __global__ void __launch_bounds__(BCOLS, 7) k_bwd_f32(Work w) {
+    chain_wait();
     // 1D item-major grid (a y dimension would cap the batch at 65535 items)
     const int cb = blockIdx.x % w.max_cb, item = blockIdx.x / w.max_cb, tid = threadIdx.x;
     const Toy& T = w.toys[w.toy_of[item]];
@@ -295,14 +296,14 @@ cudaError_t launch_bwd(const Work& w, int n, int max_cb, cudaStream_t s) {
     const unsigned grid = (unsigned)n * (unsigned)w.max_cb;   // decoded with w.max_cb
     const bool mes = w.nes > 1;   // several energy slices of the Eq. 4 terms
     if (w.gc) {   // the Gram-Charlier response (one quenching group)
-        if (w.multi_set && mes) k_bwd_f32<true, true, true><<<grid, BCOLS, 0, s>>>(w);
-        else if (w.multi_set) k_bwd_f32<true, false, true><<<grid, BCOLS, 0, s>>>(w);
-        else if (mes) k_bwd_f32<false, true, true><<<grid, BCOLS, 0, s>>>(w);
-        else k_bwd_f32<false, false, true><<<grid, BCOLS, 0, s>>>(w);
-    } else if (w.multi_set && mes) k_bwd_f32<true, true><<<grid, BCOLS, 0, s>>>(w);
-    else if (w.multi_set) k_bwd_f32<true, false><<<grid, BCOLS, 0, s>>>(w);
-    else if (mes) k_bwd_f32<false, true><<<grid, BCOLS, 0, s>>>(w);
-    else k_bwd_f32<false, false><<<grid, BCOLS, 0, s>>>(w);
+        if (w.multi_set && mes) launch_chained(k_bwd_f32<true, true, true>, grid, BCOLS, 0, s, w);
+        else if (w.multi_set) launch_chained(k_bwd_f32<true, false, true>, grid, BCOLS, 0, s, w);
+        else if (mes) launch_chained(k_bwd_f32<false, true, true>, grid, BCOLS, 0, s, w);
+        else launch_chained(k_bwd_f32<false, false, true>, grid, BCOLS, 0, s, w);
+    } else if (w.multi_set && mes) launch_chained(k_bwd_f32<true, true>, grid, BCOLS, 0, s, w);
+    else if (w.multi_set) launch_chained(k_bwd_f32<true, false>, grid, BCOLS, 0, s, w);
+    else if (mes) launch_chained(k_bwd_f32<false, true>, grid, BCOLS, 0, s, w);
+    else launch_chained(k_bwd_f32<false, false>, grid, BCOLS, 0, s, w);
     return cudaGetLastError();
 }
 
@@ -313,6 +314,7 @@ cudaError_t launch_bwd(const Work& w, int n, int max_cb, cudaStream_t s) {
 // 35 us for 52).  The sum over column blocks keeps its order.
 static_assert(PMAX <= 32, "one lane per parameter");
 __global__ void __launch_bounds__(128) k_gather(Work w, int n, double* nll_out, double* grad_out, int want_grad) {
+    chain_wait();
     const int item = blockIdx.x * 4 + (threadIdx.x >> 5), j = threadIdx.x & 31;
     if (item >= n) return;
     const Toy& T = w.toys[w.toy_of[item]];
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(128) k_gather(Work w, int n, double* nll_out, 
 }
 
 cudaError_t launch_gather(const Work& w, int n, double* nll_out, double* grad_out, int want_grad, cudaStream_t s) {
-    k_gather<<<(n + 3) / 4, 128, 0, s>>>(w, n, nll_out, grad_out, want_grad);
+    launch_chained(k_gather, (n + 3) / 4, 128, 0, s, w, n, nll_out, grad_out, want_grad);
     return cudaGetLastError();
 }
 

@@ -62,6 +62,7 @@ __device__ __forceinline__ void kahan_fma2(f2& acc, f2& nc, f2 a, f2 b, f2 bl) {
 // GC: the Gram-Charlier response (resp_shape32_gc, the toy's skewness and kurtosis terms).
 template <bool TAG, bool COLS, bool MES, int WPC = 2, bool GC = false>
 __global__ void __launch_bounds__(32 * WPC) k_fwd_f32(Work w) {
+    chain_wait();
     // 1D item-major grid (a y dimension would cap the batch at 65535 items)
     const int unit = WPC == 2 ? (int)blockIdx.x : (int)(blockIdx.x >> 1);
     const int tile = unit % w.max_tiles, item = unit / w.max_tiles, tid = threadIdx.x;
@@ -351,6 +352,7 @@ __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.ar
 
 template <bool TAG, bool COLS, bool MES, bool GC>
 __global__ void __launch_bounds__(32 * (SG + 2)) k_fwd_split(Work w) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char split_raw[];
     SplitShared& sh = *reinterpret_cast<SplitShared*>(split_raw);
     const int unit = blockIdx.x >> 1, q = blockIdx.x & 1;
@@ -560,19 +562,19 @@ static cudaError_t fwd_split_variant(const Work& w, unsigned grid, cudaStream_t 
         if (e != cudaSuccess) return e;
         set[gc] = sizeof(SplitShared);
     }
-    k<<<2 * grid, 32 * (SG + 2), sizeof(SplitShared), s>>>(w);
+    launch_chained(k, 2 * grid, 32 * (SG + 2), sizeof(SplitShared), s, w);
     return cudaGetLastError();
 }
 
 template <int WPC, bool GC = false>
 static void fwd_f32_variant(const Work& w, unsigned grid, int any_tag, int any_cols, bool mes, cudaStream_t s) {
     const unsigned g = grid * (2 / WPC);
-    if (any_tag && any_cols && mes) k_fwd_f32<true, true, true, WPC, GC><<<g, 32 * WPC, 0, s>>>(w);
-    else if (any_cols && mes) k_fwd_f32<false, true, true, WPC, GC><<<g, 32 * WPC, 0, s>>>(w);
-    else if (any_tag && any_cols) k_fwd_f32<true, true, false, WPC, GC><<<g, 32 * WPC, 0, s>>>(w);
-    else if (any_tag) k_fwd_f32<true, false, false, WPC, GC><<<g, 32 * WPC, 0, s>>>(w);
-    else if (any_cols) k_fwd_f32<false, true, false, WPC, GC><<<g, 32 * WPC, 0, s>>>(w);
-    else k_fwd_f32<false, false, false, WPC, GC><<<g, 32 * WPC, 0, s>>>(w);
+    if (any_tag && any_cols && mes) launch_chained(k_fwd_f32<true, true, true, WPC, GC>, g, 32 * WPC, 0, s, w);
+    else if (any_cols && mes) launch_chained(k_fwd_f32<false, true, true, WPC, GC>, g, 32 * WPC, 0, s, w);
+    else if (any_tag && any_cols) launch_chained(k_fwd_f32<true, true, false, WPC, GC>, g, 32 * WPC, 0, s, w);
+    else if (any_tag) launch_chained(k_fwd_f32<true, false, false, WPC, GC>, g, 32 * WPC, 0, s, w);
+    else if (any_cols) launch_chained(k_fwd_f32<false, true, false, WPC, GC>, g, 32 * WPC, 0, s, w);
+    else launch_chained(k_fwd_f32<false, false, false, WPC, GC>, g, 32 * WPC, 0, s, w);
 }
 
 cudaError_t launch_fwd_f32(const Work& w, int n, int max_tiles, int any_tag, int any_cols, cudaStream_t s) {

@@ -264,6 +264,27 @@ cudaError_t launch_mid64(const Work& w, int n, int Mmax, int nwmax, int Lmax, in
 cudaError_t launch_bwd64(const Work& w, int n, cudaStream_t s);
 cudaError_t mid64_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail);
 cudaError_t launch_fwd_tc(const Work& w, int n, int max_tiles, cudaStream_t s);
+// A kernel of an evaluation's chain, launched while the one before still runs: its blocks take their places
+// as that one's last blocks leave, and chain_wait() at its start waits for the whole of it (one
+// multivariate call 160 -> 151 us, 52 calls 249 -> 241; letting the blocks in from the start of the
+// kernel before put them where they fitted first, unevenly: 283).  Captured launches (bx_fit, a caller's
+// graph) stay plain.
+template <class... P, class... A>
+void launch_chained(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool plain = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = plain ? 0 : 1;
+    cudaLaunchKernelEx(&cfg, k, P(args)...);   // an error stays for the caller's cudaGetLastError
+}
 cudaError_t launch_fwd_f32(const Work& w, int n, int max_tiles, int any_tag, int any_cols, cudaStream_t s);
 // Dynamic shared memory the assembly kernel needs per item for these sizes, and the most the
 // device allows it (the opt-in limit less the kernel's static shared memory).
@@ -317,6 +338,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // Wait for the phase with the given parity; false when the time budget ran out.
+// First statement of the kernels launch_chained launches: wait for the kernel before (and with it for all
+// before that one); after a plain launch there is nothing to wait for.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned long long budget_ns) {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer();
