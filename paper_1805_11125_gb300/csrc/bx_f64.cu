@@ -231,7 +231,9 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
     const int K = T.K, N = T.N, M = T.M, NES = T.n_es;
     const double* th = w.theta + (size_t)item * w.tstride;
     const int ie = chunk * 32 + lane;
-    const int grp = MULTI ? ie / T.Ncs : 0, i = ie - grp * T.Ncs;
+    // (a chunk lies within one set: with several, Ncs is a multiple of 128; with one, the lanes past its
+    // last column stay in it too, since the warp shares the block sums below)
+    const int grp = MULTI && T.n_set > 1 ? ie / T.Ncs : 0, i = ie - grp * T.Ncs;
     const bool in = ie < T.Next && i < N;
     const size_t at = (size_t)item * w.Npad + ie;
     double* aW = w.aW + (size_t)item * w.nes * w.Npad;
