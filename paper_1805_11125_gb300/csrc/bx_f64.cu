@@ -615,7 +615,7 @@ __device__ void marg_chunk(const Work& w, const Toy& T, int item, int chunk) {
         for (int k = 0; k < KMAX; ++k) {
             double x = 0.0;
             if (k < K && in) {
-                const double wk = T.n_set > 1 ? set_weight<true>(T, k, grp) : 1.0;
+                const double wk = T.n_set > 1 || T.n_shell > 0 ? set_weight<true>(T, k, grp) : 1.0;
                 x = wk == 0.0 ? 0.0 : wk * T.shapes[(size_t)k * T.N + i];
             }
             v[k] = x * GW;

@@ -1,7 +1,8 @@
 """FP64 models whose column sets do not fill whole 32-column chunks: one radial shell (a single set of
 columns through the several-set kernels) and a plain dataset beside a quenched one, on grids whose last
-chunk holds one to a few columns behind one or more blocks of 128.  Against the oracle with the FP64
-tolerances of tests/test_gpu_parity.py."""
+chunk holds one to a few columns behind one or more blocks of 128; and a single shell that holds only a
+fraction of a species' events, in the energy spectra and in the Eq. 4 histograms.  Against the oracle
+with the FP64 tolerances of tests/test_gpu_parity.py (the FP32 ones for that mode)."""
 import dataclasses
 
 import numpy as np
@@ -51,4 +52,21 @@ def test_a_plain_dataset_beside_a_quenched_one(n_grid):
     m = bx.Model([a, b], precision=bx.BX_FP64, max_batch=2)
     for t, s in enumerate((a, b)):
         compare(m, s, s.theta_true, t)
+    m.close()
+
+
+@pytest.mark.parametrize("prec,rel,ftol,gtol", [(bx.BX_FP64, 1e-10, 1e-7, 1e-9), (bx.BX_FP32, 1e-5, 1e-3, 1e-3)])
+def test_one_shell_with_a_fraction_of_the_events(prec, rel, ftol, gtol):
+    s = model_spec(300)
+    frac = np.linspace(0.5, 0.9, s.K)[:, None]
+    s = with_data(dataclasses.replace(s, shell_ly=np.array([1.03]), shell_frac=frac))
+    th = s.theta_true
+    m = bx.Model(s, precision=prec)
+    ok, wr, wa = per_bin_ok(m.expected(th), O.expected(s, th), rel=rel, abs_frac=1e-8)
+    assert ok, (wr, wa)
+    fo, go = O.nll(s, th, grad=True)
+    f, g = m.nll_grad(th)
+    assert 2 * abs(f - fo) <= ftol, (f, fo)
+    lhs = np.abs(g[:s.P] - go) * np.abs(th)
+    assert np.all(lhs <= gtol * (1 + np.abs(go * th)))
     m.close()
