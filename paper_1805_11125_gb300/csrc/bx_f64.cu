@@ -50,6 +50,7 @@ constexpr int RUNB = 16;                // the same in the adjoint
 constexpr double HMAX = 0.2;            // largest spacing / sigma of a sampled column
 constexpr double HPOLY = 1.25;          // largest w / sigma of kind P (its polynomial's rest: poly_coef)
 constexpr size_t MID64_FIXED = 24688;   // shared memory set aside beside an item's spectra (mid64_smem_budget)
+constexpr double ZRUN = 37.0;           // |z| of the runs of kind P: z^2 / 2 < 700 (exp_tab)
 constexpr int NPOLY = 16;               // kind P: terms of the bin-mass polynomial in z^2
 enum { KIND_S = 0, KIND_P = 1, KIND_D = 2 };
 
@@ -335,9 +336,12 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
                 kind = KIND_S;
             } else {
                 cls = G64_CI;
-                kind = gc || hw > HPOLY || hw * w.band > 8.0 * HPOLY ? KIND_D : KIND_P;
-                if (kind == KIND_P) amp = norm * INV_SQRT_2PI * hw;
                 bins(bandf + 1.0f, g0, g1);
+                // kind P where its polynomial holds and its runs start in the range of exp_tab (a start
+                // may lie up to RUN64 - 1 bins below the first bin of the column)
+                const double z0 = ((double)(g0 - RUN64) * T.w - mu) * isig, z1 = ((double)g1 * T.w - mu) * isig;
+                kind = gc || hw > HPOLY || hw * w.band > 8.0 * HPOLY || fmax(-z0, z1) > ZRUN ? KIND_D : KIND_P;
+                if (kind == KIND_P) amp = norm * INV_SQRT_2PI * hw;
             }
             if (!valid || g0 >= g1) {
                 g0 = g1 = 0;

@@ -1,0 +1,126 @@
+"""How well the FP64 model knows the bins far from a column's mean.
+
+Line sources on a few neighbouring columns leave most of the axis to the response's tails: the expected
+counts are compared with the oracle's relative to themselves, and -lnL and its gradient with one event
+there.
+
+Tolerance of a tail: its argument z = (m w - mu) / sigma carries a few roundings of mu / sigma and of
+z, dz = 4 (mu / sigma + |z|) 2^-53 on either side, and the tail changes by |z| dz relative; the bin is
+a difference of two tails, which loses a factor h |z| (h = w / sigma) below 1; the terms of the sums
+and the pile-up weights another 32 roundings."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1805_11125_gb300 import bx, inputs as I
+
+pytestmark = pytest.mark.gpu
+
+TILE = 128
+EPS = 2.0 ** -53
+
+
+def line_spec(sigma, M, L=1, tag=False, kB=0.011, width=1.0, cols=(61, 64)):
+    """Three lines on neighbouring columns near 0.49 MeV (mean 220 to 235 npe), constant width."""
+    N, K = 128, 2
+    shapes = np.zeros((K, N))
+    shapes[0, cols[0]:cols[1]] = (0.5, 0.3, 0.2)
+    shapes[1, cols[0] + 1:cols[1]] = (0.4, 0.6)
+    E = I.grid_energies(N, 1.0)
+    g = I.pileup_spectrum(L, width) if L > 1 else np.ones(1)
+    s = I.ModelSpec(name="line", n_grid=N, e_max=1.0, shapes=shapes, stop_pow=I.stopping_power(E), pileup=g,
+                    width=width, m_lo=0, m_hi=M, tag_frac=np.array([0.2, 0.6]) if tag else None,
+                    species=["a", "b"])
+    s.theta_true = np.array([4e3, 2e3, 500.0, 0.0, 0.0, sigma ** 2, kB, 0.05, 1.0])
+    return s
+
+
+def columns(s, th):
+    """(mu, sigma) of the columns with support."""
+    _, mu, sig, _ = O.quench(s, th)
+    on = s.shapes.sum(0) > 0
+    return mu[on], sig[on]
+
+
+def score(s, th):
+    """Distance of every bin from the nearest column with support, in its sigma."""
+    mu, sig = columns(s, th)
+    c = (np.arange(s.m_hi) + 0.5) * s.width
+    return np.min(np.abs(c[:, None] - mu) / sig, axis=1)
+
+
+def tile_mask(s, th, band, mu, sig):
+    """[m_hi, columns]: the bins of the tiles that each column's band touches."""
+    r0 = np.maximum(0, np.floor((mu - band * sig) / s.width)).astype(int)
+    r1 = np.minimum(s.m_hi, np.floor((mu + band * sig) / s.width).astype(int) + 1)
+    t = np.arange(s.m_hi)[:, None] // TILE
+    return (r0 < r1) & (t >= r0 // TILE) & (t <= (r1 - 1) // TILE)
+
+
+def touched(s, th, band=8.0, by=np.all):
+    """Bins that every line reaches (by=np.any: some line)."""
+    return by(tile_mask(s, th, band, *columns(s, th)), axis=1)
+
+
+def tail_tol(s, th):
+    mu, sig = columns(s, th)
+    z = score(s, th)
+    h = s.width / sig.min()
+    dz = 4 * (mu.max() / sig.min() + z) * EPS
+    return 32 * EPS + (2 * z * dz + 4 * EPS) / np.minimum(1.0, h * np.maximum(z, 1.0))
+
+
+def complete(s, th):
+    """Bins whose pile-up comes from touched tiles only (below the lines the next tile down is missing)."""
+    first = int(np.argmax(touched(s, th)))
+    m = np.arange(s.m_hi)
+    return (s.L == 1) | (first == 0) | (m >= first + s.L) | ((m + 0.5) * s.width > columns(s, th)[0].min())
+
+
+def empty(s):
+    n = sum(s.hist_sizes().values())
+    return s.with_counts(np.zeros(n))
+
+
+def grad_ok(g, go, th):
+    lhs = np.abs(g - go) * np.abs(th)
+    return np.all(lhs <= 1e-9 * (1 + np.abs(go * th))), float(np.max(lhs / (1 + np.abs(go * th))))
+
+
+# ---- bands wider than the default
+
+@pytest.mark.parametrize("sigma", [0.7, 2.3, 4.5, 12.0])
+@pytest.mark.parametrize("band", [33.0, 36.0, 40.0])
+def test_wide_band_tails_relative_to_themselves(band, sigma):
+    s = empty(line_spec(sigma, 700))
+    th = s.theta_true
+    m = bx.Model(s, precision=bx.BX_FP64, band_sigmas=band)
+    mg, mo = m.expected(th), O.expected(s, th)
+    z = score(s, th)
+    use = touched(s, th, band) & (z < min(band, 37.0))
+    assert np.all(mo[use] > 0)
+    rel = np.abs(mg[use] / mo[use] - 1)
+    assert np.all(rel <= tail_tol(s, th)[use]), (float(rel.max()), float(z[use][np.argmax(rel / tail_tol(s, th)[use])]))
+    m.close()
+
+
+@pytest.mark.parametrize("band,z_event", [(36.0, -35.4), (40.0, -36.7), (40.0, 36.0), (20.0, 15.0)])
+@pytest.mark.parametrize("sigma", [4.5, 6.0])
+def test_event_at_the_end_of_a_wide_band(band, z_event, sigma):
+    s = empty(line_spec(sigma, 700))
+    th = s.theta_true
+    mu, sig = columns(s, th)
+    c = (np.arange(s.m_hi) + 0.5) * s.width
+    edge = mu.min() if z_event < 0 else mu.max()
+    b = int(np.argmin(np.abs((c - edge) / sig[0] - z_event)))
+    s.counts["sub"][b] = 1.0
+    m = bx.Model(s, precision=bx.BX_FP64, band_sigmas=band, max_batch=6)
+    fo, go = O.nll(s, th, grad=True)
+    for n in (1, 6):
+        f, g = m.nll_batch(np.stack([th] * n), grad=True)
+        assert np.all(2 * np.abs(f - fo) <= 1e-7), (f, fo)
+        ok, worst = grad_ok(g[-1], go, th)
+        assert ok, worst
+    m.close()
