@@ -530,8 +530,8 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
     w.gl64 = f64 ? g64_total(m->Mmax) : 0;
     w.wt_threads64 = f64 ? g64_wt_threads(m->Mmax) : 0;
     // 32-sample tiles a column's samples can touch: 18 sigma at 0.1 sigma a sample and one more each
-    // side (under 186 samples); a band wider than 8 sigma puts the columns on the bins
-    w.nslot64 = m->band <= 8.0 ? 7 : (m->Mmax + 31) / 32 + 1;
+    // side (under 186 samples); any other band than the default puts the columns on the bins
+    w.nslot64 = m->band == 8.0 ? 7 : (m->Mmax + 31) / 32 + 1;
     const size_t c64 = f64 ? cap : 0;
     const bool species = m->precision == BX_TF32X3;
     struct A {

@@ -15,8 +15,10 @@
 // below 1e-16 (at 6 sigma 6e-10 of the value there, at 8 sigma, the end of the band, 5e-5).
 // Columns too narrow for that (h > 0.2 at d = w) form class CI on the bins themselves, each entry
 // the exact bin mass: phi(z) times a polynomial in z^2 (kind P, sigma >= 0.8 w), or the difference of
-// erfc tails (kind D: narrower still, or a narrow Gram-Charlier column).  A band wider than 8 sigma
-// puts every column into CI (its far tails are then asked for, relative to themselves).
+// erfc tails (kind D: narrower still, or a narrow Gram-Charlier column).  Any band_sigmas but the
+// default 8 puts every column into CI, with all bins of the 128-bin tiles that its band touches: a wider
+// band asks for the far tails relative to themselves, and a narrower one cuts the response where it is
+// not small, which a stencil cannot follow.
 //
 // The adjoint is the exact transpose: the row weights go through the transposed stencils onto the
 // class grids (k_wt64), and each column sums Wt p, Wt z p, Wt z^2 p over its own samples.
@@ -50,6 +52,7 @@ constexpr int RUNB = 16;                // the same in the adjoint
 constexpr double HMAX = 0.2;            // largest spacing / sigma of a sampled column
 constexpr double HPOLY = 1.25;          // largest w / sigma of kind P (its polynomial's rest: poly_coef)
 constexpr size_t MID64_FIXED = 24688;   // shared memory set aside beside an item's spectra (mid64_smem_budget)
+constexpr double BAND_S = 8.0;          // band_sigmas of the sampled columns (the default)
 constexpr double ZRUN = 37.0;           // |z| of the runs of kind P: z^2 / 2 < 700 (exp_tab)
 constexpr int NPOLY = 16;               // kind P: terms of the bin-mass polynomial in z^2
 enum { KIND_S = 0, KIND_P = 1, KIND_D = 2 };
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
             bins(bandf, g0, g1);
             const bool valid = ok && g0 < g1 && (!MULTI || nz);
             if (valid) nrow = g1 - g0;
-            if (hw <= HMAX && w.band <= 8.0) {
+            if (hw <= HMAX && w.band == BAND_S) {
                 int c2 = 0;
                 while (c2 < G64_NC - 1 && 2.0 * h <= HMAX) {
                     h *= 2.0;
@@ -336,11 +339,17 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
                 kind = KIND_S;
             } else {
                 cls = G64_CI;
-                bins(bandf + 1.0f, g0, g1);
+                if (w.band == BAND_S) {
+                    bins(bandf + 1.0f, g0, g1);
+                } else {   // every bin of the tiles that the band touches
+                    g0 &= ~(TM - 1);
+                    g1 = min(M, (g1 + TM - 1) & ~(TM - 1));
+                }
                 // kind P where its polynomial holds and its runs start in the range of exp_tab (a start
                 // may lie up to RUN64 - 1 bins below the first bin of the column)
                 const double z0 = ((double)(g0 - RUN64) * T.w - mu) * isig, z1 = ((double)g1 * T.w - mu) * isig;
-                kind = gc || hw > HPOLY || hw * w.band > 8.0 * HPOLY || fmax(-z0, z1) > ZRUN ? KIND_D : KIND_P;
+                const double zm = fmax(-z0, z1);
+                kind = gc || hw > HPOLY || zm > ZRUN || (w.band != BAND_S && hw * zm > 8.0 * HPOLY) ? KIND_D : KIND_P;
                 if (kind == KIND_P) amp = norm * INV_SQRT_2PI * hw;
             }
             if (!valid || g0 >= g1) {

@@ -1,8 +1,10 @@
-"""How well the FP64 model knows the bins far from a column's mean.
+"""Which bins a column of the FP64 model reaches, and how well the bins far from its mean are known.
 
-Line sources on a few neighbouring columns leave most of the axis to the response's tails: the expected
-counts are compared with the oracle's relative to themselves, and -lnL and its gradient with one event
-there.
+A column (true-energy point) contributes to every bin of each 128-bin tile that its response band
+(band_sigmas) touches, and to no bin of any other tile.  Line sources on a few neighbouring columns
+leave most of the axis to the response's tails: the expected counts are compared relative to
+themselves.  References: the oracle (no band) where the touched tiles hold all that matters, and the
+oracle's response matrix under the rule above for bands that cut it.
 
 Tolerance of a tail: its argument z = (m w - mu) / sigma carries a few roundings of mu / sigma and of
 z, dz = 4 (mu / sigma + |z|) 2^-53 on either side, and the tail changes by |z| dz relative; the bin is
@@ -92,7 +94,7 @@ def grad_ok(g, go, th):
 # ---- bands wider than the default
 
 @pytest.mark.parametrize("sigma", [0.7, 2.3, 4.5, 12.0])
-@pytest.mark.parametrize("band", [33.0, 36.0, 40.0])
+@pytest.mark.parametrize("band", [10.0, 12.0, 20.0, 33.0, 36.0, 40.0])
 def test_wide_band_tails_relative_to_themselves(band, sigma):
     s = empty(line_spec(sigma, 700))
     th = s.theta_true
@@ -123,4 +125,73 @@ def test_event_at_the_end_of_a_wide_band(band, z_event, sigma):
         assert np.all(2 * np.abs(f - fo) <= 1e-7), (f, fo)
         ok, worst = grad_ok(g[-1], go, th)
         assert ok, worst
+    m.close()
+
+
+# ---- bands that cut the response
+
+def cut_reference(s, th, band):
+    """(expected counts, -lnL, gradient by central differences) of the energy spectra when every column
+    reaches the touched tiles only (the tiles held fixed in the differences)."""
+    _, mu0, sig0, _ = O.quench(s, th)
+    sup = s.shapes.sum(0) > 0
+    tiles = tile_mask(s, th, band, mu0, sig0)
+    for t in range(0, s.m_hi, TILE):   # a tile takes the columns from the first to the last that touches it
+        i = np.nonzero(tiles[t] & sup)[0]
+        tiles[t:t + TILE] = False
+        if len(i):
+            tiles[t:t + TILE, i[0]:i[-1] + 1] = True
+
+    def expect(t):
+        R, _ = O.response(s, t)
+        v = (R * tiles) @ s.shapes.T
+        w = [1 - s.tag_frac, s.tag_frac] if s.tag_frac is not None else [np.ones(s.K)]
+        return np.concatenate([O.pileup(s, t[s.K + 5], v @ (t[:s.K] * x)) for x in w])
+
+    n = s.counts_vector()
+
+    def nll(t):
+        u = expect(t)
+        with np.errstate(divide="ignore", invalid="ignore"):
+            return np.sum(u - n + np.where(n > 0, n * np.log(n / u), 0.0))
+
+    g = np.zeros(s.P)
+    for j in range(s.P):
+        if th[j] == 0.0 or j == s.K + 6:
+            continue
+        h = 1e-4 * abs(th[j])
+        d = []
+        for q in (h, h / 2):
+            a, b = th.copy(), th.copy()
+            a[j] += q
+            b[j] -= q
+            d.append((nll(a) - nll(b)) / (2 * q))
+        g[j] = (4 * d[1] - d[0]) / 3
+    return expect(th), nll(th), g
+
+
+@pytest.mark.parametrize("band,sigma,skew", [(3.0, 30.0, 0.0), (3.5, 9.0, 0.0), (4.5, 3.0, 0.0), (6.0, 60.0, 0.0),
+                                             (7.9, 20.0, 0.0), (3.0, 30.0, 0.3), (4.0, 12.0, 0.05)])
+@pytest.mark.parametrize("tag", [False, True])
+def test_band_that_cuts_the_response(band, sigma, skew, tag):
+    s = line_spec(sigma, 640, L=17, tag=tag)
+    rng = np.random.default_rng(4)
+    sh = s.shapes.copy()
+    sh[1, 40:90] += rng.random(50) / 50
+    s = dataclasses.replace(s, shapes=sh, resp_skew=skew)
+    th = s.theta_true
+    th[s.K + 1:s.K + 3] = 0.3, 1e-4
+    mu = cut_reference(empty(s), th, band)[0]
+    s = s.with_counts(np.where(mu > 0.5, np.floor(mu) + rng.integers(0, 2, mu.size), 0.0))
+    mo, fo, go = cut_reference(s, th, band)
+    m = bx.Model(s, precision=bx.BX_FP64, band_sigmas=band, max_batch=5)
+    mg = m.expected(th)
+    assert np.all(np.abs(mg - mo) <= 1e-12 * mo.max() + 1e-10 * np.abs(mo)), float(np.max(np.abs(mg - mo)) / mo.max())
+    for n in (1, 5):
+        f, g = m.nll_batch(np.stack([th] * n), grad=True)
+        assert np.all(2 * np.abs(f - fo) <= 1e-7), (f, fo)
+        # (the differences: 1e-4 steps extrapolated, rounding 1e-12 of -lnL over 1e-4)
+        lhs = np.abs(g[-1] - go) * np.abs(th)
+        lhs[s.K + 6] = 0.0
+        assert np.all(lhs <= 1e-6 * (1 + np.abs(go * th)) + 1e-7 * abs(fo)), lhs
     m.close()
