@@ -168,7 +168,10 @@ typedef struct {
     int precision;              /* bx_precision */
     int max_batch;              /* largest n of bx_nll_batch / bx_fit (>= 1) */
     double band_sigmas;         /* response entries with |m w - mu_i| > band_sigmas sigma_i
-                                   are skipped (their mass is < 1e-15); 0 -> 8 */
+                                   may be skipped (their mass is < 1e-15 at the default); 0 -> 8.
+                                   BX_FP64 skips whole tiles: a column contributes to all bins
+                                   [128 t, 128 t + 128) of the tiles that its band touches, and
+                                   to none of the others */
     double watchdog_s;          /* time budget of any device-side wait; 0 -> 2 s */
 } bx_options;
 

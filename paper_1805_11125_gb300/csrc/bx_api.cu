@@ -565,6 +565,11 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.mc64, m->any_cols ? sizeof(double) * c64 * (w.Npad / 32) * w.nes * 32 : 16},
         {(void**)&w.wt64, sizeof(double) * c64 * (2 + w.nes) * w.gl64},
         {(void**)&w.wv64, sizeof(double) * c64 * 2 * w.Mpad},
+        {(void**)&w.ctile64, sizeof(uint2) * c64 * (w.Npad / 32)},
+        {(void**)&w.tmask64, sizeof(unsigned long long) * c64},
+        {(void**)&w.rows64, sizeof(unsigned) * c64 * 2 * 3 * (w.Mpad / 32)},
+        {(void**)&w.xany64, sizeof(int) * c64},
+        {(void**)&w.xw64, sizeof(double) * c64 * 2 * w.Mpad},
         {(void**)&w.part64, sizeof(double) * c64 * 2 * ((m->nwmax + 31) / 32) * 4},
         {(void**)&w.v, species ? 2 * tv * cap * w.Mpad * US : 16},   // hi, lo planes
         {(void**)&w.rowW, tv * cap * (2 + w.nes) * w.Mpad},

@@ -11,8 +11,13 @@
 // grouped by width into classes c = 0 .. 6 with sample spacing d = 2^c w, such that h = d / sigma
 // lies in (0.1, 0.2]: a column takes 90 - 180 samples whatever its width (its bins are 16 sigma / w,
 // 160 - 640 at w = 1 npe).  Down a column the samples follow by a recurrence (two multiplications
-// each) from an exact start every RUN64 samples.  The stencil's error relative to a column's peak is
-// below 1e-16 (at 6 sigma 6e-10 of the value there, at 8 sigma, the end of the band, 5e-5).
+// each) from an exact start every RUN64 samples.
+// A column contributes to every bin of the 128-bin tiles that its band (8 sigma) touches and to no other
+// tile; its samples end one sigma past the band.  The stencil is good to about 1e-17 of the largest
+// sample it meets, so a bin with content nearby is known to 1e-14 of itself: up to 4.6 sigma from the
+// nearest column at a spacing of 0.2 sigma, 7 sigma at 0.1.  In the tails beyond (k_lam64 marks them) the
+// bins whose counts matter relative to themselves -- those with an event, and the expected counts a
+// caller asks for -- take the exact bin masses of their tile's columns (tail_bins, tail_adjoint).
 // Columns too narrow for that (h > 0.2 at d = w) form class CI on the bins themselves, each entry
 // the exact bin mass: phi(z) times a polynomial in z^2 (kind P, sigma >= 0.8 w), or the difference of
 // erfc tails (kind D: narrower still, or a narrow Gram-Charlier column).  Any band_sigmas but the
@@ -27,7 +32,8 @@
 //   k_cols64   per column: mu, sigma, normalisation, window masses, spectra, class, sample range
 //   k_dens64   per 32-sample tile of a class grid: F_h[g] = sum_i A_i S_h[i] p_i[g], and for the
 //              Eq. 4 terms each column's sum_g p_i[g] Gt_s[g]
-//   k_lam64    per bin: lambda_h[m] from the class grids; per chunk: the Eq. 4 sums of every species
+//   k_lam64    per bin: lambda_h[m] from the class grids, and whether it lies in the tails; per chunk:
+//              the Eq. 4 sums of every species
 //   k_pile64   per 32 window bins: Eq. 2, the -lnL terms and weights 1 - n/mu
 //   k_marg64   per item: Eq. 4 marginals and their terms, -lnL, the species' adjoint coefficients
 //   k_corr64   per 32 axis bins: adjoint of Eq. 2;   k_wt64: row weights onto the class grids
@@ -195,6 +201,8 @@ __global__ void __launch_bounds__(128) k_scan64(Work w, int nblk) {
         if (tid == 0) {
             w.status[item] = any ? (int)BX_EDOMAIN : 0;
             w.cmask64[item] = 0;
+            w.xany64[item] = 0;
+            w.tmask64[item] = 0ull;
         }
     }
     // (with several column sets a set starts on a block: Ncs is a multiple of 128)
@@ -223,6 +231,14 @@ __global__ void __launch_bounds__(128) k_scan64(Work w, int nblk) {
     if (tid == 127) w.qtot64[(size_t)item * (w.Npad / 128) + blk] = make_double2(ax + x, ay + y);
 }
 
+// Bins [r0, r1) within nsig sigma of a column's mean.
+__device__ __forceinline__ void near_bins(double mu, double sig, double w, int M, float nsig, int& r0, int& r1) {
+    const float muf = (float)mu, sigf = (float)sig, wf = (float)w, iwf = 1.0f / wf;
+    const float e_min = -2.0f * wf, e_max = (M + 2.0f) * wf;
+    r0 = max(0, (int)floorf(fminf(fmaxf(muf - nsig * sigf, e_min), e_max) * iwf));
+    r1 = min(M, (int)floorf(fminf(fmaxf(muf + nsig * sigf, e_min), e_max) * iwf) + 1);
+}
+
 // One thread per column, a warp per 32-column chunk: Eq. 1's mean and width, the normalisation
 // 1/Phi(mu/sigma), the masses of the energy slices, the spectra S_h[i] = sum_k r_k c_{h,k} s_k[i]
 // times the column's amplitude, its class, kind and sample range, and per chunk the sample range of
@@ -242,6 +258,7 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
     const size_t at = (size_t)item * w.Npad + ie;
     double* aW = w.aW + (size_t)item * w.nes * w.Npad;
     int g0 = 0, g1 = 0, cls = -1, kind = KIND_S, nrow = 0;
+    unsigned tlo = 0u, thi = 0u;   // tiles of 128 bins that the column's band touches
     Col64 cc{0.0, 1.0, 0.0, 0.0};
     double2 sp = make_double2(0.0, 0.0);
     Gen64 gen{0.0, 0.0, 0.0, 0.0};   // mu, 1/sigma, 1 - e^(-h^2), amplitude
@@ -314,14 +331,14 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
             // variant; 6.5e-15 without the cut, 5.2e-14 in the erfc form this replaced).
             const float muf = (float)mu, sigf = (float)sig, bandf = (float)w.band, wf = (float)T.w;
             double h = hw, amp = norm;
-            const float e_min = -2.0f * wf, e_max = (M + 2.0f) * wf, iwf = 1.0f / wf;
-            auto bins = [&](float nsig, int& r0, int& r1) {
-                r0 = max(0, (int)floorf(fminf(fmaxf(muf - nsig * sigf, e_min), e_max) * iwf));
-                r1 = min(M, (int)floorf(fminf(fmaxf(muf + nsig * sigf, e_min), e_max) * iwf) + 1);
-            };
-            bins(bandf, g0, g1);
+            near_bins(mu, sig, T.w, M, bandf, g0, g1);
             const bool valid = ok && g0 < g1 && (!MULTI || nz);
-            if (valid) nrow = g1 - g0;
+            if (valid) {
+                nrow = g1 - g0;
+                const unsigned long long tm = (2ull << ((g1 - 1) / TM)) - (1ull << (g0 / TM));
+                tlo = (unsigned)tm;
+                thi = (unsigned)(tm >> 32);
+            }
             if (hw <= HMAX && w.band == BAND_S) {
                 int c2 = 0;
                 while (c2 < G64_NC - 1 && 2.0 * h <= HMAX) {
@@ -340,7 +357,7 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
             } else {
                 cls = G64_CI;
                 if (w.band == BAND_S) {
-                    bins(bandf + 1.0f, g0, g1);
+                    near_bins(mu, sig, T.w, M, bandf + 1.0f, g0, g1);
                 } else {   // every bin of the tiles that the band touches
                     g0 &= ~(TM - 1);
                     g1 = min(M, (g1 + TM - 1) & ~(TM - 1));
@@ -369,6 +386,12 @@ __global__ void __launch_bounds__(128) k_cols64(Work w, int nblk) {
     if (w.count_units) {
         const int r = __reduce_add_sync(0xffffffffu, nrow);
         if (lane == 0 && r) atomicAdd(w.units, (unsigned long long)r);
+    }
+    tlo = __reduce_or_sync(0xffffffffu, tlo);
+    thi = __reduce_or_sync(0xffffffffu, thi);
+    if (lane == 0) {
+        w.ctile64[(size_t)item * (w.Npad / 32) + chunk] = make_uint2(tlo, thi);
+        if (tlo | thi) atomicOr(&w.tmask64[item], (unsigned long long)thi << 32 | tlo);
     }
     int mask = 0;
     for (int c = 0; c <= G64_NC; ++c) {
@@ -639,8 +662,25 @@ __device__ void marg_chunk(const Work& w, const Toy& T, int item, int chunk) {
     }
 }
 
+// Rows of bits per bin of one spectrum's axis (k_lam64 writes all three).
+enum { ROWS_TAIL = 0, ROWS_STRONG = 1, ROWS_EXACT = 2, ROWS_N = 3 };
+__device__ __forceinline__ unsigned* bin_rows(const Work& w, int item, int h, int which) {
+    return w.rows64 + (((size_t)item * 2 + h) * ROWS_N + which) * (w.Mpad / 32);
+}
+__device__ __forceinline__ bool row_bit(const unsigned* r, int m) { return (r[m >> 5] >> (m & 31)) & 1u; }
+// A bin in the tails of everything near it: below 2^-TAIL_BITS of the largest sample that its stencils
+// meet (top: that sample's exponent word).  The stencil is good to about 1e-17 of that sample: to 1e-14
+// of a bin above the line (4.6 to 7 sigma from the columns, for spacings of 0.2 to 0.1 sigma), and no
+// longer at the end of the samples.
+constexpr int TAIL_BITS = 14, STRONG_BITS = 3;
+__device__ __forceinline__ bool in_tail(double v, int top) {
+    const int e = __double2hiint(v);
+    return e <= top - (TAIL_BITS << 20) || e < (40 << 20);
+}
+
 // lambda_h[m]: the stencil of bin m's phase over each class's samples around its cell, plus CI.  A
-// bin no column's samples reach (every class's own cell empty) is exactly 0, as the band says.  The
+// bin no column's samples reach (every class's own cell empty) and a tile that no column's band touches
+// are exactly 0; the bins in the tails of a touched tile are marked for k_pile64.  The
 // first nrb CTAs of an item do that; the others take the marginal sums of four chunks each.
 // nplane: the forward's partial planes (small batches), added in the order of its four warps.
 template <bool TAG>
@@ -654,67 +694,264 @@ __global__ void __launch_bounds__(128) k_lam64(Work w, int nrb, int nall, int np
         return;
     }
     const int M = T.M, present = w.cmask64[item];
+    const bool touched = w.band != BAND_S || ((w.tmask64[item] >> blk) & 1ull);   // (128 bins: one tile)
     if (blk * 128 >= M) return;
     // the samples of a class that the CTA's 128 bins meet, the planes added, in shared memory
     const size_t ps = (size_t)w.gl64 * 2;   // between planes
     const double* F = w.F64 + (size_t)item * nplane * ps;
-    __shared__ double sF[TAG ? 2 : 1][128 + 2 * R64];
-    double s = 0.0, t = 0.0;
-    bool hs = false, ht = false;
+    constexpr int H = TAG ? 2 : 1;
+    __shared__ double sF[H][128 + 2 * R64];
+    __shared__ __align__(16) int s_top[H][4];
+    // stages class c's samples for the bins: sample g + R64 of the staged ones is a bin's own
+    // (top: the largest of them, by exponent word per bin width)
+    auto stage = [&](int c, int off, int (&top)[H]) {
+        int t[H] = {};
+        const bool ci = c == G64_CI;
+        const int g0 = ci ? blk * 128 - R64 : (blk * 128) >> c, ng = (ci ? 127 : 127 >> c) + 1 + 2 * R64;
+        const int len = g64_len(M, c);
+        __syncthreads();
+        for (int q = threadIdx.x; q < H * ng; q += 128) {
+            const int hh = q / ng, g = q - hh * ng;
+            double v = 0.0;
+            if (g0 + g >= 0 && g0 + g < len) {
+                const double* f = F + (size_t)hh * w.gl64 + off + g0 + g;
+                v = nplane == 1 ? f[0] : (f[0] + f[ps]) + (f[2 * ps] + f[3 * ps]);
+            }
+            sF[hh][g] = v;
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+                if (h == hh) t[h] = max(t[h], __double2hiint(v) & 0x7fffffff);
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const int r = __reduce_max_sync(0xffffffffu, t[h]);
+            if ((threadIdx.x & 31) == 0) s_top[h][threadIdx.x >> 5] = r;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const int r = max(max(s_top[h][0], s_top[h][1]), max(s_top[h][2], s_top[h][3]));
+            top[h] = max(top[h], r - (ci ? 0 : c << 20));
+        }
+        return ci ? (int)threadIdx.x : (m >> c) - g0;
+    };
+    double lam[H];
+    bool any[H];
+    int top[H];   // exponent word of the largest sample staged, per bin width
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        lam[h] = 0.0;
+        any[h] = false;
+        top[h] = 0;
+    }
     int off = 0;
     for (int c = 0; c <= G64_NC; ++c) {
         if ((present >> c) & 1) {
-            const bool ci = c == G64_CI;
-            const int g0 = ci ? blk * 128 : (blk * 128) >> c, ng = ci ? 128 : (127 >> c) + 1 + 2 * R64;
-            const int len = g64_len(M, c);
-            __syncthreads();
-            for (int q = threadIdx.x; q < (TAG ? 2 : 1) * ng; q += 128) {
-                const int hh = q / ng, g = q - hh * ng;
-                double v = 0.0;
-                if (g0 + g < len) {
-                    const double* f = F + (size_t)hh * w.gl64 + off + g0 + g;
-                    v = nplane == 1 ? f[0] : (f[0] + f[ps]) + (f[2 * ps] + f[3 * ps]);
-                }
-                sF[hh][g] = v;
-            }
-            __syncthreads();
+            const int g = stage(c, off, top);
             if (m < M) {
-                if (ci) {
-                    s += sF[0][threadIdx.x];
-                    hs |= sF[0][threadIdx.x] != 0.0;
-                    if (TAG) {
-                        t += sF[TAG ? 1 : 0][threadIdx.x];
-                        ht |= sF[TAG ? 1 : 0][threadIdx.x] != 0.0;
-                    }
-                } else {
+                double a[H];
+#pragma unroll
+                for (int h = 0; h < H; ++h) a[h] = c == G64_CI ? sF[h][g + R64] : 0.0;
+                if (c != G64_CI) {
                     const double* st = g64_stencil(w, c, m & ((1 << c) - 1));
-                    const int g = (m >> c) - g0;   // sample g - R64 of the class
-                    double a = 0.0, b = 0.0;
 #pragma unroll 11
-                    for (int j = 0; j < TAPS; ++j) {
-                        a = fma(st[j], sF[0][g + j], a);
-                        if (TAG) b = fma(st[j], sF[TAG ? 1 : 0][g + j], b);
-                    }
-                    s += a;
-                    t += b;
-                    hs |= sF[0][g + R64] != 0.0;
-                    if (TAG) ht |= sF[TAG ? 1 : 0][g + R64] != 0.0;
+                    for (int j = 0; j < TAPS; ++j)
+#pragma unroll
+                        for (int h = 0; h < H; ++h) a[h] = fma(st[j], sF[h][g + j], a[h]);
+                }
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    lam[h] += a[h];
+                    any[h] |= sF[h][g + R64] != 0.0;
                 }
             }
         }
         off += g64_len(M, c);
     }
-    if (m >= M) return;
-    double* lam = w.lam + (size_t)item * 2 * w.Mpad;
-    lam[m] = hs ? s : 0.0;
-    if (TAG) lam[w.Mpad + m] = ht ? t : 0.0;
+    if (w.band != BAND_S) {
+        for (int h = 0; h < H; ++h)
+            if (m < M) w.lam[((size_t)item * 2 + h) * w.Mpad + m] = any[h] ? lam[h] : 0.0;
+        return;
+    }
+    bool tail = false, strong[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        lam[h] = m < M && any[h] && touched ? lam[h] : 0.0;
+        if (m < M) w.lam[((size_t)item * 2 + h) * w.Mpad + m] = lam[h];
+        strong[h] = __double2hiint(lam[h]) >= max(top[h] - (STRONG_BITS << 20), 40 << 20);
+        tail |= m < M && touched && in_tail(lam[h], top[h]);
+    }
+    // the largest of all samples staged bounds each bin's; only where that leaves a doubt, its own
+    const bool doubt = __syncthreads_or(tail);
+    if (doubt) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) top[h] = 0;
+        off = 0;
+        for (int c = 0; c <= G64_NC; ++c) {
+            if ((present >> c) & 1) {
+                int all[H] = {};
+                const int g = stage(c, off, all);
+                for (int j = 0; m < M && j < TAPS; ++j)
+#pragma unroll
+                    for (int h = 0; h < H; ++h)
+                        top[h] = max(top[h], (__double2hiint(sF[h][g + j]) & 0x7fffffff) - (c == G64_CI ? 0 : c << 20));
+            }
+            off += g64_len(M, c);
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const unsigned bt = __ballot_sync(0xffffffffu, doubt && m < M && touched && in_tail(lam[h], top[h]));
+        const unsigned bs = __ballot_sync(0xffffffffu, strong[h]);
+        if ((threadIdx.x & 31) == 0) {
+            bin_rows(w, item, h, ROWS_TAIL)[m >> 5] = bt;
+            bin_rows(w, item, h, ROWS_STRONG)[m >> 5] = bs;
+            bin_rows(w, item, h, ROWS_EXACT)[m >> 5] = 0u;
+        }
+    }
+}
+
+// ------------------------------------------------------------------ bins in the tails
+
+// Whether some column of the chunk, this column, touches the tile with its band.
+__device__ __forceinline__ bool chunk_touches(const Work& w, int item, int chunk, int tile) {
+    const uint2 t = w.ctile64[(size_t)item * (w.Npad / 32) + chunk];
+    return ((tile < 32 ? t.x >> tile : t.y >> (tile - 32)) & 1u) != 0u;
+}
+__device__ __forceinline__ bool column_touches(const Work& w, const Toy& T, int item, int ie, int tile) {
+    const size_t at = (size_t)item * w.Npad + ie;
+    if (w.colc64[at].x < 0) return false;
+    const Col64 cc = w.col64[at];
+    int r0, r1;
+    near_bins(cc.mu, cc.sig, T.w, T.M, (float)w.band, r0, r1);
+    return r0 < r1 && tile >= r0 / TM && tile <= (r1 - 1) / TM;
+}
+
+// lambda_h[m] summed over the columns that touch the bin's tile, each bin mass the difference of erfc tails; by
+// the whole block (128 threads).  A first pass over the columns finds the largest term to a few bits (the
+// exponents and z^2 in FP32), the second evaluates those within 2^-70 of it: FP64 erfc costs about 100
+// operations, and a few hundred of the columns matter.
+__device__ double exact_bin(const Work& w, const Toy& T, int item, int h, int m, double* red) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const size_t cb = (size_t)item * w.Npad;
+    const bool gc = T.gc1 != 0.0 || T.gc2 != 0.0;
+    const double ya = (double)m * T.w, yb = (double)(m + 1) * T.w;
+    float top = -3.0e38f;
+    double sum = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int ch = wid; ch * 32 < T.Next; ch += 4) {
+            if (!chunk_touches(w, item, ch, m / TM)) continue;
+            const int ie = ch * 32 + lane;
+            const double2 S2 = w.colS[cb + ie];
+            const double S = h ? S2.y : S2.x;
+            if (S != 0.0 && column_touches(w, T, item, ie, m / TM)) {
+                const Gen64 gen = w.gen64[cb + ie];
+                const double za = (ya - gen.x) * gen.y, zb = (yb - gen.x) * gen.y;
+                const float z = (float)(za > 0.0 ? za : zb < 0.0 ? zb : 0.0);
+                const float e = (float)((__double2hiint(S) >> 20) & 0x7ff) - 0.72134752f * z * z;
+                if (pass == 0) {
+                    top = fmaxf(top, e);
+                } else if (e >= top - 70.0f) {
+                    bool fa, fb;
+                    const double ta = edge_tail(T, za, gc, fa), tb = edge_tail(T, zb, gc, fb);
+                    const double D = tb - ta + ((!fa && fb) ? 1.0 : 0.0);
+                    sum = fma(S * (w.col64[cb + ie].norm / gen.w), D, sum);
+                }
+            }
+        }
+        __syncthreads();   // (red: the bin before)
+        if (pass == 0) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+            if (lane == 0) red[wid] = top;
+            __syncthreads();
+            top = (float)fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
+        } else {
+            sum = warp_sum(sum);
+            if (lane == 0) red[wid] = sum;
+            __syncthreads();
+            sum = (red[0] + red[1]) + (red[2] + red[3]);
+        }
+    }
+    return sum;
+}
+
+// Data in the tails (ev: bins of this CTA's 32 with an event, or all of them for the expected counts).
+// Those bins' own lambda is replaced by exact_bin's; and, unless their pile-up comes from well within the
+// columns (a strong bin at a shift with at least 1 % of the largest g: the tails then enter below 1e-12),
+// that of every tail bin within the reach of g.  The bins are marked for the adjoint.
+__device__ __noinline__ void tail_bins(const Work& w, const Toy& T, int item, int h, unsigned ev, int m0, int Lt,
+                                       const double* sg, double* sx) {
+    __shared__ unsigned s_need[(MAX_L + 32) / 32 + 1];
+    __shared__ double s_red[4];
+    const int tid = threadIdx.x, nrow = 32 + Lt - 1;
+    const unsigned *tail = bin_rows(w, item, h, ROWS_TAIL), *strong = bin_rows(w, item, h, ROWS_STRONG);
+    double gm = 0.0;
+    for (int d = tid; d < Lt; d += 128) gm = fmax(gm, sg[d]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+    if ((tid & 31) == 0) s_red[tid >> 5] = gm;
+    for (int q = tid; q <= nrow / 32; q += 128) s_need[q] = 0u;
+    __syncthreads();
+    gm = 0.01 * fmax(fmax(s_red[0], s_red[1]), fmax(s_red[2], s_red[3]));
+    for (unsigned e = ev; e; e &= e - 1u) {
+        const int b = __ffs(e) - 1, m = m0 + b, Lb = min(Lt, m + 1), q0 = Lt - 1 + b;   // sx[q0]: the bin
+        bool lit = false;
+        for (int d = 1 + tid; d < Lb; d += 128) lit |= sg[d] >= gm && row_bit(strong, m - d);
+        const bool own = __syncthreads_or(lit);
+        for (int d = tid; d < (own ? 1 : Lb); d += 128)
+            if (row_bit(tail, m - d)) atomicOr(&s_need[(q0 - d) >> 5], 1u << ((q0 - d) & 31));
+    }
+    __syncthreads();
+    for (int q0 = 0; q0 < nrow; q0 += 32)
+        for (unsigned r = s_need[q0 >> 5]; r; r &= r - 1u) {
+            const int q = q0 + __ffs(r) - 1, m = m0 - (Lt - 1) + q;
+            const double v = exact_bin(w, T, item, h, m, s_red);
+            if (tid == 0) {
+                sx[q] = v;
+                atomicOr(&bin_rows(w, item, h, ROWS_EXACT)[m >> 5], 1u << (m & 31));
+                w.xany64[item] = 1;
+            }
+        }
+    __syncthreads();
+}
+
+// The adjoint of the bins that tail_bins took (their row weights xw64 are not in rowW), for one column:
+// sums of the species-summed weights times the bin mass and its derivatives (E[0 .. 2]), and of the
+// weights times the mass (E[3], E[4]: vetoed, tagged), as kind D's.
+__device__ __noinline__ void tail_adjoint(const Work& w, const Toy& T, int item, int ie, double Ss, double St, double mu,
+                                          double isig, double (&E)[5]) {
+    const bool gc = T.gc1 != 0.0 || T.gc2 != 0.0;
+    for (int h = 0; h < (T.has_tag ? 2 : 1); ++h) {
+        const unsigned* rows = bin_rows(w, item, h, ROWS_EXACT);
+        const double S = h ? St : Ss;
+        for (int b = 0; b * 32 < T.M; ++b)
+            for (unsigned r = rows[b]; r; r &= r - 1u) {
+                const int m = b * 32 + __ffs(r) - 1;
+                if (!column_touches(w, T, item, ie, m / TM)) continue;
+                const double W = w.xw64[((size_t)item * 2 + h) * w.Mpad + m];
+                const double za = ((double)m * T.w - mu) * isig, zb = ((double)(m + 1) * T.w - mu) * isig;
+                bool fa, fb;
+                const double ta = edge_tail(T, za, gc, fa), tb = edge_tail(T, zb, gc, fb);
+                double pa = INV_SQRT_2PI * exp(-0.5 * za * za), pb = INV_SQRT_2PI * exp(-0.5 * zb * zb);
+                if (gc) {
+                    pa *= gc_density_factor(T, za);
+                    pb *= gc_density_factor(T, zb);
+                }
+                const double q = W * (tb - ta + ((!fa && fb) ? 1.0 : 0.0));
+                E[0] = fma(q, S, E[0]);
+                E[1] = fma(-W * (pb - pa), S, E[1]);
+                E[2] = fma(-W * (zb * pb - za * pa), S, E[2]);
+                E[3 + h] += q;
+            }
+    }
 }
 
 // ------------------------------------------------------------------ assembly
 
 // CTA = 32 window bins of one spectrum of one item, a warp per quarter of the taps: Eq. 2, the
 // Baker-Cousins terms, w = 1 - n/mu, and the tile's part of -lnL (compensated) and of d/deps.
-__global__ void __launch_bounds__(128) k_pile64(Work w, int ntw, int nH, int want_grad, int want_mu) {
+__global__ void __launch_bounds__(128, 10) k_pile64(Work w, int ntw, int nH, int want_grad, int want_mu) {
     extern __shared__ __align__(16) double dsm[];
     const int t = blockIdx.x % ntw, h = (blockIdx.x / ntw) % nH, item = blockIdx.x / (ntw * nH), tid = threadIdx.x;
     double* part = w.part64 + (((size_t)item * nH + h) * ntw + t) * 4;
@@ -734,9 +971,16 @@ __global__ void __launch_bounds__(128) k_pile64(Work w, int ntw, int nH, int wan
         const int m = m0 - (Lt - 1) + q;
         sx[q] = m >= 0 && m < T.M ? lam[m] : 0.0;
     }
+    const int b = tid & 31, pt = tid >> 5, j = t * 32 + b, pl = (Lt + 3) / 4;
+    unsigned ev = 0u;   // bins in the tails whose counts matter relative to themselves
+    if (w.band == BAND_S) {
+        bool e = j < nw && row_bit(bin_rows(w, item, h, ROWS_TAIL), m0 + b);
+        if (e) e = want_mu || T.cnt[(size_t)h * nw + j] != 0.0;
+        ev = __ballot_sync(0xffffffffu, e);
+    }
     __shared__ double sc[3][32];
     __syncthreads();
-    const int b = tid & 31, pt = tid >> 5, j = t * 32 + b, pl = (Lt + 3) / 4;
+    if (ev) tail_bins(w, T, item, h, ev, m0, Lt, sg, sx);
     const int d0 = min(Lt, pt * pl), d1 = min(Lt, d0 + pl);
     const double* x = sx + (Lt - 1) + b;
     double c0 = 0.0, c1 = 0.0;
@@ -1019,7 +1263,12 @@ __global__ void __launch_bounds__(128) k_corr64(Work w, int ntm, int nH) {
     __syncthreads();
     if (pt || m >= M) return;
     const double direct = m >= m_lo ? (1.0 - eps) * wv[m - m_lo] : 0.0;
-    rowW[(size_t)h * w.Mpad + m] = direct + eps * (((c0 + c1) + sc[0][b]) + (sc[1][b] + sc[2][b]));
+    double val = direct + eps * (((c0 + c1) + sc[0][b]) + (sc[1][b] + sc[2][b]));
+    if (w.xany64[item] && row_bit(bin_rows(w, item, h, ROWS_EXACT), m)) {   // tail_adjoint's
+        w.xw64[((size_t)item * 2 + h) * w.Mpad + m] = val;
+        val = 0.0;
+    }
+    rowW[(size_t)h * w.Mpad + m] = val;
 }
 
 // ------------------------------------------------------------------ adjoint
@@ -1147,6 +1396,7 @@ __global__ void __launch_bounds__(32) k_bwd64(Work w, int nch) {
         }
     }
     const Col64 cc = w.col64[at];
+    const int exact = w.xany64[item];
     const Gen64 gen = live ? w.gen64[at] : Gen64{0.0, 0.0, 0.0, 0.0};
     double P0 = 0.0, P1 = 0.0, P2 = 0.0, Rs = 0.0, Rt = 0.0;
     double f1 = 1.0, f2 = 1.0, f0 = 0.0;   // S1 = f1 P1, S2 = f2 (P2 - f0 P0)
@@ -1306,7 +1556,17 @@ __global__ void __launch_bounds__(32) k_bwd64(Work w, int nch) {
     if (live) {
         const double* th = w.theta + (size_t)item * w.tstride;
         const double LY = th[K], a = th[K + 1], b = th[K + 2], mu = cc.mu, sig = cc.sig, isig = gen.y, amp = gen.w;
-        const double S0 = amp * P0, S1 = amp * isig * f1 * P1, S2 = amp * isig * f2 * (P2 - f0 * P0);
+        double S0 = amp * P0, S1 = amp * isig * f1 * P1, S2 = amp * isig * f2 * (P2 - f0 * P0);
+        double rs = amp * Rs, rt = amp * Rt;
+        if (exact) {
+            double E[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+            tail_adjoint(w, T, item, ie, Sv[0], Sv[1], mu, isig, E);
+            S0 = fma(cc.norm, E[0], S0);
+            S1 = fma(cc.norm * isig, E[1], S1);
+            S2 = fma(cc.norm * isig, E[2], S2);
+            rs = fma(cc.norm, E[3], rs);
+            rt = fma(cc.norm, E[4], rt);
+        }
         const double dmu = S1 - cc.mills * isig * S0;
         const double dsig = S2 + cc.mills * mu * isig * isig * S0;
         const double D = dsig / (2.0 * sig);
@@ -1317,7 +1577,6 @@ __global__ void __launch_bounds__(32) k_bwd64(Work w, int nch) {
         g[2] = D * mu * mu;        // b
         g[3] = D;                  // c
         g[4] = Gmu * LY * q.y;     // kB
-        const double rs = amp * Rs, rt = amp * Rt;
 #pragma unroll
         for (int k = 0; k < KMAX; ++k)
             if (k < K) {

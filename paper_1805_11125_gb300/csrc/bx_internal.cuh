@@ -205,6 +205,11 @@ struct Work {
     double* wt64;             // [cap][2 + nes][gl64]: row weights on the class grids
     double* wv64;             // [cap][2][Mpad]: 1 - n/mu on the window
     double* part64;           // [cap][2 * window tiles][4]: -lnL sum and compensation, d/deps, domain flag
+    uint2* ctile64;           // [cap][Npad/32]: tiles of 128 bins that the chunk's bands touch (bits)
+    unsigned long long* tmask64;   // [cap]: the same of all columns
+    unsigned* rows64;         // [cap][2][3][Mpad/32]: bits per bin (in the tails, strong, taken exactly)
+    int* xany64;              // [cap]: some bin was taken exactly
+    double* xw64;             // [cap][2][Mpad]: row weights of the bins taken exactly
     int nslot64, gl64, wt_threads64;
     const unsigned char* skip;   // [cap] or nullptr: items flagged 1 are not evaluated (-lnL = +inf)
     // 2D model buffers (UMMA K-major tiles of TF32 hi | lo halves, NSL slices x KB)

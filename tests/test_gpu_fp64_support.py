@@ -195,3 +195,114 @@ def test_band_that_cuts_the_response(band, sigma, skew, tag):
         lhs[s.K + 6] = 0.0
         assert np.all(lhs <= 1e-6 * (1 + np.abs(go * th)) + 1e-7 * abs(fo)), lhs
     m.close()
+
+
+# ---- bins beyond the default band
+
+def far_bins(s, th, zs):
+    """The bins nearest to the scores zs above the last line and below the first, inside the axis."""
+    mu, sig = columns(s, th)
+    c = (np.arange(s.m_hi) + 0.5) * s.width
+    out = []
+    for z in zs:
+        for edge, sg in ((mu.max(), 1), (mu.min(), -1)):
+            x = edge + sg * z * sig[0]
+            if c[0] <= x <= c[-1]:
+                out.append(int(np.argmin(np.abs(c - x))))
+    return sorted(set(out))
+
+
+SIGMAS = [0.6, 1.3, 3.0, 5.2, 9.9, 16.0, 39.0, 70.0]
+
+
+@pytest.mark.parametrize("L", [1, 3, 40, 400])
+@pytest.mark.parametrize("sigma", SIGMAS)
+def test_tails_of_the_default_band_relative_to_themselves(sigma, L):
+    s = empty(line_spec(sigma, 900, L=L))
+    th = s.theta_true
+    m = bx.Model(s, precision=bx.BX_FP64)
+    mg, mo = m.expected(th), O.expected(s, th)
+    reach = touched(s, th)
+    z = score(s, th)
+    use = reach & (z < 37.0)
+    use &= complete(s, th)
+    tol = tail_tol(s, th)[use]
+    rel = np.abs(mg[use] / mo[use] - 1)
+    assert np.all(rel <= tol), (float(rel.max()), float(z[use][np.argmax(rel / tol)]))
+    if L == 1:
+        assert np.all(mg[~touched(s, th, by=np.any)] == 0.0)
+    m.close()
+
+
+@pytest.mark.parametrize("L", [1, 40, 400])
+@pytest.mark.parametrize("sigma", SIGMAS)
+def test_event_beyond_the_default_band(sigma, L):
+    s0 = empty(line_spec(sigma, 900, L=L, tag=True))
+    th = s0.theta_true
+    reach = touched(s0, th)
+    rng = np.random.default_rng(1)
+    base = [rng.poisson(np.minimum(x, 1e6)).astype(float) for x in np.split(O.expected(s0, th), 2)]
+    keep = score(s0, th) < 4.0
+    reach &= complete(s0, th)
+    bins = [b for b in far_bins(s0, th, (5.0, 6.2, 7.4, 8.3, 8.8, 9.5, 12.0, 20.0, 33.0)) if reach[b]]
+    assert bins
+    for j, b in enumerate(bins):
+        s = dataclasses.replace(s0, counts={})
+        s.counts = {"sub": np.where(keep, base[0], 0.0), "tag": np.where(keep, base[1], 0.0)}
+        s.counts["tag" if j % 2 else "sub"][b] = 1.0
+        m = bx.Model(s, precision=bx.BX_FP64, max_batch=6)
+        fo, go = O.nll(s, th, grad=True)
+        for n in (1, 6):
+            f, g = m.nll_batch(np.stack([th] * n), grad=True)
+            assert np.all(2 * np.abs(f - fo) <= 1e-7), (b, f, fo)
+            ok, worst = grad_ok(g[-1], go, th)
+            assert ok, (b, worst)
+        m.close()
+
+
+@pytest.mark.parametrize("sigma", [9.9, 16.0, 39.0])
+def test_no_tile_beyond_the_default_band(sigma):
+    """Without pile-up an event in the first bins of a tile that no band touches has no expected count."""
+    s = empty(line_spec(sigma, 900))
+    th = s.theta_true.copy()
+    _, q, _, _ = O.quench(s, th)
+    # the last line's band ends on a tile's last bin
+    mu, sig = columns(s, th)
+    last = (np.ceil((mu.max() + 8 * sigma) / TILE) + (1 if sigma > 30 else 0)) * TILE - 0.5
+    th[s.K] *= (last - 8 * sigma) / mu.max()
+    end = int(last + 0.5)
+    some = touched(s, th, by=np.any)
+    assert not some[end] and some[end - 1]
+    for b, inside in ((end - 1, True), (end, False), (end + 3, False)):   # (8 sigma past the last line, and on)
+        s.counts["sub"][:] = 0.0
+        s.counts["sub"][b] = 1.0
+        m = bx.Model(s, precision=bx.BX_FP64)
+        assert (m.expected(th)[b] > 0) == inside
+        if inside:
+            assert 2 * abs(m.nll(th) - O.nll(s, th)) <= 1e-7
+        else:
+            with pytest.raises(bx.BxError) as e:
+                m.nll(th)
+            assert e.value.status == bx.BX_EDOMAIN
+        m.close()
+
+
+@pytest.mark.parametrize("skew,kurt", [(0.05, 0.05), (0.0, 0.05)])
+@pytest.mark.parametrize("sigma", [3.0, 9.9, 39.0])
+def test_gram_charlier_events_in_the_tails(sigma, skew, kurt):
+    s = empty(dataclasses.replace(line_spec(sigma, 900), resp_skew=skew, resp_kurt=kurt))
+    th = s.theta_true
+    reach = touched(s, th)
+    mo = O.expected(s, th)
+    bins = [b for b in far_bins(s, th, (5.5, 7.3, 8.5, 9.4)) if reach[b] and mo[b] > 0]
+    assert bins
+    for b in bins:
+        s.counts["sub"][:] = 0.0
+        s.counts["sub"][b] = 1.0
+        m = bx.Model(s, precision=bx.BX_FP64)
+        fo, go = O.nll(s, th, grad=True)
+        f, g = m.nll_grad(th)
+        assert 2 * abs(f - fo) <= 1e-7, (b, f, fo)
+        ok, worst = grad_ok(g, go, th)
+        assert ok, (b, worst)
+        m.close()
