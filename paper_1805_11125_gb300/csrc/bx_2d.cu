@@ -893,8 +893,8 @@ __global__ void __launch_bounds__(TP, 2) k_pile2d(Work w, int want_mu) {
             drain_add(tbase, (it & 1) * NSL, pu, true);      // summed in registers
         }
         tc_fence_before();
-        __syncthreads();
-        if (pp.abort) break;
+        // one vote for the block: a thread ahead of the others may set the flag again before they read it
+        if (__syncthreads_or(pp.abort)) break;
         if (fresh) {
             table(it + 1);
             if (tid == 0) multiply(it + 1);
@@ -1103,8 +1103,7 @@ __global__ void __launch_bounds__(TP, 2) k_corr2d(Work w) {
                     }
                 }
             }
-            __syncthreads();
-            if (pp.abort) break;
+            if (__syncthreads_or(pp.abort)) break;   // one vote for the block, as in k_pile2d
         }
         if (tid == 0) {
             if (!drain_copies(pp, waited, issued)) atomicOr(&pp.abort, 1);
