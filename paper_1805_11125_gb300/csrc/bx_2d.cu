@@ -1465,17 +1465,9 @@ __global__ void __launch_bounds__(128) k_gather2d(Work w, int n, double* nll_out
 // ------------------------------------------------------------------ launchers
 
 
-template <typename F>
-static cudaError_t set_smem(F* kern, size_t bytes, size_t& cached) {
-    if (bytes <= cached) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) cached = bytes;
-    return e;
-}
-
 // stage 1: templates and the forward GEMM; stage 2: pile-up and -lnL; stage 3: adjoint.
 cudaError_t launch_eval2d(const Work& w, int n, int want_grad, int want_mu, int stage, cudaStream_t s) {
-    static size_t c_fwd = 0, c_fwd_bf = 0, c_pile = 0, c_corr = 0, c_bwd = 0;
+    static SmemOptIn c_fwd, c_fwd_bf, c_pile, c_corr, c_bwd;
     cudaError_t e = cudaSuccess;
     if (stage == 1) {
         // the forward stage of one item: 174 us with one CTA here, 129 with eight
@@ -1484,21 +1476,21 @@ cudaError_t launch_eval2d(const Work& w, int n, int want_grad, int want_mu, int 
         const size_t sm = (size_t)(6 * A_FLOATS + 2 * TILE3_FLOATS) * 4 + 128;
         if (w.precision == BX_BF16X3) {
             k_trate<true><<<(unsigned)n * (unsigned)w.tr_kb, NSL * TRS<true>, 0, s>>>(w);
-            if ((e = set_smem(k_fwd2d<true>, sm, c_fwd_bf)) != cudaSuccess) return e;
+            if ((e = smem_opt_in(c_fwd_bf, k_fwd2d<true>, sm)) != cudaSuccess) return e;
             k_fwd2d<true><<<(unsigned)n * (unsigned)w.max_tiles, TF + 32, sm, s>>>(w);
         } else {
             k_trate<false><<<(unsigned)n * (unsigned)w.tr_kb, NSL * TRS<false>, 0, s>>>(w);
-            if ((e = set_smem(k_fwd2d<false>, sm, c_fwd)) != cudaSuccess) return e;
+            if ((e = smem_opt_in(c_fwd, k_fwd2d<false>, sm)) != cudaSuccess) return e;
             k_fwd2d<false><<<(unsigned)n * (unsigned)w.max_tiles, TF + 32, sm, s>>>(w);
         }
     } else if (stage == 2) {
-        if ((e = set_smem(k_pile2d, TP_SMEM, c_pile)) != cudaSuccess) return e;
+        if ((e = smem_opt_in(c_pile, k_pile2d, TP_SMEM)) != cudaSuccess) return e;
         k_pile2d<<<(unsigned)n * (unsigned)w.win_tiles, TP, TP_SMEM, s>>>(w, want_mu);
     } else if (stage == 3 && want_grad) {
-        if ((e = set_smem(k_corr2d, TP_SMEM, c_corr)) != cudaSuccess) return e;
+        if ((e = smem_opt_in(c_corr, k_corr2d, TP_SMEM)) != cudaSuccess) return e;
         k_corr2d<<<(unsigned)n * (unsigned)w.max_tiles, TP, TP_SMEM, s>>>(w);
         const size_t sb = (size_t)(6 * A_FLOATS + 2 * TILE_FLOATS + 3 * KMAX * NSL) * 4 + 128;
-        if ((e = set_smem(k_bwd2d, sb, c_bwd)) != cudaSuccess) return e;
+        if ((e = smem_opt_in(c_bwd, k_bwd2d, sb)) != cudaSuccess) return e;
         k_bwd2d<<<(unsigned)n * (unsigned)w.max_cb, T2 + 32, sb, s>>>(w);
     }
     return cudaGetLastError();

@@ -1590,16 +1590,6 @@ __global__ void __launch_bounds__(32) k_bwd64(Work w, int nch) {
 
 // ------------------------------------------------------------------ launchers
 
-// Dynamic shared memory beyond the default (48 KB less the kernel's static share): opted in once
-// per size, as the other assembly kernels do.
-template <typename F>
-static cudaError_t smem64(F* kern, size_t bytes, size_t& set) {
-    if (bytes <= 24 * 1024 || bytes <= set) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) set = bytes;
-    return e;
-}
-
 cudaError_t launch_prep64(const Work& w, int n, cudaStream_t s) {
     const int nblk = w.Npad / 128;
     k_scan64<<<(unsigned)n * nblk, 128, 0, s>>>(w, nblk);
@@ -1638,8 +1628,10 @@ cudaError_t launch_mid64(const Work& w, int n, int Mmax, int nwmax, int Lmax, in
     const int ntw = (nwmax + 31) / 32, ntm = (Mmax + 31) / 32;
     const size_t sp = (size_t)(2 * Lmax + 31) * sizeof(double);
     cudaError_t e;
-    static size_t set_pile = 0, set_corr = 0;
-    if ((e = smem64(k_pile64, sp, set_pile)) != cudaSuccess || (e = smem64(k_corr64, sp, set_corr)) != cudaSuccess) return e;
+    static SmemOptIn set_pile, set_corr;
+    if (sp > 24 * 1024 &&   // (the default limit is 48 KB with a kernel's static share)
+        ((e = smem_opt_in(set_pile, k_pile64, sp)) != cudaSuccess || (e = smem_opt_in(set_corr, k_corr64, sp)) != cudaSuccess))
+        return e;
     k_pile64<<<(unsigned)n * ntw * nH, 128, sp, s>>>(w, ntw, nH, want_grad, want_mu);
     k_marg64<<<n, MG, 0, s>>>(w, ntw, nH, want_grad, want_mu);
     if (want_grad) k_corr64<<<(unsigned)n * ntm * nH, 128, sp, s>>>(w, ntm, nH);

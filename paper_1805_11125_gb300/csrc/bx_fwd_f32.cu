@@ -554,14 +554,11 @@ __global__ void __launch_bounds__(32 * (SG + 2)) k_fwd_split(Work w) {
 
 template <bool TAG, bool COLS, bool MES>
 static cudaError_t fwd_split_variant(const Work& w, unsigned grid, cudaStream_t s) {
-    static size_t set[2] = {0, 0};   // opted in once per kernel
+    static SmemOptIn set[2];
     const int gc = w.gc ? 1 : 0;
     const auto k = gc ? k_fwd_split<TAG, COLS, MES, true> : k_fwd_split<TAG, COLS, MES, false>;
-    if (!set[gc]) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SplitShared));
-        if (e != cudaSuccess) return e;
-        set[gc] = sizeof(SplitShared);
-    }
+    const cudaError_t e = smem_opt_in(set[gc], k, sizeof(SplitShared));
+    if (e != cudaSuccess) return e;
     launch_chained(k, 2 * grid, 32 * (SG + 2), sizeof(SplitShared), s, w);
     return cudaGetLastError();
 }

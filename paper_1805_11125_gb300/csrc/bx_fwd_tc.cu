@@ -240,13 +240,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_fwd_tc(Work w) {
 }
 
 cudaError_t launch_fwd_tc(const Work& w, int n, int max_tiles, cudaStream_t s) {
-    const int smem = (int)sizeof(SmemTC) + 128;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    const size_t smem = sizeof(SmemTC) + 128;
+    static SmemOptIn set;
+    const cudaError_t e = smem_opt_in(set, k_fwd_tc, smem);
+    if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)n * (unsigned)w.max_tiles;   // decoded with w.max_tiles
     k_fwd_tc<<<grid, TC_THREADS, smem, s>>>(w);
     return cudaGetLastError();

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "bx.h"
+#include "bx_smem.h"
 
 namespace bx {
 
@@ -269,6 +270,17 @@ cudaError_t launch_mid64(const Work& w, int n, int Mmax, int nwmax, int Lmax, in
 cudaError_t launch_bwd64(const Work& w, int n, cudaStream_t s);
 cudaError_t mid64_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail);
 cudaError_t launch_fwd_tc(const Work& w, int n, int max_tiles, cudaStream_t s);
+// A kernel's dynamic shared memory on the current device: opted in once per device and size (also legal
+// while a stream is captured).
+template <typename F>
+cudaError_t smem_opt_in(SmemOptIn& done, F* kern, size_t bytes) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)done.ensure(dev, bytes, [&](size_t b) {
+        return (int)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+    });
+}
 // A kernel of an evaluation's chain, launched while the one before still runs: its blocks take their places
 // as that one's last blocks leave, and chain_wait() at its start waits for the whole of it (one
 // multivariate call 160 -> 151 us, 52 calls 249 -> 241; letting the blocks in from the start of the

@@ -922,25 +922,17 @@ cudaError_t mid_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t
 cudaError_t launch_mid(const Work& w, int n, int Mmax, int nwmax, int Lmax, int want_grad, int want_mu,
                        cudaStream_t s) {
     const size_t smem = mid_dynamic_smem(w, Mmax, nwmax, Lmax);
-    // the attribute is set once per size (outside any stream capture that replays it)
     if (w.precision == BX_TF32X3) {
-        static size_t set = 0;
-        if (smem > set) {
-            const cudaError_t e = cudaFuncSetAttribute(k_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            set = smem;
-        }
+        static SmemOptIn set;
+        const cudaError_t e = smem_opt_in(set, k_mid, smem);
+        if (e != cudaSuccess) return e;
         k_mid<<<n, MID_THREADS, smem, s>>>(w, want_grad, want_mu);
         return cudaGetLastError();
     }
-    static size_t set32[2] = {0, 0};
+    static SmemOptIn set32[2];
     const int mes = w.nes > 1 ? 1 : 0;   // several energy slices of the Eq. 4 terms
-    if (smem > set32[mes]) {
-        const cudaError_t e = cudaFuncSetAttribute(mes ? k_mid32<true> : k_mid32<false>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        set32[mes] = smem;
-    }
+    const cudaError_t e = smem_opt_in(set32[mes], mes ? k_mid32<true> : k_mid32<false>, smem);
+    if (e != cudaSuccess) return e;
     if (mes) launch_chained(k_mid32<true>, n, MID_THREADS, smem, s, w, want_grad, want_mu);
     else launch_chained(k_mid32<false>, n, MID_THREADS, smem, s, w, want_grad, want_mu);
     return cudaGetLastError();
