@@ -183,7 +183,8 @@ int bx_model_create(const bx_model_desc* descs, int n_toys, const bx_options* op
  * assembly stage would need more shared memory than the device allows a thread block: it
  * holds the window's spectra, the full axis of Eq. 3 spectra, the pile-up spectrum and the
  * per-column Eq. 4 weights.  On a GB300 that bounds e.g. an 8192-point grid to an axis of
- * about 2000 bins; the 1D limits above are the upper bounds of each size alone.) */
+ * about 2000 bins; the 1D limits above are the upper bounds of each size alone.  BX_FP64 has the
+ * limit 4 m_hi + 6 (m_hi - m_lo) + n_pileup <= 25962, each the largest of the model's toys.) */
 /* Several energy estimators of each dataset, fitted jointly (Sec. 3: the charge, the number of
  * detected photons and the number of fired channels are each an observable N_x with its own
  * response R_x of Eq. 1).  descs holds n_data x n_est descriptions, dataset-major: descs[t n_est + e]

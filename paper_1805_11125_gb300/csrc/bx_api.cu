@@ -509,14 +509,22 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
     w.ncs2d = m->ncs2d;
     if (!m->is2d) {   // the assembly stage holds one item's spectra and columns in shared memory
         size_t need = 0, avail = 0;
-        const cudaError_t e = m->precision == BX_FP64 ? mid64_smem_budget(w, m->Mmax, m->nwmax, m->Lmax, &need, &avail)
-                                                      : mid_smem_budget(w, m->Mmax, m->nwmax, m->Lmax, &need, &avail);
+        const bool f64 = m->precision == BX_FP64;
+        cudaError_t e = cudaSuccess;
+        if (f64) g64_size_limit(m->Mmax, m->nwmax, m->Lmax, &need, &avail);
+        else e = mid_smem_budget(w, m->Mmax, m->nwmax, m->Lmax, &need, &avail);
         const int bad = e != cudaSuccess ? 1 : need > avail ? 2 : 0;
         if (bad) {
             cudaStreamSynchronize(m->stream);
             const int nwm = m->nwmax, Mm = m->Mmax, Lm = m->Lmax, np = w.Npad;
             free_model(m);
             if (bad == 1) return bx_set_error(BX_ECUDA, "assembly kernel attributes: %s", cudaGetErrorString(e));
+            if (f64)
+                return bx_set_error(BX_EINVAL,
+                                    "window %d, axis %d and pile-up %d: an FP64 model's sizes are limited to %zu B of "
+                                    "spectra per item (a thread block's shared memory), these need %zu B: use a "
+                                    "smaller window, axis or pile-up spectrum",
+                                    nwm, Mm, Lm, avail, need);
             return bx_set_error(BX_EINVAL,
                                 "the assembly stage needs %zu B of shared memory per item (window %d, axis %d, "
                                 "pile-up %d, %d columns); the device allows %zu B: use a smaller window, axis, "

@@ -57,7 +57,6 @@ constexpr int RUN64 = 16;               // samples per exact start of the recurr
 constexpr int RUNB = 16;                // the same in the adjoint
 constexpr double HMAX = 0.2;            // largest spacing / sigma of a sampled column
 constexpr double HPOLY = 1.25;          // largest w / sigma of kind P (its polynomial's rest: poly_coef)
-constexpr size_t MID64_FIXED = 24688;   // shared memory set aside beside an item's spectra (mid64_smem_budget)
 constexpr double BAND_S = 8.0;          // band_sigmas of the sampled columns (the default)
 constexpr double ZRUN = 37.0;           // |z| of the runs of kind P: z^2 / 2 < 700 (exp_tab)
 constexpr int NPOLY = 16;               // kind P: terms of the bin-mass polynomial in z^2
@@ -1655,18 +1654,13 @@ cudaError_t launch_bwd64(const Work& w, int n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// The sizes an FP64 model takes: one item's spectra on the axis and the window and the pile-up
-// spectrum within a thread block's shared memory (the bound bx_model_create has always stated; the
-// kernels here need less).
-cudaError_t mid64_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail) {
-    (void)w;
-    *need = (size_t)(4 * Mmax + 6 * nwmax + Lmax) * sizeof(double) + 64;
-    int dev = 0, optin = 0;
-    cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-    *avail = (size_t)optin - MID64_FIXED;
-    return cudaSuccess;
+// The sizes an FP64 model takes: 4 values per axis bin, 6 per window bin and one per pile-up bin within
+// 207,696 bytes.  That is what the spectra of one item took of a thread block's shared memory while one
+// block assembled an item; the kernels here need only 2 L + 31 doubles, and the limit stands as a limit of
+// the interface.
+void g64_size_limit(int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail) {
+    *need = (size_t)(4 * Mmax + 6 * nwmax + Lmax) * sizeof(double);
+    *avail = 207696;
 }
 
 }  // namespace bx

@@ -268,7 +268,7 @@ cudaError_t launch_fwd64(const Work& w, int n, int any_tag, int any_cols, cudaSt
 cudaError_t launch_mid64(const Work& w, int n, int Mmax, int nwmax, int Lmax, int nH, int want_grad, int want_mu,
                          cudaStream_t s);
 cudaError_t launch_bwd64(const Work& w, int n, cudaStream_t s);
-cudaError_t mid64_smem_budget(const Work& w, int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail);
+void g64_size_limit(int Mmax, int nwmax, int Lmax, size_t* need, size_t* avail);
 cudaError_t launch_fwd_tc(const Work& w, int n, int max_tiles, cudaStream_t s);
 // A kernel's dynamic shared memory on the current device: opted in once per device and size (also legal
 // while a stream is captured).
