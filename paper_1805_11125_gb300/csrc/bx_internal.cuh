@@ -354,13 +354,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for the phase with the given parity; false when the time budget ran out.
 // First statement of the kernels launch_chained launches: wait for the kernel before (and with it for all
 // before that one); after a plain launch there is nothing to wait for.
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Wait for the phase with the given parity; false when the time budget ran out.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned long long budget_ns) {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer();
@@ -592,20 +592,6 @@ __device__ __forceinline__ float log1p_minus_x32(float x) {
     p = fmaf(s2, p, 2.0f / 5.0f);
     p = fmaf(s2, p, 2.0f / 3.0f);
     return fmaf(s2 * s, p, -(x * x) * r);
-}
-
-// Baker-Cousins term (mu - n) + n ln(n/mu) (n > 0) and its weight 1 - n/mu in FP32 for
-// x = (n - mu)/mu in [BC_XLO, BC_XHI] (every bin of a reasonable fit): written as
-// n (log1p(x) - x) + (n - mu) x, a sum of two terms within a factor ~3 of the result, so the
-// term carries an FP32 relative error with no systematic sign.  Other bins take the FP64
-// form.  Returns false outside the range.
-__device__ __forceinline__ bool bc_term32(double n, double mu, double& term, double& wb) {
-    const float d = (float)(n - mu);
-    const float x = d / (float)mu;
-    if (!(x >= BC_XLO && x <= BC_XHI)) return false;
-    term = (double)fmaf((float)n, log1p_minus_x32(x), d * x);
-    wb = (double)(-x);
-    return true;
 }
 
 // Shell integral of r^2 exp((r - r_iv)/lam): F and dF/dlam.

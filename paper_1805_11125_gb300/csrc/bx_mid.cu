@@ -12,9 +12,9 @@
 //          sum_k A_k p_k[rho] (closed-form shell integrals) and pulse-shape bins
 //          sum_k A_k q_k[j]; with several energy slices W_s of the window, one such
 //          marginal, radial and pulse-shape histogram per slice (G_W,s, aW_s, a_s);
-//   -lnL   sum of mu - n + n log1p((n - mu)/mu): in a cancellation-free FP32 form where
-//          mu/2 <= n <= 2 mu and in double-float elsewhere (FP64 beyond its range); the sum in FP64 with Neumaier compensation inside
-//          each thread (k_mid32: compensated FP32) and TwoSum-style merging across the block.
+//   -lnL   sum of mu - n + n log1p((n - mu)/mu): each term in double-float (FP64 beyond its
+//          range); the sum in FP64 with Neumaier compensation inside each thread (k_mid32:
+//          compensated FP32) and TwoSum-style merging across the block.
 // With want_grad it also writes the adjoint inputs of the response stage: per row the
 // pile-up-correlated residual weights wt_h[m] and G_W[m], per species the coefficients
 // that turn them into dNLL/dR[m,i], and the gradient of eps, s_r and the parts of the
