@@ -16,13 +16,13 @@
 // Every GEMM is M = 128 (output rows, or true-energy columns in the adjoint) x N = NSL x
 // K = 32 per k-block.  The A tile is generated by the CUDA cores into shared memory (the
 // response by the bias-free FP32 generator of bx_resp.cuh) or is a window of a table of the
-// pile-up kernel g (toeplitz_table), the B tile arrives by a bulk copy from a tile written by the previous stage.  The forward
+// pile-up kernel g (toeplitz_table), the B tile arrives by a bulk copy from a tile written by
+// the previous stage.  The forward
 // splits both operands in three (split3: an 8-bit hi on a grid shared by the k-block's
 // row or slice, then TF32 mid and lo), which makes the hi*hi products exact in the FP32
 // accumulator; the other GEMMs split into TF32 hi and lo, and one thread issues hi*lo,
-// lo*hi, then hi*hi (the small products
-// first: the tensor core's FP32 accumulation truncates, so the small terms are added while
-// the partial sum is still small).  The forward and the pile-up GEMMs drain their accumulator
+// lo*hi, then hi*hi (the small products first: the tensor core's FP32 accumulation truncates,
+// so the small terms are added while the partial sum is still small).  The forward and the pile-up GEMMs drain their accumulator
 // after every k-block and sum in registers, adding back each k-block's expected truncation
 // (trunc_comp), so that no systematic error of the accumulation reaches -lnL.
 // Every wait is bounded by the watchdog budget; on expiry the CTA records ERR_TIMEOUT,
@@ -305,7 +305,8 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w, int np) {
             df sk[KMAX];
 #pragma unroll
             for (int k = 0; k < KMAX; ++k)
-                sk[k] = k < K && i < T.N ? df{T.shapes32[(size_t)k * T.N + i], T.shapes32l[(size_t)k * T.N + i]} : df{0.f, 0.f};
+                sk[k] = k < K && i < T.N ? df{T.shapes32[(size_t)k * T.N + i], T.shapes32l[(size_t)k * T.N + i]}
+                                         : df{0.f, 0.f};
             for (int ss = 0; ss < 4; ++ss)
                 for (int c = 0; c < T.n_cls[ss]; ++c) {
                     df acc{0.f, 0.f};
@@ -334,7 +335,8 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w, int np) {
             if (last) {
                 __threadfence();
                 if (tid < 4 * KMAX)
-                    for (int q = 0; q < np; ++q) s_wmax[tid] = max(s_wmax[tid], (unsigned)__ldcg(&all[q * 4 * KMAX + tid]).x);
+                    for (int q = 0; q < np; ++q)
+                        s_wmax[tid] = max(s_wmax[tid], (unsigned)__ldcg(&all[q * 4 * KMAX + tid]).x);
                 if (tid == 0) w.prep_count[item] = 0;
                 __syncthreads();
             }
@@ -390,8 +392,8 @@ __global__ void __launch_bounds__(512) k_coef2d(Work w, int np) {
 }
 
 // T_r tiles of one item: grid = items x tr_kb k-blocks of 32 true-energy columns; thread =
-// slice b and a share of the k-block's columns (NSL x TRS threads).  T_r[i,b] = ut[i,b] sum_c q[b][c] W[set(b), c][i], with the class
-// sums W of k_coef2d, in double-float (split coefficients, shapes and modulation, TwoProduct by
+// slice b and a share of the k-block's columns (NSL x TRS threads).
+// T_r[i,b] = ut[i,b] sum_c q[b][c] W[set(b), c][i], with the class sums W of k_coef2d, in double-float (split coefficients, shapes and modulation, TwoProduct by
 // FMA, TwoSum): ~2^-44 relative instead of the FP32 roundings of every factor and partial sum,
 // which all the rows that T_r[i,b] meets in the GEMM would share, so that they would not average
 // out over a bin's sum.  It is split in three on one grid per slice (from k_coef2d's upper bound
@@ -806,8 +808,11 @@ __global__ void __launch_bounds__(TF + 32, 1) k_fwd2d(Work w) {
 // ------------------------------------------------------------------ pile-up + -lnL
 
 // Window tile t: rows m = m_lo + 128 t + 127 - l.  A[l, c] = g[m - m'] (input row m' = 32 kb + c, a
-// Toeplitz table), B = Y tiles; k-block it + 1 is multiplied into the other accumulator while it is drained; D = sum_d g[d] Y[m - d, b].  Epilogue: mu, the Baker-Cousins terms (cancellation-
-// free FP32 form where mu/2 <= n <= 2 mu, double-float otherwise; compensated sums), w = 1 - n/mu.
+// Toeplitz table), B = Y tiles; k-block it + 1 is multiplied into the other accumulator while it is
+// drained; D = sum_d g[d] Y[m - d, b].  Epilogue: mu, the Baker-Cousins terms (cancellation-free FP32
+// form where mu/2 <= n <= 2 mu, double-float otherwise; compensated sums), w = 1 - n/mu.  -lnL and the eps
+// derivative are sums over a thread's 32 slices of a row, then over the rows: their last bits follow that
+// order (chains of 64 slices, shared by two threads, cost 8 us of one item's 68 and 47 of 256 items' 624).
 __global__ void __launch_bounds__(TP, 2) k_pile2d(Work w, int want_mu) {
     extern __shared__ unsigned char smem_raw[];
     float* Ahi = align128(smem_raw);   // Toeplitz table of g, TP_KB k-blocks
@@ -1028,7 +1033,8 @@ __global__ void __launch_bounds__(TP, 2) k_pile2d(Work w, int want_mu) {
 // ------------------------------------------------------------------ adjoint of Eq. 2
 
 // Output rows m = 128 t + 127 - l over the whole axis; A[l, c] = g[(m_lo + j) - m] with window row
-// j = 32 kb + c (a Toeplitz table; the w tiles hold zeros beyond the window), B = w tiles; Wt = (1 - eps) w + eps D, stored as the adjoint's B tiles.
+// j = 32 kb + c (a Toeplitz table; the w tiles hold zeros beyond the window), B = w tiles;
+// Wt = (1 - eps) w + eps D, stored as the adjoint's B tiles.
 __global__ void __launch_bounds__(TP, 2) k_corr2d(Work w) {
     extern __shared__ unsigned char smem_raw[];
     float* Ahi = align128(smem_raw);   // Toeplitz table of g, TP_KB k-blocks
@@ -1454,7 +1460,8 @@ __global__ void __launch_bounds__(128) k_gather2d(Work w, int n, double* nll_out
     if (!st && j < T.P) {
         const int slot = j < T.K ? 5 + j : j < T.K + 5 ? j - T.K : j == T.K + 6 ? GPN : -1;
         // the column blocks' partials, or (eps) the window tiles'
-        const double* gp = slot >= 0 ? w.gpart2d + (size_t)item * MAX_CB * (GPN + 1) + slot : w.geps2d + (size_t)item * MAX_TILES;
+        const double* gp = slot >= 0 ? w.gpart2d + (size_t)item * MAX_CB * (GPN + 1) + slot
+                                     : w.geps2d + (size_t)item * MAX_TILES;
         const int np = slot >= 0 ? T.n_cb : nt, step = slot >= 0 ? GPN + 1 : 1;
 #pragma unroll 8
         for (int q = 0; q < np; ++q) g += gp[(size_t)q * step];

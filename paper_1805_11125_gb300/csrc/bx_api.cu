@@ -569,7 +569,7 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.chk64, sizeof(int2) * c64 * (w.Npad / 32) * (G64_NC + 1)},
         {(void**)&w.cmask64, sizeof(int) * c64},
         {(void**)&w.ap64, m->any_cols ? sizeof(double) * c64 * w.nslot64 * w.nes * w.Npad : 16},
-        {(void**)&w.F64, sizeof(double) * (f64 ? std::max((size_t)cap, (size_t)4 * std::min(cap, G64_SPLIT)) : 0) * 2 * w.gl64},
+        {(void**)&w.F64, sizeof(double) * std::max(c64, 4 * std::min(c64, (size_t)G64_SPLIT)) * 2 * w.gl64},
         {(void**)&w.mc64, m->any_cols ? sizeof(double) * c64 * (w.Npad / 32) * w.nes * 32 : 16},
         {(void**)&w.wt64, sizeof(double) * c64 * (2 + w.nes) * w.gl64},
         {(void**)&w.wv64, sizeof(double) * c64 * 2 * w.Mpad},
@@ -880,7 +880,8 @@ static int eval_host(bx_model* m, int n, const int* toy_idx, const double* theta
     }
     // A small call is bound by its copies and synchronisations: from a pinned buffer, and with the error
     // word, -lnL and the gradients as one block, it makes one copy each way and waits once (pageable
-    // copies wait one by one: one multivariate FP32 call 177 -> 158 us).  Larger calls go straight from and to the caller's arrays.
+    // copies wait one by one: one multivariate FP32 call 177 -> 158 us).  Larger calls go straight from
+    // and to the caller's arrays.
     const size_t nt = (size_t)n * P, nr = 1 + n + (grad && want_grad ? nt : 0);
     if (m->host_pin && nll && (nt + nr) * sizeof(double) <= HOST_PIN_BYTES) {
         double *pt = m->host_pin, *pr = pt + nt;

@@ -1477,7 +1477,8 @@ __global__ void __launch_bounds__(32) k_bwd64(Work w, int nch) {
                 if (__any_sync(0xffffffffu, isP))
                     for (int r0 = 0; r0 < ng; r0 += RUNB) {
                         // centres z, density p; edges ze = z - h/2 .., density pe (both over sqrt(2 pi))
-                        double z = (((double)(g0 + r0) + 0.5) * d - gen.x) * gen.y, ze = ((double)(g0 + r0) * d - gen.x) * gen.y;
+                        double z = (((double)(g0 + r0) + 0.5) * d - gen.x) * gen.y;
+                        double ze = ((double)(g0 + r0) * d - gen.x) * gen.y;
                         double p = exp_tab(-0.5 * z * z, sE), rho = exp_tab(-(z + 0.5 * h) * h, sE);
                         double pe = exp_tab(-0.5 * ze * ze, sE), re = exp_tab(-(ze + 0.5 * h) * h, sE);
 #pragma unroll 2
@@ -1628,9 +1629,10 @@ cudaError_t launch_mid64(const Work& w, int n, int Mmax, int nwmax, int Lmax, in
     const size_t sp = (size_t)(2 * Lmax + 31) * sizeof(double);
     cudaError_t e;
     static SmemOptIn set_pile, set_corr;
-    if (sp > 24 * 1024 &&   // (the default limit is 48 KB with a kernel's static share)
-        ((e = smem_opt_in(set_pile, k_pile64, sp)) != cudaSuccess || (e = smem_opt_in(set_corr, k_corr64, sp)) != cudaSuccess))
-        return e;
+    if (sp > 24 * 1024) {   // (the default limit is 48 KB with a kernel's static share)
+        if ((e = smem_opt_in(set_pile, k_pile64, sp)) != cudaSuccess) return e;
+        if ((e = smem_opt_in(set_corr, k_corr64, sp)) != cudaSuccess) return e;
+    }
     k_pile64<<<(unsigned)n * ntw * nH, 128, sp, s>>>(w, ntw, nH, want_grad, want_mu);
     k_marg64<<<n, MG, 0, s>>>(w, ntw, nH, want_grad, want_mu);
     if (want_grad) k_corr64<<<(unsigned)n * ntm * nH, 128, sp, s>>>(w, ntm, nH);

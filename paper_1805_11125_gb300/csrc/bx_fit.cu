@@ -446,7 +446,8 @@ __global__ void __launch_bounds__(32) k_fit(FitDev F) {
             const unsigned mn = __ballot_sync(0xffffffffu, noise);
             if (noise) {
                 const double h = up - th[jl];
-                sh.res[ne + __popc(mn & ((1u << lane) - 1u))] = 0.5 * fabs(ep + em - 2.0 * fcur - sh.H[SIDX(jl, jl)] * h * h);
+                sh.res[ne + __popc(mn & ((1u << lane) - 1u))] =
+                    0.5 * fabs(ep + em - 2.0 * fcur - sh.H[SIDX(jl, jl)] * h * h);
             }
             ne += __popc(mn);
         }
@@ -607,7 +608,8 @@ __global__ void __launch_bounds__(32) k_fit(FitDev F) {
                     }
                     for (int k = 0; k < NLS; ++k) {
                         const double a = ldexp(1.0, -k);
-                        slot_t(k)[i] = sh.fr[i] ? fmin(fmax(th[i] + fmin(fmax(a * sh.d[i], -lim), lim), lo[i]), hi[i]) : th[i];
+                        slot_t(k)[i] =
+                            sh.fr[i] ? fmin(fmax(th[i] + fmin(fmax(a * sh.d[i], -lim), lim), lo[i]), hi[i]) : th[i];
                     }
                 }
                 for (int k = lane; k < S; k += 32) F.skip[s0 + k] = k < NLS ? 0 : 1;

@@ -347,8 +347,12 @@ struct SplitShared {
     float P[SG][FCH32 / 2][SPW];
     float gg[MAX_ES][64];             // Gg_s of the rows
 };
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_sync(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
 
 template <bool TAG, bool COLS, bool MES, bool GC>
 __global__ void __launch_bounds__(32 * (SG + 2)) k_fwd_split(Work w) {
@@ -422,7 +426,8 @@ __global__ void __launch_bounds__(32 * (SG + 2)) k_fwd_split(Work w) {
     const float mfa = (float)(g0 + lane), mfb = (float)(g0 + lane + 32);
     const float gc3 = GC ? (float)T.gc1 : 0.f, gc4 = GC ? (float)T.gc2 : 0.f;
     auto shape = [&](bool wide, float th, float tl, const ColG& cg) {
-        if constexpr (GC) return wide ? resp_shape32_gc_t<true>(th, tl, cg, gc3, gc4) : resp_shape32_gc_t<false>(th, tl, cg, gc3, gc4);
+        if constexpr (GC)
+            return wide ? resp_shape32_gc_t<true>(th, tl, cg, gc3, gc4) : resp_shape32_gc_t<false>(th, tl, cg, gc3, gc4);
         else return wide ? resp_shape32_t<true>(th, tl, cg) : resp_shape32_t<false>(th, tl, cg);
     };
     const size_t cbase = (size_t)item * w.Npad;

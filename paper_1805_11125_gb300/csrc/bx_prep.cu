@@ -174,7 +174,8 @@ __device__ void block_scan_df(df& a, df& b, df& ta, df& tb, float* sh) {
 template <bool MULTI, bool GC, bool SHELL, bool PARTS>
 __global__ void __launch_bounds__(256, 3) k_prep32(Work w, int np) {
     const int nparts = PARTS ? np : 1;
-    const int item = PARTS ? blockIdx.x / nparts : blockIdx.x, part = PARTS ? blockIdx.x % nparts : 0, tid = threadIdx.x, lane = tid & 31;
+    const int item = PARTS ? blockIdx.x / nparts : blockIdx.x, part = PARTS ? blockIdx.x % nparts : 0;
+    const int tid = threadIdx.x, lane = tid & 31;
     if (w.skip && w.skip[item]) {
         if (tid == 0 && part == 0) w.status[item] = STATUS_SKIPPED;
         return;
@@ -487,7 +488,8 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w, int np) {
     }
     if (PARTS) {   // this part's ranges out; the last part of the item merges them
         int2* mine = w.prep_part + ((size_t)item * PREP_PARTS + part) * (MAX_SETS * MAX_TILES + 1);
-        for (int j = tid; j < nt; j += blockDim.x) mine[j] = make_int2(s_tlo[j / MAX_TILES][j % MAX_TILES], s_thi[j / MAX_TILES][j % MAX_TILES]);
+        for (int j = tid; j < nt; j += blockDim.x)
+            mine[j] = make_int2(s_tlo[j / MAX_TILES][j % MAX_TILES], s_thi[j / MAX_TILES][j % MAX_TILES]);
         if (tid == 0) mine[MAX_SETS * MAX_TILES] = make_int2(s_bad, 0);
         __threadfence();
         __syncthreads();
@@ -508,7 +510,8 @@ __global__ void __launch_bounds__(256, 3) k_prep32(Work w, int np) {
         }
         if (tid == 0) {
             int any = 0;
-            for (int q = 0; q < nparts; ++q) any |= __ldcg(&all[(size_t)q * (MAX_SETS * MAX_TILES + 1) + MAX_SETS * MAX_TILES]).x;
+            for (int q = 0; q < nparts; ++q)
+                any |= __ldcg(&all[(size_t)q * (MAX_SETS * MAX_TILES + 1) + MAX_SETS * MAX_TILES]).x;
             w.status[item] = any ? (int)BX_EDOMAIN : 0;
             w.prep_count[item] = 0;   // for the next evaluation
         }

@@ -107,8 +107,8 @@ __device__ __forceinline__ void centre_step2(f2 th, f2 tl, const ColPair& k, f2 
 // resp_shape32_t<true> of two columns at two rows (th, tl) and (uh, ul).  The scalar form's values
 // to the last bit, in fewer operations: with q = th^2 + ql the reduced argument is taken negated,
 // -f = (q + n) + ql (odd polynomial coefficients negated), the polynomial is that of 8 x 2^f (exact), so
-// that the node weights become 5/8 and 1, and 2^n is added to the exponent field.  |t| <= 11 (the caller checks it) keeps the result
-// normal and exp2_neg's clamp out of reach.
+// that the node weights become 5/8 and 1, and 2^n is added to the exponent field.  |t| <= 11 (the caller
+// checks it) keeps the result normal and exp2_neg's clamp out of reach.
 __device__ __forceinline__ void resp_shape32_x4(const ColPair& k, f2 th, f2 tl, f2 uh, f2 ul, f2& R0, f2& R1) {
     const f2 magic = f2_dup(12582912.0f);
     const f2 nth = f2_neg(th), nuh = f2_neg(uh);
