@@ -575,7 +575,8 @@ static int model_create(const bx_model_desc* descs, int n_toys, const bx_options
         {(void**)&w.wv64, sizeof(double) * c64 * 2 * w.Mpad},
         {(void**)&w.ctile64, sizeof(uint2) * c64 * (w.Npad / 32)},
         {(void**)&w.tmask64, sizeof(unsigned long long) * c64},
-        {(void**)&w.rows64, sizeof(unsigned) * c64 * 2 * 3 * (w.Mpad / 32)},
+        {(void**)&w.rows64, sizeof(unsigned) * c64 * 2 * 2 * (w.Mpad / 32)},
+        {(void**)&w.top64, sizeof(int) * c64 * 2 * MAX_TILES},
         {(void**)&w.xany64, sizeof(int) * c64},
         {(void**)&w.xw64, sizeof(double) * c64 * 2 * w.Mpad},
         {(void**)&w.part64, sizeof(double) * c64 * 2 * ((m->nwmax + 31) / 32) * 4},

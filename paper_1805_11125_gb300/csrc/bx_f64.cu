@@ -13,11 +13,11 @@
 // 160 - 640 at w = 1 npe).  Down a column the samples follow by a recurrence (two multiplications
 // each) from an exact start every RUN64 samples.
 // A column contributes to every bin of the 128-bin tiles that its band (8 sigma) touches and to no other
-// tile; its samples end one sigma past the band.  The stencil is good to about 1e-17 of the largest
-// sample it meets, so a bin with content nearby is known to 1e-14 of itself: up to 4.6 sigma from the
-// nearest column at a spacing of 0.2 sigma, 7 sigma at 0.1.  In the tails beyond (k_lam64 marks them) the
-// bins whose counts matter relative to themselves -- those with an event, and the expected counts a
-// caller asks for -- take the exact bin masses of their tile's columns (tail_bins, tail_adjoint).
+// tile; its samples end one sigma past the band.  A bin with content within about 3.5 sigma is known to
+// 1e-14 of itself (the stencil is good to 1e-17 of the largest sample it meets, the columns that end before
+// the bin are below 4e-15 of it).  In the tails beyond (k_lam64 marks them) the error of lambda is bounded,
+// and the bins whose expected count needs better -- those with an event, and the expected counts a caller
+// asks for -- take the exact bin masses of their tile's columns (tail_bins, tail_adjoint).
 // Columns too narrow for that (h > 0.2 at d = w) form class CI on the bins themselves, each entry
 // the exact bin mass: phi(z) times a polynomial in z^2 (kind P, sigma >= 0.8 w), or the difference of
 // erfc tails (kind D: narrower still, or a narrow Gram-Charlier column).  Any band_sigmas but the
@@ -661,17 +661,17 @@ __device__ void marg_chunk(const Work& w, const Toy& T, int item, int chunk) {
     }
 }
 
-// Rows of bits per bin of one spectrum's axis (k_lam64 writes all three).
-enum { ROWS_TAIL = 0, ROWS_STRONG = 1, ROWS_EXACT = 2, ROWS_N = 3 };
+// Rows of bits per bin of one spectrum's axis (k_lam64 writes both).
+enum { ROWS_TAIL = 0, ROWS_EXACT = 1, ROWS_N = 2 };
 __device__ __forceinline__ unsigned* bin_rows(const Work& w, int item, int h, int which) {
     return w.rows64 + (((size_t)item * 2 + h) * ROWS_N + which) * (w.Mpad / 32);
 }
 __device__ __forceinline__ bool row_bit(const unsigned* r, int m) { return (r[m >> 5] >> (m & 31)) & 1u; }
 // A bin in the tails of everything near it: below 2^-TAIL_BITS of the largest sample that its stencils
-// meet (top: that sample's exponent word).  The stencil is good to about 1e-17 of that sample: to 1e-14
-// of a bin above the line (4.6 to 7 sigma from the columns, for spacings of 0.2 to 0.1 sigma), and no
-// longer at the end of the samples.
-constexpr int TAIL_BITS = 14, STRONG_BITS = 3;
+// meet (top: that sample's exponent word).  That is from 3.1 to 3.9 sigma past the last column, for
+// spacings of 0.2 to 0.1 sigma.  Nearer, the columns that end before the bin (9 sigma) are below 4e-15 of
+// it and the stencil is good to 2e-16; at 6 sigma these are 1e-10 and 9e-14 (a dense spectrum).
+constexpr int TAIL_BITS = 7;
 __device__ __forceinline__ bool in_tail(double v, int top) {
     const int e = __double2hiint(v);
     return e <= top - (TAIL_BITS << 20) || e < (40 << 20);
@@ -679,7 +679,7 @@ __device__ __forceinline__ bool in_tail(double v, int top) {
 
 // lambda_h[m]: the stencil of bin m's phase over each class's samples around its cell, plus CI.  A
 // bin no column's samples reach (every class's own cell empty) and a tile that no column's band touches
-// are exactly 0; the bins in the tails of a touched tile are marked for k_pile64.  The
+// are exactly 0; the bins in the tails are marked for k_pile64 (the bins of such a tile too).  The
 // first nrb CTAs of an item do that; the others take the marginal sums of four chunks each.
 // nplane: the forward's partial planes (small batches), added in the order of its four warps.
 template <bool TAG>
@@ -772,13 +772,13 @@ __global__ void __launch_bounds__(128) k_lam64(Work w, int nrb, int nall, int np
             if (m < M) w.lam[((size_t)item * 2 + h) * w.Mpad + m] = any[h] ? lam[h] : 0.0;
         return;
     }
-    bool tail = false, strong[H];
+    bool tail = false;
 #pragma unroll
     for (int h = 0; h < H; ++h) {
         lam[h] = m < M && any[h] && touched ? lam[h] : 0.0;
         if (m < M) w.lam[((size_t)item * 2 + h) * w.Mpad + m] = lam[h];
-        strong[h] = __double2hiint(lam[h]) >= max(top[h] - (STRONG_BITS << 20), 40 << 20);
-        tail |= m < M && touched && in_tail(lam[h], top[h]);
+        if (threadIdx.x == 0) w.top64[((size_t)item * 2 + h) * MAX_TILES + blk] = top[h];
+        tail |= m < M && in_tail(lam[h], top[h]);
     }
     // the largest of all samples staged bounds each bin's; only where that leaves a doubt, its own
     const bool doubt = __syncthreads_or(tail);
@@ -800,11 +800,9 @@ __global__ void __launch_bounds__(128) k_lam64(Work w, int nrb, int nall, int np
     }
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-        const unsigned bt = __ballot_sync(0xffffffffu, doubt && m < M && touched && in_tail(lam[h], top[h]));
-        const unsigned bs = __ballot_sync(0xffffffffu, strong[h]);
+        const unsigned bt = __ballot_sync(0xffffffffu, doubt && m < M && in_tail(lam[h], top[h]));
         if ((threadIdx.x & 31) == 0) {
             bin_rows(w, item, h, ROWS_TAIL)[m >> 5] = bt;
-            bin_rows(w, item, h, ROWS_STRONG)[m >> 5] = bs;
             bin_rows(w, item, h, ROWS_EXACT)[m >> 5] = 0u;
         }
     }
@@ -875,33 +873,162 @@ __device__ double exact_bin(const Work& w, const Toy& T, int item, int h, int m,
     return sum;
 }
 
-// Data in the tails (ev: bins of this CTA's 32 with an event, or all of them for the expected counts).
-// Those bins' own lambda is replaced by exact_bin's; and, unless their pile-up comes from well within the
-// columns (a strong bin at a shift with at least 1 % of the largest g: the tails then enter below 1e-12),
-// that of every tail bin within the reach of g.  The bins are marked for the adjoint.
-__device__ __noinline__ void tail_bins(const Work& w, const Toy& T, int item, int h, unsigned ev, int m0, int Lt,
-                                       const double* sg, double* sx) {
-    __shared__ unsigned s_need[(MAX_L + 32) / 32 + 1];
-    __shared__ double s_red[4];
-    const int tid = threadIdx.x, nrow = 32 + Lt - 1;
-    const unsigned *tail = bin_rows(w, item, h, ROWS_TAIL), *strong = bin_rows(w, item, h, ROWS_STRONG);
-    double gm = 0.0;
-    for (int d = tid; d < Lt; d += 128) gm = fmax(gm, sg[d]);
+// log2 of a positive normal number, to FP32's precision (its range may exceed FP32's).
+__device__ __forceinline__ float log2_f64(double x) {
+    const int hi = __double2hiint(x);
+    return (float)((hi >> 20) - 1023) + log2f((float)__hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(x)));
+}
+
+// How far the stencil's lambda may be off in 32 bins (lane b: bin m, if on; the same in each of the block's
+// four warps), over a count whose log2 is lm (l2max: log2 of more than any column's largest bin).  Summed
+// over the columns in FP32: whole, a column whose samples end before the bin (9 sigma) or that does not touch
+// its tile (its samples go one sigma past its band); of any column the stencil's 1e-17 of the density 2.3
+// sigma nearer; and, where the stencil reaches past the end of the samples, 0.04 of the density there, 2^-4
+// less per sigma (bounds of the errors in 40 digits at spacings of 0.1 to 0.2 sigma, from 3 sigma on).
+// Columns below 2^-70 of every count are passed over; 2000 columns take a few us, an exact bin mass of every
+// column that matters 12 us a bin.
+__device__ float tail_error(const Work& w, const Toy& T, int item, int h, bool on, int m, float lm, float l2max) {
+    __shared__ float s_err[4][32];
+    const int tid = threadIdx.x, lane = tid & 31, part = tid >> 5;
+    const float wf = (float)T.w, y = ((float)m + 0.5f) * wf;
+    const int tile = m / TM;
+    float ylo = on ? y : 3.0e38f, yhi = on ? y : -3.0e38f, lmin = on ? lm : 3.0e38f;   // (of all warps alike)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
-    if ((tid & 31) == 0) s_red[tid >> 5] = gm;
-    for (int q = tid; q <= nrow / 32; q += 128) s_need[q] = 0u;
-    __syncthreads();
-    gm = 0.01 * fmax(fmax(s_red[0], s_red[1]), fmax(s_red[2], s_red[3]));
-    for (unsigned e = ev; e; e &= e - 1u) {
-        const int b = __ffs(e) - 1, m = m0 + b, Lb = min(Lt, m + 1), q0 = Lt - 1 + b;   // sx[q0]: the bin
-        bool lit = false;
-        for (int d = 1 + tid; d < Lb; d += 128) lit |= sg[d] >= gm && row_bit(strong, m - d);
-        const bool own = __syncthreads_or(lit);
-        for (int d = tid; d < (own ? 1 : Lb); d += 128)
-            if (row_bit(tail, m - d)) atomicOr(&s_need[(q0 - d) >> 5], 1u << ((q0 - d) & 31));
+    for (int o = 16; o > 0; o >>= 1) {
+        ylo = fminf(ylo, __shfl_xor_sync(0xffffffffu, ylo, o));
+        yhi = fmaxf(yhi, __shfl_xor_sync(0xffffffffu, yhi, o));
+        lmin = fminf(lmin, __shfl_xor_sync(0xffffffffu, lmin, o));
+    }
+    auto score = [&](float gap, float isig) { return fmaxf((gap - 0.5f * wf) * isig, 0.f); };
+    auto near = [&](float mu, float isig) {   // 2.3 sigma nearer than the nearest of the bins
+        return fmaxf(score(fmaxf(fmaxf(ylo - mu, mu - yhi), 0.f), isig) - 2.3f, 0.f);
+    };
+    // the warp's groups of 32 columns with one near enough (loads of several groups in flight)
+    unsigned long long todo = 0ull;
+    const Gen64* gen64 = w.gen64 + (size_t)item * w.Npad;
+    const int ng = (T.Next + 127 - 32 * part) / 128;
+#pragma unroll 8
+    for (int g = 0; g < ng; ++g) {
+        const int ie = min(g * 128 + part * 32 + lane, T.Next - 1);
+        const double2 ms = *reinterpret_cast<const double2*>(gen64 + ie);   // mean, 1 / sigma
+        const float zl = near((float)ms.x, (float)ms.y);
+        if (__any_sync(0xffffffffu, l2max - 0.72134752f * zl * zl - lmin > -13.f)) todo |= 1ull << g;
+    }
+    float err = 0.f;
+    for (; todo; todo &= todo - 1ull) {   // lane: a column, then each live column for 32 bins
+        const int ie = (__ffsll((long long)todo) - 1) * 128 + part * 32 + lane;
+        float mu = 0.f, isig = 0.f, l2 = -3.0e38f;   // l2: log2 of the bin mass at the mean
+        int tiles = 0;   // first and last tile that the column touches
+        if (ie < T.Next) {
+            const size_t at = (size_t)item * w.Npad + ie;
+            const double2 S2 = w.colS[at];
+            const Gen64 gen = gen64[ie];
+            const Col64 cc = w.col64[at];
+            const double S = fabs(h ? S2.y : S2.x), norm = cc.norm;
+            mu = (float)gen.x;
+            isig = (float)gen.y;
+            if (w.colc64[at].x >= 0 && S > 0.0)
+                l2 = log2_f64(S) + log2f((float)norm / (float)gen.w * isig * wf * 0.39894228f);
+            int r0, r1;
+            near_bins(cc.mu, cc.sig, T.w, T.M, (float)w.band, r0, r1);
+            tiles = (r0 / TM) << 16 | (max(r1 - 1, 0) / TM);
+        }
+        const float zl = near(mu, isig);
+        unsigned live = __ballot_sync(0xffffffffu, l2 - 0.72134752f * zl * zl - lmin > -13.f);
+        for (; live; live &= live - 1u) {
+            const int q = __ffs(live) - 1;   // (1e-17 of it: 2^-70)
+            const float kx = __shfl_sync(0xffffffffu, mu, q), ky = __shfl_sync(0xffffffffu, isig, q);
+            const float top = __shfl_sync(0xffffffffu, l2, q) - lm;
+            const int kt = __shfl_sync(0xffffffffu, tiles, q);
+            const float z = score(fabsf(y - kx), ky), zn = fmaxf(z - 2.3f, 0.f);
+            err = fmaf(1e-17f, exp2f(fmaf(-0.72134752f * zn, zn, top)), err);
+            if (z > 5.7f) {
+                const bool out = z > 8.9f || tile < kt >> 16 || tile > (kt & 0xffff);
+                err += exp2f(out ? fmaf(-0.72134752f * z, z, top) : top - 63.1f - 4.f * (9.f - z));
+            }
+        }
     }
     __syncthreads();
+    s_err[part][lane] = err;
+    __syncthreads();
+    return (s_err[0][lane] + s_err[1][lane]) + (s_err[2][lane] + s_err[3][lane]);
+}
+
+// Data in the tails: the lambdas (in sx) that those bins' expected counts (mu, from the stencils' values)
+// need better are replaced by exact_bin's and marked for the adjoint; whether there were any.  No lambda
+// of the reach is further off than 1.7e-17 of the largest density within 10 sigma of it (a column at the
+// end of its samples; what columns have in a tile next to those they touch counts against a bin's own lambda
+// only).  A bin for which that is below 1e-12 needs nothing; if it is for the tails in its
+// reach (nearly every bin with pile-up from the columns themselves), at most its own lambda; the reach of
+// any other bin is looked through.
+__device__ __noinline__ bool tail_bins(const Work& w, const Toy& T, int item, int h, unsigned ev, int m0, int Lt,
+                                       double eps, const double* sg, double* sx, const double* mu) {
+    __shared__ unsigned s_need[(MAX_L + 32) / 32 + 1];
+    __shared__ double s_red[4];
+    const int tid = threadIdx.x, lane = tid & 31, nrow = 32 + Lt - 1;
+    const unsigned* tail = bin_rows(w, item, h, ROWS_TAIL);
+    const unsigned long long touched = w.tmask64[item];   // (lambda is exactly 0 in the other tiles)
+    double gs = 0.0;
+    for (int d = tid; d < Lt; d += 128) gs += fabs(sg[d]);
+    gs = warp_sum(gs);
+    if (lane == 0) s_red[tid >> 5] = gs;
+    for (int q = tid; q <= nrow / 32; q += 128) s_need[q] = 0u;
+    int top = 0;   // class c: sigma below 10 2^c bins (the last class: any)
+    {
+        const int cm = w.cmask64[item] & ((1 << G64_NC) - 1), c = 31 - __clz(cm | 1);
+        const int R = c == G64_NC - 1 ? T.M : 100 << c;
+        int first = INT_MAX;   // tail of the reach, in whole words of 32 bins
+        for (int q = max(m0 - (Lt - 1), 0) / 32 + lane; q * 32 < min(m0 + 32, T.M); q += 32)
+            if (tail[q] && ((touched >> (q * 32 / TM)) & 1ull)) first = min(first, q * 32);
+        first = __reduce_min_sync(0xffffffffu, first);
+        const int t0 = max(min(first, m0) - R, 0) / TM, t1 = min(m0 + 32 + R, T.M - 1) / TM;
+        for (int t = t0 + lane; t <= t1; t += 32) top = max(top, w.top64[((size_t)item * 2 + h) * MAX_TILES + t]);
+        top = __reduce_max_sync(0xffffffffu, top);
+    }
+    __syncthreads();
+    gs = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
+    // (the Gram-Charlier density at 9 sigma is this much more than the Gaussian's)
+    const double gcf = 1.0 + 702.0 * fabs(T.gc1) + 6078.0 * fabs(T.gc2);
+    const double bound = 1.7e-5 * gcf * __hiloint2double(top + (1 << 20), 0), reach = bound * fabs(eps) * gs;
+    const float tol = (float)(1e-14 / gcf);   // of a bin's expected count
+    // (no count: no error is small enough)
+    auto log2_mu = [&](int b) { return mu[b] > 1e-290 ? log2_f64(mu[b]) : -3.0e38f; };
+    ev &= ~__ballot_sync(0xffffffffu, mu[lane] >= bound + reach);   // (a bin's own lambda is as good)
+    if (!ev) return false;
+    int all = 0;   // the largest sample of any tile (and 2^40 of it: a column's mean may lie off the axis)
+    for (int t = lane; t * TM < T.M; t += 32) all = max(all, w.top64[((size_t)item * 2 + h) * MAX_TILES + t]);
+    const float l2max = (float)((__reduce_max_sync(0xffffffffu, all) >> 20) - 1023) + 40.f;
+    const unsigned own = ev & __ballot_sync(0xffffffffu, mu[lane] >= reach && mu[lane] > 1e-290);
+    unsigned any = 0u;
+    if (own) {
+        const bool on = (own >> lane) & 1u;
+        const float err = tail_error(w, T, item, h, on, m0 + lane, log2_mu(lane), l2max);
+        any = __ballot_sync(0xffffffffu, on && !(err <= tol));
+        if (tid < 32 && ((any >> lane) & 1u)) atomicOr(&s_need[(Lt - 1 + lane) >> 5], 1u << ((Lt - 1 + lane) & 31));
+    }
+    if (ev & ~own) {
+        float lm0 = 3.0e38f;   // the smallest of their counts
+        for (unsigned e = ev & ~own; e; e &= e - 1u) lm0 = fminf(lm0, log2_mu(__ffs(e) - 1));
+        for (int q0 = 0; q0 < nrow; q0 += 32) {   // the bins of sx, 32 at a time
+            const int q = q0 + lane, mq = m0 - (Lt - 1) + q;
+            const bool on = q < nrow && mq >= 0 && mq < T.M && ((touched >> (mq / TM)) & 1ull) && row_bit(tail, mq);
+            if (!__syncthreads_or(on)) continue;
+            const float err = tail_error(w, T, item, h, on, mq, lm0, l2max);
+            bool need = false;
+            for (unsigned e = ev & ~own; e; e &= e - 1u) {
+                const int b = __ffs(e) - 1, d = Lt - 1 + b - q;   // its shift, and its weight in mu
+                if (on && d >= 0 && d < Lt) {
+                    const double c = fabs(eps * sg[d] + (d == 0 ? 1.0 - eps : 0.0));
+                    need |= c > 0.0 && !(err * exp2f(lm0 - log2_mu(b)) * (float)c <= tol);
+                }
+            }
+            const unsigned bits = __ballot_sync(0xffffffffu, need);
+            if (tid == 0) s_need[q0 >> 5] |= bits;
+            any |= bits;
+        }
+    }
+    __syncthreads();
+    if (!any) return false;
     for (int q0 = 0; q0 < nrow; q0 += 32)
         for (unsigned r = s_need[q0 >> 5]; r; r &= r - 1u) {
             const int q = q0 + __ffs(r) - 1, m = m0 - (Lt - 1) + q;
@@ -913,6 +1040,7 @@ __device__ __noinline__ void tail_bins(const Work& w, const Toy& T, int item, in
             }
         }
     __syncthreads();
+    return true;
 }
 
 // The adjoint of the bins that tail_bins took (their row weights xw64 are not in rowW), for one column:
@@ -949,7 +1077,9 @@ __device__ __noinline__ void tail_adjoint(const Work& w, const Toy& T, int item,
 // ------------------------------------------------------------------ assembly
 
 // CTA = 32 window bins of one spectrum of one item, a warp per quarter of the taps: Eq. 2, the
-// Baker-Cousins terms, w = 1 - n/mu, and the tile's part of -lnL (compensated) and of d/deps.
+// Baker-Cousins terms, w = 1 - n/mu, and the tile's part of -lnL (compensated) and of d/deps.  With an
+// event in the tails the sum is taken again if tail_bins changed a lambda (100 toys: 155 -> 172 us; the
+// bound of 10 CTAs keeps the registers at 48, 47 without the tails).
 __global__ void __launch_bounds__(128, 10) k_pile64(Work w, int ntw, int nH, int want_grad, int want_mu) {
     extern __shared__ __align__(16) double dsm[];
     const int t = blockIdx.x % ntw, h = (blockIdx.x / ntw) % nH, item = blockIdx.x / (ntw * nH), tid = threadIdx.x;
@@ -977,23 +1107,30 @@ __global__ void __launch_bounds__(128, 10) k_pile64(Work w, int ntw, int nH, int
         if (e) e = want_mu || T.cnt[(size_t)h * nw + j] != 0.0;
         ev = __ballot_sync(0xffffffffu, e);
     }
-    __shared__ double sc[3][32];
+    __shared__ double sc[4][32];
     __syncthreads();
-    if (ev) tail_bins(w, T, item, h, ev, m0, Lt, sg, sx);
     const int d0 = min(Lt, pt * pl), d1 = min(Lt, d0 + pl);
     const double* x = sx + (Lt - 1) + b;
-    double c0 = 0.0, c1 = 0.0;
-    int d = d0;
+    double cv = 0.0;
+    for (;;) {
+        double c0 = 0.0, c1 = 0.0;
+        int d = d0;
 #pragma unroll 4
-    for (; d + 1 < d1; d += 2) {
-        c0 = fma(sg[d], x[-d], c0);
-        c1 = fma(sg[d + 1], x[-d - 1], c1);
+        for (; d + 1 < d1; d += 2) {
+            c0 = fma(sg[d], x[-d], c0);
+            c1 = fma(sg[d + 1], x[-d - 1], c1);
+        }
+        if (d < d1) c0 = fma(sg[d], x[-d], c0);
+        if (pt) sc[pt - 1][b] = c0 + c1;
+        __syncthreads();
+        if (pt == 0) cv = ((c0 + c1) + sc[0][b]) + (sc[1][b] + sc[2][b]);
+        if (!ev) break;
+        if (pt == 0) sc[3][b] = (1.0 - eps) * x[0] + eps * cv;
+        __syncthreads();
+        if (!tail_bins(w, T, item, h, ev, m0, Lt, eps, sg, sx, sc[3])) break;
+        ev = 0u;   // once more with the better values
     }
-    if (d < d1) c0 = fma(sg[d], x[-d], c0);
-    if (pt) sc[pt - 1][b] = c0 + c1;
-    __syncthreads();
     if (pt) return;
-    const double cv = ((c0 + c1) + sc[0][b]) + (sc[1][b] + sc[2][b]);
     bool dom = false;
     Neu acc{0.0, 0.0};
     double geps = 0.0;

@@ -208,7 +208,8 @@ struct Work {
     double* part64;           // [cap][2 * window tiles][4]: -lnL sum and compensation, d/deps, domain flag
     uint2* ctile64;           // [cap][Npad/32]: tiles of 128 bins that the chunk's bands touch (bits)
     unsigned long long* tmask64;   // [cap]: the same of all columns
-    unsigned* rows64;         // [cap][2][3][Mpad/32]: bits per bin (in the tails, strong, taken exactly)
+    unsigned* rows64;         // [cap][2][2][Mpad/32]: bits per bin (in the tails, taken exactly)
+    int* top64;               // [cap][2][MAX_TILES]: exponent word of the largest sample of each tile, per bin
     int* xany64;              // [cap]: some bin was taken exactly
     double* xw64;             // [cap][2][Mpad]: row weights of the bins taken exactly
     int nslot64, gl64, wt_threads64;

@@ -306,3 +306,49 @@ def test_gram_charlier_events_in_the_tails(sigma, skew, kurt):
         ok, worst = grad_ok(g, go, th)
         assert ok, (b, worst)
         m.close()
+
+
+# ---- a spectrum that ends
+
+@pytest.mark.parametrize("sigma,skew", [(4.0, 0.0), (9.9, 0.0), (21.0, 0.0), (44.0, 0.0), (13.0, 0.05)])
+@pytest.mark.parametrize("L", [1, 2, 40, 150])
+def test_past_the_end_of_a_spectrum(sigma, skew, L):
+    """Many columns up to an end: bins past it are known to 2e-12 of themselves although the columns further
+    back end before them, and an event there has its -lnL and gradient.  (Reference: the response matrix
+    under the tile rule; the pile-up of a bin may hold tails known to 1e-12 of it.)"""
+    s = line_spec(sigma, 900, L=L, tag=True)
+    sh = np.zeros((2, 128))
+    sh[0, 25:64] = np.linspace(1.0, 3.0, 39)
+    sh[1, 30:64] = np.linspace(2.0, 1.0, 34)
+    s = dataclasses.replace(s, shapes=sh / sh.sum(1, keepdims=True), resp_skew=skew, resp_kurt=skew, counts={})
+    th = s.theta_true.copy()
+    th[:s.K] *= 30.0
+    th[s.K + 1:s.K + 3] = 0.1, 1e-4
+    s = empty(s)
+    mo = cut_reference(s, th, 8.0)[0]
+    m = bx.Model(s, precision=bx.BX_FP64)
+    mg = m.expected(th)
+    m.close()
+    z = np.tile(score(s, th), 2)
+    use = (mo > 1e-200) & (z < 30)
+    rel = np.abs(mg[use] / mo[use] - 1)
+    tol = 2e-12 + np.tile(tail_tol(s, th), 2)[use]
+    assert np.all(rel <= tol), (float(rel.max()), float(z[use][np.argmax(rel / tol)]))
+    # events where 1e-3 to 1e-40 are expected
+    rng = np.random.default_rng(2)
+    n = rng.poisson(np.maximum(mo, 0.0)).astype(float)
+    for lo, hi in ((1e-4, 1e-2), (1e-12, 1e-9), (1e-40, 1e-20)):
+        b = np.nonzero((mo > lo) & (mo < hi))[0]
+        if len(b):
+            n[b[len(b) // 2]] = 1.0
+    s = s.with_counts(n)
+    _, fo, go = cut_reference(s, th, 8.0)
+    m = bx.Model(s, precision=bx.BX_FP64, max_batch=6)
+    for k in (1, 6):
+        f, g = m.nll_batch(np.stack([th] * k), grad=True)
+        assert np.all(2 * np.abs(f - fo) <= 1e-7), (f, fo)
+        lhs = np.abs(g[-1] - go) * np.abs(th)
+        lhs[s.K + 6] = 0.0
+        # (differences of a -lnL with terms that change by their whole size over a step: 1e-5 of each)
+        assert np.all(lhs <= 1e-5 * (1 + np.abs(go * th)) + 1e-7 * abs(fo)), lhs
+    m.close()
