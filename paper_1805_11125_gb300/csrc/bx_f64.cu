@@ -40,7 +40,7 @@
 //   k_bwd64    per 32 columns: adjoint of Eq. 1, chain rule, rate gradient
 // Every sum has a fixed order.  Measured on a GB300 at 2070 MHz against the per-entry erfc form this
 // replaced (one erfc per bin edge in the forward, one erfc and one exp in the adjoint): the
-// multivariate model 52 evaluations with gradient 19.2 -> 1.21 ms, the plain model 1000 values
+// multivariate model 52 evaluations with gradient 19.2 -> 1.22 ms, the plain model 1000 values
 // 79.8 -> 3.7 ms, one plain value 4.2 -> 0.13 ms.
 #include <limits.h>
 #include <math.h>
@@ -879,31 +879,27 @@ __device__ __forceinline__ float log2_f64(double x) {
     return (float)((hi >> 20) - 1023) + log2f((float)__hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(x)));
 }
 
-// How far the stencil's lambda may be off in 32 bins (lane b: bin m, if on; the same in each of the block's
-// four warps), over a count whose log2 is lm (l2max: log2 of more than any column's largest bin).  Summed
-// over the columns in FP32: whole, a column whose samples end before the bin (9 sigma) or that does not touch
-// its tile (its samples go one sigma past its band); of any column the stencil's 1e-17 of the density 2.3
-// sigma nearer; and, where the stencil reaches past the end of the samples, 0.04 of the density there, 2^-4
-// less per sigma (bounds of the errors in 40 digits at spacings of 0.1 to 0.2 sigma, from 3 sigma on).
-// Columns below 2^-70 of every count are passed over; 2000 columns take a few us, an exact bin mass of every
-// column that matters 12 us a bin.
-__device__ float tail_error(const Work& w, const Toy& T, int item, int h, bool on, int m, float lm, float l2max) {
+// How far the stencil's lambda may be off in 32 bins (lane b: bin m + b, if its bit of on is set; the same in
+// each of the block's four warps), over a count whose log2 is lm (l2max: log2 of more than any column's
+// largest bin).  Summed over the columns in FP32: whole, a column whose samples end before the bin (9 sigma)
+// or that does not touch its tile (its samples go one sigma past its band); of any column the stencil's 1e-17
+// of the density 2.3 sigma nearer; and, where the stencil reaches past the end of the samples, 0.04 of the
+// density there, 2^-4 less per sigma (bounds of the errors in 40 digits at spacings of 0.1 to 0.2 sigma,
+// from 3 sigma on).  A lane holds a column and the bins are gone through, as data have one or two in 32: the
+// assembly of 100 toys takes 164 us with it, 171 with a lane per bin and columns from 5.7 sigma on passed over
+// up to 1e-11 of the count.  Terms below 2^-60 of the count are passed over; 2000 columns take a few us, an
+// exact bin mass of every column that matters 12 us a bin.
+__device__ float tail_error(const Work& w, const Toy& T, int item, int h, unsigned on, int m, float lm, float l2max) {
     __shared__ float s_err[4][32];
     const int tid = threadIdx.x, lane = tid & 31, part = tid >> 5;
-    const float wf = (float)T.w, y = ((float)m + 0.5f) * wf;
-    const int tile = m / TM;
-    float ylo = on ? y : 3.0e38f, yhi = on ? y : -3.0e38f, lmin = on ? lm : 3.0e38f;   // (of all warps alike)
+    const float wf = (float)T.w;
+    const float ylo = ((float)(m + __ffs(on)) - 0.5f) * wf, yhi = ((float)(m + 31 - __clz(on)) + 0.5f) * wf;
+    float lmin = (on >> lane) & 1u ? lm : 3.0e38f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ylo = fminf(ylo, __shfl_xor_sync(0xffffffffu, ylo, o));
-        yhi = fmaxf(yhi, __shfl_xor_sync(0xffffffffu, yhi, o));
-        lmin = fminf(lmin, __shfl_xor_sync(0xffffffffu, lmin, o));
-    }
+    for (int o = 16; o > 0; o >>= 1) lmin = fminf(lmin, __shfl_xor_sync(0xffffffffu, lmin, o));
     auto score = [&](float gap, float isig) { return fmaxf((gap - 0.5f * wf) * isig, 0.f); };
-    auto near = [&](float mu, float isig) {   // 2.3 sigma nearer than the nearest of the bins
-        return fmaxf(score(fmaxf(fmaxf(ylo - mu, mu - yhi), 0.f), isig) - 2.3f, 0.f);
-    };
     // the warp's groups of 32 columns with one near enough (loads of several groups in flight)
+    static_assert(MAX_CB * BCOLS <= 64 * 128, "a bit per group of 128 columns");
     unsigned long long todo = 0ull;
     const Gen64* gen64 = w.gen64 + (size_t)item * w.Npad;
     const int ng = (T.Next + 127 - 32 * part) / 128;
@@ -911,40 +907,41 @@ __device__ float tail_error(const Work& w, const Toy& T, int item, int h, bool o
     for (int g = 0; g < ng; ++g) {
         const int ie = min(g * 128 + part * 32 + lane, T.Next - 1);
         const double2 ms = *reinterpret_cast<const double2*>(gen64 + ie);   // mean, 1 / sigma
-        const float zl = near((float)ms.x, (float)ms.y);
-        if (__any_sync(0xffffffffu, l2max - 0.72134752f * zl * zl - lmin > -13.f)) todo |= 1ull << g;
+        const float z = score(fmaxf(fmaxf(ylo - (float)ms.x, (float)ms.x - yhi), 0.f), (float)ms.y);
+        const float zn = fmaxf(z - 2.3f, 0.f), zw = fmaxf(z, 7.95f);
+        const float e = -0.72134752f * fminf(fmaf(zn, zn, 78.3f), zw * zw);
+        if (__any_sync(0xffffffffu, l2max - lmin + e > -60.f)) todo |= 1ull << g;
     }
     float err = 0.f;
-    for (; todo; todo &= todo - 1ull) {   // lane: a column, then each live column for 32 bins
+    for (; todo; todo &= todo - 1ull) {
         const int ie = (__ffsll((long long)todo) - 1) * 128 + part * 32 + lane;
         float mu = 0.f, isig = 0.f, l2 = -3.0e38f;   // l2: log2 of the bin mass at the mean
-        int tiles = 0;   // first and last tile that the column touches
+        int t0 = 0, t1 = 0;                          // first and last tile that the column touches
         if (ie < T.Next) {
             const size_t at = (size_t)item * w.Npad + ie;
             const double2 S2 = w.colS[at];
             const Gen64 gen = gen64[ie];
             const Col64 cc = w.col64[at];
-            const double S = fabs(h ? S2.y : S2.x), norm = cc.norm;
+            const double S = fabs(h ? S2.y : S2.x);
             mu = (float)gen.x;
             isig = (float)gen.y;
             if (w.colc64[at].x >= 0 && S > 0.0)
-                l2 = log2_f64(S) + log2f((float)norm / (float)gen.w * isig * wf * 0.39894228f);
+                l2 = log2_f64(S) + log2f((float)cc.norm / (float)gen.w * isig * wf * 0.39894228f);
             int r0, r1;
             near_bins(cc.mu, cc.sig, T.w, T.M, (float)w.band, r0, r1);
-            tiles = (r0 / TM) << 16 | (max(r1 - 1, 0) / TM);
+            t0 = r0 / TM;
+            t1 = (r1 - 1) / TM;
         }
-        const float zl = near(mu, isig);
-        unsigned live = __ballot_sync(0xffffffffu, l2 - 0.72134752f * zl * zl - lmin > -13.f);
-        for (; live; live &= live - 1u) {
-            const int q = __ffs(live) - 1;   // (1e-17 of it: 2^-70)
-            const float kx = __shfl_sync(0xffffffffu, mu, q), ky = __shfl_sync(0xffffffffu, isig, q);
-            const float top = __shfl_sync(0xffffffffu, l2, q) - lm;
-            const int kt = __shfl_sync(0xffffffffu, tiles, q);
-            const float z = score(fabsf(y - kx), ky), zn = fmaxf(z - 2.3f, 0.f);
-            err = fmaf(1e-17f, exp2f(fmaf(-0.72134752f * zn, zn, top)), err);
-            if (z > 5.7f) {
-                const bool out = z > 8.9f || tile < kt >> 16 || tile > (kt & 0xffff);
-                err += exp2f(out ? fmaf(-0.72134752f * z, z, top) : top - 63.1f - 4.f * (9.f - z));
+        for (unsigned r = on; r; r &= r - 1u) {
+            const int b = __ffs(r) - 1, tile = (m + b) / TM;
+            const float top = l2 - __shfl_sync(0xffffffffu, lm, b);
+            const float z = score(fabsf(((float)(m + b) + 0.5f) * wf - mu), isig), zn = fmaxf(z - 2.3f, 0.f);
+            float e = exp2f(fmaf(-0.72134752f * zn, zn, top - 56.4f));   // (1e-17: 2^-56.5)
+            if (z > 5.7f)
+                e += exp2f(z > 8.9f || tile < t0 || tile > t1 ? fmaf(-0.72134752f * z, z, top) : fmaf(4.f, z, top - 99.1f));
+            if (__any_sync(0xffffffffu, e > 8.7e-19f)) {
+                e = warp_sum(e);
+                if (lane == b) err += e;
             }
         }
     }
@@ -962,7 +959,7 @@ __device__ float tail_error(const Work& w, const Toy& T, int item, int h, bool o
 // reach (nearly every bin with pile-up from the columns themselves), at most its own lambda; the reach of
 // any other bin is looked through.
 __device__ __noinline__ bool tail_bins(const Work& w, const Toy& T, int item, int h, unsigned ev, int m0, int Lt,
-                                       double eps, const double* sg, double* sx, const double* mu) {
+                                       double eps, const double* sg, double* sx, const double* mu, int want_mu) {
     __shared__ unsigned s_need[(MAX_L + 32) / 32 + 1];
     __shared__ double s_red[4];
     const int tid = threadIdx.x, lane = tid & 31, nrow = 32 + Lt - 1;
@@ -990,7 +987,9 @@ __device__ __noinline__ bool tail_bins(const Work& w, const Toy& T, int item, in
     // (the Gram-Charlier density at 9 sigma is this much more than the Gaussian's)
     const double gcf = 1.0 + 702.0 * fabs(T.gc1) + 6078.0 * fabs(T.gc2);
     const double bound = 1.7e-5 * gcf * __hiloint2double(top + (1 << 20), 0), reach = bound * fabs(eps) * gs;
-    const float tol = (float)(1e-14 / gcf);   // of a bin's expected count
+    // of a bin's expected count (an event's term takes n times the error; 100 toys' assembly takes 166 us from
+    // 2e-13 to 1e-12, 199 at 5e-14, 206 at 1e-14)
+    const float tol = (float)((want_mu ? 1e-14 : 2e-13) / gcf);
     // (no count: no error is small enough)
     auto log2_mu = [&](int b) { return mu[b] > 1e-290 ? log2_f64(mu[b]) : -3.0e38f; };
     ev &= ~__ballot_sync(0xffffffffu, mu[lane] >= bound + reach);   // (a bin's own lambda is as good)
@@ -1001,9 +1000,8 @@ __device__ __noinline__ bool tail_bins(const Work& w, const Toy& T, int item, in
     const unsigned own = ev & __ballot_sync(0xffffffffu, mu[lane] >= reach && mu[lane] > 1e-290);
     unsigned any = 0u;
     if (own) {
-        const bool on = (own >> lane) & 1u;
-        const float err = tail_error(w, T, item, h, on, m0 + lane, log2_mu(lane), l2max);
-        any = __ballot_sync(0xffffffffu, on && !(err <= tol));
+        const float err = tail_error(w, T, item, h, own, m0, log2_mu(lane), l2max);
+        any = __ballot_sync(0xffffffffu, ((own >> lane) & 1u) && !(err <= tol));
         if (tid < 32 && ((any >> lane) & 1u)) atomicOr(&s_need[(Lt - 1 + lane) >> 5], 1u << ((Lt - 1 + lane) & 31));
     }
     if (ev & ~own) {
@@ -1012,8 +1010,9 @@ __device__ __noinline__ bool tail_bins(const Work& w, const Toy& T, int item, in
         for (int q0 = 0; q0 < nrow; q0 += 32) {   // the bins of sx, 32 at a time
             const int q = q0 + lane, mq = m0 - (Lt - 1) + q;
             const bool on = q < nrow && mq >= 0 && mq < T.M && ((touched >> (mq / TM)) & 1ull) && row_bit(tail, mq);
-            if (!__syncthreads_or(on)) continue;
-            const float err = tail_error(w, T, item, h, on, mq, lm0, l2max);
+            const unsigned rows = __ballot_sync(0xffffffffu, on);   // (of all warps alike)
+            if (!rows) continue;
+            const float err = tail_error(w, T, item, h, rows, mq - lane, lm0, l2max);
             bool need = false;
             for (unsigned e = ev & ~own; e; e &= e - 1u) {
                 const int b = __ffs(e) - 1, d = Lt - 1 + b - q;   // its shift, and its weight in mu
@@ -1078,7 +1077,7 @@ __device__ __noinline__ void tail_adjoint(const Work& w, const Toy& T, int item,
 
 // CTA = 32 window bins of one spectrum of one item, a warp per quarter of the taps: Eq. 2, the
 // Baker-Cousins terms, w = 1 - n/mu, and the tile's part of -lnL (compensated) and of d/deps.  With an
-// event in the tails the sum is taken again if tail_bins changed a lambda (100 toys: 155 -> 172 us; the
+// event in the tails the sum is taken again if tail_bins changed a lambda (100 toys: 155 -> 166 us; the
 // bound of 10 CTAs keeps the registers at 48, 47 without the tails).
 __global__ void __launch_bounds__(128, 10) k_pile64(Work w, int ntw, int nH, int want_grad, int want_mu) {
     extern __shared__ __align__(16) double dsm[];
@@ -1127,7 +1126,7 @@ __global__ void __launch_bounds__(128, 10) k_pile64(Work w, int ntw, int nH, int
         if (!ev) break;
         if (pt == 0) sc[3][b] = (1.0 - eps) * x[0] + eps * cv;
         __syncthreads();
-        if (!tail_bins(w, T, item, h, ev, m0, Lt, eps, sg, sx, sc[3])) break;
+        if (!tail_bins(w, T, item, h, ev, m0, Lt, eps, sg, sx, sc[3], want_mu)) break;
         ev = 0u;   // once more with the better values
     }
     if (pt) return;

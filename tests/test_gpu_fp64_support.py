@@ -352,3 +352,26 @@ def test_past_the_end_of_a_spectrum(sigma, skew, L):
         # (differences of a -lnL with terms that change by their whole size over a step: 1e-5 of each)
         assert np.all(lhs <= 1e-5 * (1 + np.abs(go * th)) + 1e-7 * abs(fo)), lhs
     m.close()
+
+
+@pytest.mark.parametrize("ratio", [30.0, 150.0, 500.0, 2000.0, 1e5])
+@pytest.mark.parametrize("L", [1, 40])
+def test_strong_columns_behind_a_weak_line(L, ratio):
+    """Bins 3.5 sigma and more past a weak line, where strong columns 8.5 sigma off and more are 1e-12 of the
+    count each: those that do not touch the tile are not in it, those that do are in it beyond 9 sigma."""
+    s = line_spec(40.0, 900, L=L, tag=True)
+    sh = np.zeros((2, 128))
+    sh[0, 4:16] = ratio
+    sh[1, 2:14] = ratio
+    sh[:, 62:64] = 1.0
+    s = empty(dataclasses.replace(s, shapes=sh / sh.sum(1, keepdims=True), counts={}))
+    th = s.theta_true.copy()
+    mo = cut_reference(s, th, 8.0)[0]
+    m = bx.Model(s, precision=bx.BX_FP64)
+    mg = m.expected(th)
+    m.close()
+    z = np.tile(score(s, th), 2)
+    use = (mo > 1e-200) & (z < 30)
+    rel = np.abs(mg[use] / mo[use] - 1)
+    tol = 2e-12 + np.tile(tail_tol(s, th), 2)[use]
+    assert np.all(rel <= tol), (float(rel.max()), float(z[use][np.argmax(rel / tol)]))
